@@ -6,6 +6,8 @@
 // to finish (atomic ticket after a fence) sums the per-CTA partials in a fixed order, so the
 // result does not depend on scheduling.  The solver scalars stay on the device; the last CTA
 // also performs the scalar update of the Krylov recurrence.
+#include <algorithm>
+
 #include "blas.cuh"
 #include "ctx.h"
 #include "lowprec.cuh"
@@ -20,6 +22,20 @@ template <class P> struct VecArgs {
 
 constexpr int NT = 256;
 
+// body(j, k) for every site j of [0, n) and storage chunk k.  The units of work are (chunk, tile of NT
+// sites), dealt to the CTAs of a right-hand side in turn: a short range (a 4096-site lattice in FP64 has
+// 16 tiles of 12 chunks) still reaches all SMs, and a long one gives each thread several units, so that
+// the reductions that follow run over few warps.
+template <class P, class Body> __device__ __forceinline__ void for_chunks(long n, Body body)
+{
+    const int nt = (int)((n + NT - 1) / NT), nu = nt * P::NCHUNK;
+    for (int u = blockIdx.x; u < nu; u += gridDim.x) {
+        const int k = P::NCHUNK == 1 ? 0 : u / nt;
+        const long j = (long)(u - k * nt) * NT + threadIdx.x;
+        if (j < n) body(j, k);
+    }
+}
+
 // ----------------------------------------------------------------------------- BiCGStab steps
 // Scalars per right-hand side in KScal (blas.cuh).  r holds s = r - alpha v after the s-step.
 
@@ -30,22 +46,24 @@ __global__ void __launch_bounds__(NT) k_bicg_init(VecArgs<P> va, typename P::SEl
 {
     using R = typename P::R;
     const long rb = (long)blockIdx.y * va.rs;
-    R acc = 0;
-    for (long j = (long)blockIdx.x * NT + threadIdx.x; j < va.n; j += (long)gridDim.x * NT)
-        for (int k = 0; k < P::NCHUNK; k++) {
-            cpx<R> c[P::CW], z[P::CW];
-            P::ld_chunk(r + rb, va.V, va.off + j, k, c);
+    RunSum<R> acc;
+    for_chunks<P>(va.n, [&](long j, int k) {
+        cpx<R> c[P::CW], z[P::CW];
+        R a = 0;
+        P::ld_chunk(r + rb, va.V, va.off + j, k, c);
 #pragma unroll
-            for (int q = 0; q < P::CW; q++) {
-                acc += c[q].re * c[q].re + c[q].im * c[q].im;
-                z[q] = {R(0), R(0)};
-            }
-            P::st_chunk(rh + rb, va.V, va.off + j, k, c);
-            P::st_chunk(p + rb, va.V, va.off + j, k, c);
-            P::st_chunk(x + rb, va.V, va.off + j, k, z);
+        for (int q = 0; q < P::CW; q++) {
+            a += c[q].re * c[q].re + c[q].im * c[q].im;
+            z[q] = {R(0), R(0)};
         }
-    double v[1] = {(double)acc};
-    if (grid_sum<1, NT>(v, part, ticket)) {
+        P::st_chunk(rh + rb, va.V, va.off + j, k, c);
+        P::st_chunk(p + rb, va.V, va.off + j, k, c);
+        P::st_chunk(x + rb, va.V, va.off + j, k, z);
+        acc.add(a);
+    });
+    RunSum<R> sums[1] = {acc};
+    double v[1];
+    if (grid_sum_run<1, NT, R>(sums, v, part, ticket)) {
         KScal &s = sc[blockIdx.y];
         s.rho = make_double2(v[0], 0.0);
         s.rr = v[0];
@@ -63,21 +81,21 @@ __global__ void __launch_bounds__(NT) k_bicg_alpha(VecArgs<P> va, const typename
     using R = typename P::R;
     if (!sc[blockIdx.y].active) return;
     const long rb = (long)blockIdx.y * va.rs;
-    R are = 0, aim = 0;
-    for (long j = (long)blockIdx.x * NT + threadIdx.x; j < va.n; j += (long)gridDim.x * NT)
-        for (int k = 0; k < P::NCHUNK; k++) {
-            cpx<R> c[P::CW], d[P::CW];
-            P::ld_chunk(rh + rb, va.V, va.off + j, k, c);
-            P::ld_chunk(v + rb, va.V, va.off + j, k, d);
+    RunSum<R> are, aim;
+    for_chunks<P>(va.n, [&](long j, int k) {
+        cpx<R> c[P::CW], d[P::CW], a = {R(0), R(0)};
+        P::ld_chunk(rh + rb, va.V, va.off + j, k, c);
+        P::ld_chunk(v + rb, va.V, va.off + j, k, d);
 #pragma unroll
-            for (int q = 0; q < P::CW; q++) {
-                cpx<R> t = cmulc(c[q], d[q]);
-                are += t.re;
-                aim += t.im;
-            }
+        for (int q = 0; q < P::CW; q++) {
+            cmacc(a, c[q], d[q]);
         }
-    double val[2] = {(double)are, (double)aim};
-    if (grid_sum<2, NT>(val, part, ticket)) {
+        are.add(a.re);
+        aim.add(a.im);
+    });
+    RunSum<R> sums[2] = {are, aim};
+    double val[2];
+    if (grid_sum_run<2, NT, R>(sums, val, part, ticket)) {
         KScal &s = sc[blockIdx.y];
         double den = val[0] * val[0] + val[1] * val[1];
         if (den == 0.0 || !(den == den)) {
@@ -100,15 +118,14 @@ __global__ void __launch_bounds__(NT) k_bicg_s(VecArgs<P> va, typename P::SElem 
     if (!s.active) return;
     const cpx<R> al = {R(s.alpha.x), R(s.alpha.y)};
     const long rb = (long)blockIdx.y * va.rs;
-    for (long j = (long)blockIdx.x * NT + threadIdx.x; j < va.n; j += (long)gridDim.x * NT)
-        for (int k = 0; k < P::NCHUNK; k++) {
-            cpx<R> c[P::CW], d[P::CW];
-            P::ld_chunk(r + rb, va.V, va.off + j, k, c);
-            P::ld_chunk(v + rb, va.V, va.off + j, k, d);
+    for_chunks<P>(va.n, [&](long j, int k) {
+        cpx<R> c[P::CW], d[P::CW];
+        P::ld_chunk(r + rb, va.V, va.off + j, k, c);
+        P::ld_chunk(v + rb, va.V, va.off + j, k, d);
 #pragma unroll
-            for (int q = 0; q < P::CW; q++) c[q] = c[q] - cmul(al, d[q]);
-            P::st_chunk(r + rb, va.V, va.off + j, k, c);
-        }
+        for (int q = 0; q < P::CW; q++) cmsub(c[q], al, d[q]);
+        P::st_chunk(r + rb, va.V, va.off + j, k, c);
+    });
 }
 
 template <class P>
@@ -119,22 +136,24 @@ __global__ void __launch_bounds__(NT) k_bicg_omega(VecArgs<P> va, const typename
     using R = typename P::R;
     if (!sc[blockIdx.y].active) return;
     const long rb = (long)blockIdx.y * va.rs;
-    R tsr = 0, tsi = 0, tt = 0;
-    for (long j = (long)blockIdx.x * NT + threadIdx.x; j < va.n; j += (long)gridDim.x * NT)
-        for (int k = 0; k < P::NCHUNK; k++) {
-            cpx<R> c[P::CW], d[P::CW];
-            P::ld_chunk(t + rb, va.V, va.off + j, k, c);
-            P::ld_chunk(r + rb, va.V, va.off + j, k, d);
+    RunSum<R> tsr, tsi, tt;
+    for_chunks<P>(va.n, [&](long j, int k) {
+        cpx<R> c[P::CW], d[P::CW], a = {R(0), R(0)};
+        R b = 0;
+        P::ld_chunk(t + rb, va.V, va.off + j, k, c);
+        P::ld_chunk(r + rb, va.V, va.off + j, k, d);
 #pragma unroll
-            for (int q = 0; q < P::CW; q++) {
-                cpx<R> z = cmulc(c[q], d[q]);
-                tsr += z.re;
-                tsi += z.im;
-                tt += c[q].re * c[q].re + c[q].im * c[q].im;
-            }
+        for (int q = 0; q < P::CW; q++) {
+            cmacc(a, c[q], d[q]);
+            b = fmad(c[q].re, c[q].re, fmad(c[q].im, c[q].im, b));
         }
-    double val[3] = {(double)tsr, (double)tsi, (double)tt};
-    if (grid_sum<3, NT>(val, part, ticket)) {
+        tsr.add(a.re);
+        tsi.add(a.im);
+        tt.add(b);
+    });
+    RunSum<R> sums[3] = {tsr, tsi, tt};
+    double val[3];
+    if (grid_sum_run<3, NT, R>(sums, val, part, ticket)) {
         KScal &s = sc[blockIdx.y];
         if (val[2] == 0.0 || !(val[2] == val[2])) {
             s.breakdown = 2;
@@ -158,29 +177,32 @@ __global__ void __launch_bounds__(NT) k_bicg_xr(VecArgs<P> va, typename P::SElem
     if (!s0.active) return;
     const cpx<R> al = {R(s0.alpha.x), R(s0.alpha.y)}, om = {R(s0.omega.x), R(s0.omega.y)};
     const long rb = (long)blockIdx.y * va.rs;
-    R rhre = 0, rhim = 0, rr = 0;
-    for (long j = (long)blockIdx.x * NT + threadIdx.x; j < va.n; j += (long)gridDim.x * NT)
-        for (int k = 0; k < P::NCHUNK; k++) {
-            cpx<R> xv[P::CW], pv[P::CW], sv[P::CW], tv[P::CW], hv[P::CW];
-            P::ld_chunk(x + rb, va.V, va.off + j, k, xv);
-            P::ld_chunk(p + rb, va.V, va.off + j, k, pv);
-            P::ld_chunk(r + rb, va.V, va.off + j, k, sv);
-            P::ld_chunk(t + rb, va.V, va.off + j, k, tv);
-            P::ld_chunk(rh + rb, va.V, va.off + j, k, hv);
+    RunSum<R> rhre, rhim, rr;
+    for_chunks<P>(va.n, [&](long j, int k) {
+        cpx<R> xv[P::CW], pv[P::CW], sv[P::CW], tv[P::CW], hv[P::CW], a = {R(0), R(0)};
+        R b = 0;
+        P::ld_chunk(x + rb, va.V, va.off + j, k, xv);
+        P::ld_chunk(p + rb, va.V, va.off + j, k, pv);
+        P::ld_chunk(r + rb, va.V, va.off + j, k, sv);
+        P::ld_chunk(t + rb, va.V, va.off + j, k, tv);
+        P::ld_chunk(rh + rb, va.V, va.off + j, k, hv);
 #pragma unroll
-            for (int q = 0; q < P::CW; q++) {
-                xv[q] = xv[q] + cmul(al, pv[q]) + cmul(om, sv[q]);
-                sv[q] = sv[q] - cmul(om, tv[q]);
-                cpx<R> z = cmulc(hv[q], sv[q]);
-                rhre += z.re;
-                rhim += z.im;
-                rr += sv[q].re * sv[q].re + sv[q].im * sv[q].im;
-            }
-            P::st_chunk(x + rb, va.V, va.off + j, k, xv);
-            P::st_chunk(r + rb, va.V, va.off + j, k, sv);
+        for (int q = 0; q < P::CW; q++) {
+            cmac(xv[q], al, pv[q]);
+            cmac(xv[q], om, sv[q]);
+            cmsub(sv[q], om, tv[q]);
+            cmacc(a, hv[q], sv[q]);
+            b = fmad(sv[q].re, sv[q].re, fmad(sv[q].im, sv[q].im, b));
         }
-    double val[3] = {(double)rhre, (double)rhim, (double)rr};
-    if (grid_sum<3, NT>(val, part, ticket)) {
+        P::st_chunk(x + rb, va.V, va.off + j, k, xv);
+        P::st_chunk(r + rb, va.V, va.off + j, k, sv);
+        rhre.add(a.re);
+        rhim.add(a.im);
+        rr.add(b);
+    });
+    RunSum<R> sums[3] = {rhre, rhim, rr};
+    double val[3];
+    if (grid_sum_run<3, NT, R>(sums, val, part, ticket)) {
         KScal &s = sc[blockIdx.y];
         s.rr = val[2];
         s.iters += 1;
@@ -214,16 +236,18 @@ __global__ void __launch_bounds__(NT) k_bicg_p(VecArgs<P> va, typename P::SElem 
     if (!s.active) return;
     const cpx<R> be = {R(s.beta.x), R(s.beta.y)}, om = {R(s.omega.x), R(s.omega.y)};
     const long rb = (long)blockIdx.y * va.rs;
-    for (long j = (long)blockIdx.x * NT + threadIdx.x; j < va.n; j += (long)gridDim.x * NT)
-        for (int k = 0; k < P::NCHUNK; k++) {
-            cpx<R> pv[P::CW], rv[P::CW], vv[P::CW];
-            P::ld_chunk(p + rb, va.V, va.off + j, k, pv);
-            P::ld_chunk(r + rb, va.V, va.off + j, k, rv);
-            P::ld_chunk(v + rb, va.V, va.off + j, k, vv);
+    for_chunks<P>(va.n, [&](long j, int k) {
+        cpx<R> pv[P::CW], rv[P::CW], vv[P::CW];
+        P::ld_chunk(p + rb, va.V, va.off + j, k, pv);
+        P::ld_chunk(r + rb, va.V, va.off + j, k, rv);
+        P::ld_chunk(v + rb, va.V, va.off + j, k, vv);
 #pragma unroll
-            for (int q = 0; q < P::CW; q++) pv[q] = rv[q] + cmul(be, pv[q] - cmul(om, vv[q]));
-            P::st_chunk(p + rb, va.V, va.off + j, k, pv);
+        for (int q = 0; q < P::CW; q++) {
+            cmsub(pv[q], om, vv[q]);
+            cmac(rv[q], be, pv[q]);
         }
+        P::st_chunk(p + rb, va.V, va.off + j, k, rv);
+    });
 }
 
 // alpha (MODE 1) or omega (MODE 2) from the per-warp partial sums a fused stencil epilogue wrote:
@@ -291,16 +315,18 @@ __global__ void __launch_bounds__(NT) k_norm2(VecArgs<P> va, const typename P::S
 {
     using R = typename P::R;
     const long rb = (long)blockIdx.y * va.rs;
-    R acc = 0;
-    for (long j = (long)blockIdx.x * NT + threadIdx.x; j < va.n; j += (long)gridDim.x * NT)
-        for (int k = 0; k < P::NCHUNK; k++) {
-            cpx<R> c[P::CW];
-            P::ld_chunk(f + rb, va.V, va.off + j, k, c);
+    RunSum<R> acc;
+    for_chunks<P>(va.n, [&](long j, int k) {
+        cpx<R> c[P::CW];
+        R a = 0;
+        P::ld_chunk(f + rb, va.V, va.off + j, k, c);
 #pragma unroll
-            for (int q = 0; q < P::CW; q++) acc += c[q].re * c[q].re + c[q].im * c[q].im;
-        }
-    double v[1] = {(double)acc};
-    if (grid_sum<1, NT>(v, part, ticket)) out[blockIdx.y] = v[0];
+        for (int q = 0; q < P::CW; q++) a = fmad(c[q].re, c[q].re, fmad(c[q].im, c[q].im, a));
+        acc.add(a);
+    });
+    RunSum<R> sums[1] = {acc};
+    double v[1];
+    if (grid_sum_run<1, NT, R>(sums, v, part, ticket)) out[blockIdx.y] = v[0];
 }
 
 // out[3r .. 3r+2] = (sum |d|^2, Re sum conj(d) e, Im sum conj(d) e) -- the exponents
@@ -312,21 +338,24 @@ __global__ void __launch_bounds__(NT) k_norm_dot(VecArgs<P> va, const typename P
 {
     using R = typename P::R;
     const long rb = (long)blockIdx.y * va.rs;
-    R nn = 0, dr = 0, di = 0;
-    for (long j = (long)blockIdx.x * NT + threadIdx.x; j < va.n; j += (long)gridDim.x * NT)
-        for (int k = 0; k < P::NCHUNK; k++) {
-            cpx<R> c[P::CW], f[P::CW];
-            P::ld_chunk(d + rb, va.V, va.off + j, k, c);
-            P::ld_chunk(e + rb, va.V, va.off + j, k, f);
+    RunSum<R> nn, dr, di;
+    for_chunks<P>(va.n, [&](long j, int k) {
+        cpx<R> c[P::CW], f[P::CW], a = {R(0), R(0)};
+        R b = 0;
+        P::ld_chunk(d + rb, va.V, va.off + j, k, c);
+        P::ld_chunk(e + rb, va.V, va.off + j, k, f);
 #pragma unroll
-            for (int q = 0; q < P::CW; q++) {
-                nn += c[q].re * c[q].re + c[q].im * c[q].im;
-                dr += c[q].re * f[q].re + c[q].im * f[q].im;
-                di += c[q].re * f[q].im - c[q].im * f[q].re;
-            }
+        for (int q = 0; q < P::CW; q++) {
+            b = fmad(c[q].re, c[q].re, fmad(c[q].im, c[q].im, b));
+            cmacc(a, c[q], f[q]);
         }
-    double v[3] = {(double)nn, (double)dr, (double)di};
-    if (grid_sum<3, NT>(v, part, ticket)) {
+        nn.add(b);
+        dr.add(a.re);
+        di.add(a.im);
+    });
+    RunSum<R> sums[3] = {nn, dr, di};
+    double v[3];
+    if (grid_sum_run<3, NT, R>(sums, v, part, ticket)) {
         out[3 * blockIdx.y] = v[0];
         out[3 * blockIdx.y + 1] = v[1];
         out[3 * blockIdx.y + 2] = v[2];
@@ -340,15 +369,14 @@ __global__ void __launch_bounds__(NT) k_axpby(VecArgs<P> va, double a, const typ
 {
     using R = typename P::R;
     const long rb = (long)blockIdx.y * va.rs;
-    for (long j = (long)blockIdx.x * NT + threadIdx.x; j < va.n; j += (long)gridDim.x * NT)
-        for (int k = 0; k < P::NCHUNK; k++) {
-            cpx<R> c[P::CW], d[P::CW];
-            P::ld_chunk(x + rb, va.V, va.off + j, k, c);
-            P::ld_chunk(y + rb, va.V, va.off + j, k, d);
+    for_chunks<P>(va.n, [&](long j, int k) {
+        cpx<R> c[P::CW], d[P::CW];
+        P::ld_chunk(x + rb, va.V, va.off + j, k, c);
+        P::ld_chunk(y + rb, va.V, va.off + j, k, d);
 #pragma unroll
-            for (int q = 0; q < P::CW; q++) d[q] = R(a) * c[q] + R(b) * d[q];
-            P::st_chunk(y + rb, va.V, va.off + j, k, d);
-        }
+        for (int q = 0; q < P::CW; q++) d[q] = R(a) * c[q] + R(b) * d[q];
+        P::st_chunk(y + rb, va.V, va.off + j, k, d);
+    });
 }
 
 // FP64 -> storage precision P with a per-right-hand-side scale: out = in * scale[r]
@@ -360,16 +388,15 @@ __global__ void __launch_bounds__(NT) k_to_low(long V, long off, long n, long rs
     const double sc = scale ? scale[blockIdx.y] : 1.0;
     const double2 *ib = in + (long)blockIdx.y * rs64;
     typename P::SElem *ob = out + (long)blockIdx.y * rsl;
-    for (long j = (long)blockIdx.x * NT + threadIdx.x; j < n; j += (long)gridDim.x * NT)
-        for (int k = 0; k < P::NCHUNK; k++) {
-            cpx<R> c[P::CW];
+    for_chunks<P>(n, [&](long j, int k) {
+        cpx<R> c[P::CW];
 #pragma unroll
-            for (int q = 0; q < P::CW; q++) {
-                double2 a = ib[(long)(k * P::CW + q) * V + off + j];
-                c[q] = {R(a.x * sc), R(a.y * sc)};
-            }
-            P::st_chunk(ob, V, off + j, k, c);
+        for (int q = 0; q < P::CW; q++) {
+            double2 a = ib[(long)(k * P::CW + q) * V + off + j];
+            c[q] = {R(a.x * sc), R(a.y * sc)};
         }
+        P::st_chunk(ob, V, off + j, k, c);
+    });
 }
 
 // x64 += scale[r] * e (e in storage precision P)
@@ -381,17 +408,16 @@ __global__ void __launch_bounds__(NT) k_add_low(long V, long off, long n, long r
     const double sc = scale ? scale[blockIdx.y] : 1.0;
     const typename P::SElem *eb = e + (long)blockIdx.y * rsl;
     double2 *xb = x + (long)blockIdx.y * rs64;
-    for (long j = (long)blockIdx.x * NT + threadIdx.x; j < n; j += (long)gridDim.x * NT)
-        for (int k = 0; k < P::NCHUNK; k++) {
-            cpx<R> c[P::CW];
-            P::ld_chunk(eb, V, off + j, k, c);
+    for_chunks<P>(n, [&](long j, int k) {
+        cpx<R> c[P::CW];
+        P::ld_chunk(eb, V, off + j, k, c);
 #pragma unroll
-            for (int q = 0; q < P::CW; q++) {
-                double2 *a = xb + (long)(k * P::CW + q) * V + off + j;
-                double2 av = *a;
-                *a = make_double2(av.x + sc * (double)c[q].re, av.y + sc * (double)c[q].im);
-            }
+        for (int q = 0; q < P::CW; q++) {
+            double2 *a = xb + (long)(k * P::CW + q) * V + off + j;
+            double2 av = *a;
+            *a = make_double2(av.x + sc * (double)c[q].re, av.y + sc * (double)c[q].im);
         }
+    });
 }
 
 // FP32 link / clover planes -> 16-bit planes of the same order
@@ -405,10 +431,15 @@ template <bool BF> __global__ void k_f32_to_low(long n, const float4 *__restrict
 
 // ----------------------------------------------------------------------------- host side
 
-static unsigned grid_for(long n)
+// CTAs per right-hand side for a range of n sites in nch chunks: one unit of for_chunks per CTA while
+// nrhs of them fit the chip (152 SMs, 8 CTAs of 256 threads each), else the same
+// number of units for each; at most 608, which the partial sums have room for
+static unsigned grid_for(long n, int nch, int nrhs)
 {
-    long g = (n + NT - 1) / NT;
-    return (unsigned)(g < 1 ? 1 : (g > 608 ? 608 : g));
+    const long units = std::max(1L, (n + NT - 1) / NT) * nch;
+    const long most = std::min(608L, std::max(1L, (1216L + nrhs - 1) / nrhs));
+    const long per = (units + most - 1) / most;
+    return (unsigned)((units + per - 1) / per);
 }
 
 ddrw_status reduce_ws(ddrw_ctx *ctx, int nrhs, double **part, unsigned **ticket)
@@ -440,7 +471,7 @@ ddrw_status Blas<P>::bicg_init(ddrw_ctx *ctx, const VecRange &vr, E *r, E *rh, E
     ddrw_status st = reduce_ws(ctx, vr.nrhs, &part, &tk);
     if (st) return st;
     VecArgs<P> va{vr.V, vr.off, vr.n, vr.rs};
-    dim3 g(grid_for(vr.n), vr.nrhs);
+    dim3 g(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs);
     ProfScope ps(ctx, PROF_BLAS, 0.0);
     ++ctx->launches;
     k_bicg_init<P><<<g, NT, 0, ctx->stream>>>(va, r, rh, p, x, sc, part, tk);
@@ -457,7 +488,7 @@ ddrw_status Blas<P>::bicg_alpha(ddrw_ctx *ctx, const VecRange &vr, const E *rh, 
     VecArgs<P> va{vr.V, vr.off, vr.n, vr.rs};
     ProfScope ps(ctx, PROF_BLAS, 0.0);
     ++ctx->launches;
-    k_bicg_alpha<P><<<dim3(grid_for(vr.n), vr.nrhs), NT, 0, ctx->stream>>>(va, rh, v, sc, part, tk);
+    k_bicg_alpha<P><<<dim3(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(va, rh, v, sc, part, tk);
     return DDRW_OK;
 }
 
@@ -467,7 +498,7 @@ void Blas<P>::bicg_s(ddrw_ctx *ctx, const VecRange &vr, E *r, const E *v, const 
     VecArgs<P> va{vr.V, vr.off, vr.n, vr.rs};
     ProfScope ps(ctx, PROF_BLAS, 0.0);
     ++ctx->launches;
-    k_bicg_s<P><<<dim3(grid_for(vr.n), vr.nrhs), NT, 0, ctx->stream>>>(va, r, v, sc);
+    k_bicg_s<P><<<dim3(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(va, r, v, sc);
 }
 
 template <class P>
@@ -480,7 +511,7 @@ ddrw_status Blas<P>::bicg_omega(ddrw_ctx *ctx, const VecRange &vr, const E *t, c
     VecArgs<P> va{vr.V, vr.off, vr.n, vr.rs};
     ProfScope ps(ctx, PROF_BLAS, 0.0);
     ++ctx->launches;
-    k_bicg_omega<P><<<dim3(grid_for(vr.n), vr.nrhs), NT, 0, ctx->stream>>>(va, t, r, sc, part, tk);
+    k_bicg_omega<P><<<dim3(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(va, t, r, sc, part, tk);
     return DDRW_OK;
 }
 
@@ -495,7 +526,7 @@ ddrw_status Blas<P>::bicg_xr(ddrw_ctx *ctx, const VecRange &vr, E *x, const E *p
     VecArgs<P> va{vr.V, vr.off, vr.n, vr.rs};
     ProfScope ps(ctx, PROF_BLAS, 0.0);
     ++ctx->launches;
-    k_bicg_xr<P><<<dim3(grid_for(vr.n), vr.nrhs), NT, 0, ctx->stream>>>(va, x, p, r, t, rh, sc, part, tk);
+    k_bicg_xr<P><<<dim3(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(va, x, p, r, t, rh, sc, part, tk);
     return DDRW_OK;
 }
 
@@ -505,7 +536,7 @@ void Blas<P>::bicg_p(ddrw_ctx *ctx, const VecRange &vr, E *p, const E *r, const 
     VecArgs<P> va{vr.V, vr.off, vr.n, vr.rs};
     ProfScope ps(ctx, PROF_BLAS, 0.0);
     ++ctx->launches;
-    k_bicg_p<P><<<dim3(grid_for(vr.n), vr.nrhs), NT, 0, ctx->stream>>>(va, p, r, v, sc);
+    k_bicg_p<P><<<dim3(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(va, p, r, v, sc);
 }
 
 template <class P>
@@ -518,7 +549,7 @@ ddrw_status Blas<P>::norm2(ddrw_ctx *ctx, const VecRange &vr, const E *f, double
     VecArgs<P> va{vr.V, vr.off, vr.n, vr.rs};
     ProfScope ps(ctx, PROF_BLAS, 0.0);
     ++ctx->launches;
-    k_norm2<P><<<dim3(grid_for(vr.n), vr.nrhs), NT, 0, ctx->stream>>>(va, f, out, part, tk);
+    k_norm2<P><<<dim3(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(va, f, out, part, tk);
     return DDRW_OK;
 }
 
@@ -532,7 +563,7 @@ ddrw_status Blas<P>::norm_dot(ddrw_ctx *ctx, const VecRange &vr, const E *d, con
     VecArgs<P> va{vr.V, vr.off, vr.n, vr.rs};
     ProfScope ps(ctx, PROF_BLAS, 0.0);
     ++ctx->launches;
-    k_norm_dot<P><<<dim3(grid_for(vr.n), vr.nrhs), NT, 0, ctx->stream>>>(va, d, e, out, part, tk);
+    k_norm_dot<P><<<dim3(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(va, d, e, out, part, tk);
     return DDRW_OK;
 }
 
@@ -542,7 +573,7 @@ void Blas<P>::axpby(ddrw_ctx *ctx, const VecRange &vr, double a, const E *x, dou
     VecArgs<P> va{vr.V, vr.off, vr.n, vr.rs};
     ProfScope ps(ctx, PROF_BLAS, 0.0);
     ++ctx->launches;
-    k_axpby<P><<<dim3(grid_for(vr.n), vr.nrhs), NT, 0, ctx->stream>>>(va, a, x, b, y);
+    k_axpby<P><<<dim3(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(va, a, x, b, y);
 }
 
 template <class P>
@@ -551,7 +582,7 @@ void to_low(ddrw_ctx *ctx, const VecRange &vr, long rsl, const double2 *in, type
 {
     ProfScope ps(ctx, PROF_BLAS, 0.0);
     ++ctx->launches;
-    k_to_low<P><<<dim3(grid_for(vr.n), vr.nrhs), NT, 0, ctx->stream>>>(vr.V, vr.off, vr.n, vr.rs, rsl, in, out, scale);
+    k_to_low<P><<<dim3(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(vr.V, vr.off, vr.n, vr.rs, rsl, in, out, scale);
 }
 
 template <class P>
@@ -559,7 +590,7 @@ void add_low(ddrw_ctx *ctx, const VecRange &vr, long rsl, const typename P::SEle
 {
     ProfScope ps(ctx, PROF_BLAS, 0.0);
     ++ctx->launches;
-    k_add_low<P><<<dim3(grid_for(vr.n), vr.nrhs), NT, 0, ctx->stream>>>(vr.V, vr.off, vr.n, vr.rs, rsl, e, x, scale);
+    k_add_low<P><<<dim3(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(vr.V, vr.off, vr.n, vr.rs, rsl, e, x, scale);
 }
 
 void f32_to_low(ddrw_ctx *ctx, const float4 *in, uint2 *out, long n, bool bf)
@@ -612,7 +643,7 @@ void f32_to_16(ddrw_ctx *ctx, const VecRange &vr, long rs16, const float4 *in, t
 {
     ProfScope ps(ctx, PROF_BLAS, 0.0);
     ++ctx->launches;
-    k_f32_to_16<P16><<<dim3(grid_for(vr.n), vr.nrhs), NT, 0, ctx->stream>>>(vr.V, vr.off, vr.n, vr.rs, rs16, in, out);
+    k_f32_to_16<P16><<<dim3(grid_for(vr.n, 1, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(vr.V, vr.off, vr.n, vr.rs, rs16, in, out);
 }
 
 template <class P16>
@@ -620,7 +651,7 @@ void fold_16_into_32(ddrw_ctx *ctx, const VecRange &vr, long rs16, typename P16:
 {
     ProfScope ps(ctx, PROF_BLAS, 0.0);
     ++ctx->launches;
-    k_fold_16_into_32<P16><<<dim3(grid_for(vr.n), vr.nrhs), NT, 0, ctx->stream>>>(vr.V, vr.off, vr.n, rs16, vr.rs, x16,
+    k_fold_16_into_32<P16><<<dim3(grid_for(vr.n, 1, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(vr.V, vr.off, vr.n, rs16, vr.rs, x16,
                                                                                    x32);
 }
 template void f32_to_16<PrecH>(ddrw_ctx *, const VecRange &, long, const float4 *, PrecH::SElem *);

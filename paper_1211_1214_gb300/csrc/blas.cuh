@@ -47,29 +47,85 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
-// Sum v[0..K) over the grid's CTAs for right-hand side blockIdx.y.  Returns true in thread 0 of the
-// last CTA, with the totals in v.  part: [nrhs][gridDim.x][K] doubles, ticket: [nrhs] zeroed.
-template <int K, int NT>
-__device__ bool grid_sum(double (&v)[K], double *part, unsigned *ticket)
+// A running sum: FP64 for FP64 fields; for FP32 arithmetic an unevaluated pair hi + lo (Knuth's
+// two-sum, about 48 significant bits against the 24 of the terms).  GB300 adds FP64 at 1/64 of its FP32
+// rate: with FP64 shuffle steps in every warp and FP64 sums over the warps, the reductions took longer
+// than the fields' passes (bicg_omega on 12 x 65536 FP16 sites 43 us, against 14 us for the
+// three passes of bicg_s, which does not reduce).
+template <typename R> struct RunSum;
+template <> struct RunSum<double> {
+    using Raw = double;
+    double s = 0.0;
+    __device__ __forceinline__ void add(double x) { s += x; }
+    __device__ __forceinline__ void join(Raw o) { s += o; }
+    __device__ __forceinline__ Raw raw() const { return s; }
+    __device__ __forceinline__ double value() const { return s; }
+    template <int W> __device__ __forceinline__ void shuffle_sum()  // lane 0: the sum over lanes 0 .. W - 1
+    {
+#pragma unroll
+        for (int o = W / 2; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    }
+};
+template <> struct RunSum<float> {
+    using Raw = float2;
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void join(Raw o)
+    {
+        const float s = __fadd_rn(hi, o.x), v = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(o.y, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, v)), __fsub_rn(o.x, v))));
+        hi = s;
+    }
+    __device__ __forceinline__ void add(float x) { join(make_float2(x, 0.f)); }
+    __device__ __forceinline__ Raw raw() const { return make_float2(hi, lo); }
+    // an overflowed or NaN sum is reported as hi gives it (lo is then NaN)
+    __device__ __forceinline__ double value() const { return (double)hi + (lo - lo == 0.f ? (double)lo : 0.0); }
+    template <int W> __device__ __forceinline__ void shuffle_sum()
+    {
+#pragma unroll
+        for (int o = W / 2; o > 0; o >>= 1) {
+            Raw q;
+            q.x = __shfl_down_sync(0xffffffffu, hi, o);
+            q.y = __shfl_down_sync(0xffffffffu, lo, o);
+            join(q);
+        }
+    }
+};
+
+// CTA totals of v[0..K) in thread 0 (the caller's other threads may go on; sm is reused only after a barrier)
+template <int K, int NT, typename R>
+__device__ __forceinline__ void cta_sum_run(RunSum<R> (&v)[K], typename RunSum<R>::Raw (*sm)[K])
 {
-    __shared__ double sm[NT / 32][K];
-    __shared__ bool last;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
-    for (int k = 0; k < K; k++) v[k] = warp_sum(v[k]);
+    for (int k = 0; k < K; k++) v[k].template shuffle_sum<32>();
     if (lane == 0)
 #pragma unroll
-        for (int k = 0; k < K; k++) sm[w][k] = v[k];
+        for (int k = 0; k < K; k++) sm[w][k] = v[k].raw();
     __syncthreads();
-    const int r = blockIdx.y, G = gridDim.x;
-    if (threadIdx.x == 0) {
-        double *pp = part + ((long)r * G + blockIdx.x) * K;
+    if (w == 0)
 #pragma unroll
         for (int k = 0; k < K; k++) {
-            double s = 0;
-            for (int i = 0; i < NT / 32; i++) s += sm[i][k];
-            pp[k] = s;
+            v[k] = RunSum<R>();
+            if (lane < NT / 32) v[k].join(sm[lane][k]);
+            v[k].template shuffle_sum<NT / 32>();
         }
+}
+
+// Sum v[0..K) over the grid's CTAs for right-hand side blockIdx.y.  Returns true in thread 0 of the
+// last CTA, with the totals in out.  part: [nrhs][gridDim.x][K] 8-byte partial sums, ticket:
+// [nrhs] zeroed.
+template <int K, int NT, typename R>
+__device__ bool grid_sum_run(RunSum<R> (&v)[K], double (&out)[K], double *part, unsigned *ticket)
+{
+    using Raw = typename RunSum<R>::Raw;
+    __shared__ Raw sm[NT / 32][K];
+    __shared__ bool last;
+    const int r = blockIdx.y, G = gridDim.x;
+    Raw *pp = reinterpret_cast<Raw *>(part) + (long)r * G * K;
+    cta_sum_run<K, NT, R>(v, sm);
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int k = 0; k < K; k++) pp[(long)blockIdx.x * K + k] = v[k].raw();
         __threadfence();
         unsigned t = atomicAdd(ticket + r, 1u);
         last = (t == (unsigned)(G - 1));
@@ -77,32 +133,28 @@ __device__ bool grid_sum(double (&v)[K], double *part, unsigned *ticket)
     __syncthreads();
     if (!last) return false;
     __threadfence();
-    double acc[K];
 #pragma unroll
-    for (int k = 0; k < K; k++) acc[k] = 0;
-    for (int i = threadIdx.x; i < G; i += NT) {
-        const double *pp = part + ((long)r * G + i) * K;
+    for (int k = 0; k < K; k++) v[k] = RunSum<R>();
+    for (int i = threadIdx.x; i < G; i += NT)
 #pragma unroll
-        for (int k = 0; k < K; k++) acc[k] += __ldcg(pp + k);
-    }
-#pragma unroll
-    for (int k = 0; k < K; k++) acc[k] = warp_sum(acc[k]);
-    __syncthreads();
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < K; k++) sm[w][k] = acc[k];
-    __syncthreads();
+        for (int k = 0; k < K; k++) v[k].join(__ldcg(pp + (long)i * K + k));
+    cta_sum_run<K, NT, R>(v, sm);
     if (threadIdx.x == 0) {
 #pragma unroll
-        for (int k = 0; k < K; k++) {
-            double s = 0;
-            for (int i = 0; i < NT / 32; i++) s += sm[i][k];
-            v[k] = s;
-        }
+        for (int k = 0; k < K; k++) out[k] = v[k].value();
         ticket[r] = 0;
         return true;
     }
     return false;
+}
+
+// the same from per-thread FP64 values, in place
+template <int K, int NT> __device__ bool grid_sum(double (&v)[K], double *part, unsigned *ticket)
+{
+    RunSum<double> q[K];
+#pragma unroll
+    for (int k = 0; k < K; k++) q[k].s = v[k];
+    return grid_sum_run<K, NT, double>(q, v, part, ticket);
 }
 
 // alpha (mode 1) or omega (mode 2) of the BiCGStab recurrence from the per-warp partial sums of a
