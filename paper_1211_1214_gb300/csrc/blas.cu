@@ -128,157 +128,143 @@ __global__ void __launch_bounds__(NT) k_bicg_s(VecArgs<P> va, typename P::SElem 
     });
 }
 
+// omega = (t, s) / (t, t) and, from the same pass over t, s and rh, the next direction's scalars:
+// rho' = (rh, s - omega t) = (rh, s) - omega (rh, t), beta = (rho' alpha) / (rho omega).  With beta
+// known here, the updates of x, r and p need one kernel (k_bicg_xrp) instead of two that
+// read and write r twice: 16 passes over a vector and 4 vector kernels per iteration, not 18 and 5.
+// val: (t, s) re, im, (t, t), (rh, s) re, im, (rh, t) re, im
+__device__ __forceinline__ void omega_beta(KScal &s, const double *val)
+{
+    if (val[2] == 0.0 || !(val[2] == val[2])) {
+        s.breakdown = 2;
+        s.active = 0;
+        s.omega = make_double2(0.0, 0.0);
+        return;
+    }
+    const double it = 1.0 / val[2];
+    const double2 om = make_double2(val[0] * it, val[1] * it);
+    const double2 rn = make_double2(val[3] - (om.x * val[5] - om.y * val[6]), val[4] - (om.x * val[6] + om.y * val[5]));
+    const double2 num = make_double2(rn.x * s.alpha.x - rn.y * s.alpha.y, rn.x * s.alpha.y + rn.y * s.alpha.x);
+    const double2 den = make_double2(s.rho.x * om.x - s.rho.y * om.y, s.rho.x * om.y + s.rho.y * om.x);
+    const double d2 = den.x * den.x + den.y * den.y;
+    s.omega = om;
+    // a zero denominator ends the recurrence after this iteration's x and r (k_bicg_xrp)
+    s.beta = d2 > 0.0 ? make_double2((num.x * den.x + num.y * den.y) / d2, (num.y * den.x - num.x * den.y) / d2)
+                      : make_double2(0.0, 0.0);
+    s.rho = d2 > 0.0 ? rn : make_double2(0.0, 0.0);
+}
+
 template <class P>
 __global__ void __launch_bounds__(NT) k_bicg_omega(VecArgs<P> va, const typename P::SElem *t,
-                                                   const typename P::SElem *r, KScal *sc, double *part,
-                                                   unsigned *ticket)
+                                                   const typename P::SElem *r, const typename P::SElem *rh, KScal *sc,
+                                                   double *part, unsigned *ticket)
 {
     using R = typename P::R;
     if (!sc[blockIdx.y].active) return;
     const long rb = (long)blockIdx.y * va.rs;
-    RunSum<R> tsr, tsi, tt;
+    RunSum<R> sums[7];
     for_chunks<P>(va.n, [&](long j, int k) {
-        cpx<R> c[P::CW], d[P::CW], a = {R(0), R(0)};
+        cpx<R> c[P::CW], d[P::CW], h[P::CW], ts = {R(0), R(0)}, hs = {R(0), R(0)}, ht = {R(0), R(0)};
         R b = 0;
         P::ld_chunk(t + rb, va.V, va.off + j, k, c);
         P::ld_chunk(r + rb, va.V, va.off + j, k, d);
+        P::ld_chunk(rh + rb, va.V, va.off + j, k, h);
 #pragma unroll
         for (int q = 0; q < P::CW; q++) {
-            cmacc(a, c[q], d[q]);
+            cmacc(ts, c[q], d[q]);
             b = fmad(c[q].re, c[q].re, fmad(c[q].im, c[q].im, b));
+            cmacc(hs, h[q], d[q]);
+            cmacc(ht, h[q], c[q]);
         }
-        tsr.add(a.re);
-        tsi.add(a.im);
-        tt.add(b);
+        sums[0].add(ts.re);
+        sums[1].add(ts.im);
+        sums[2].add(b);
+        sums[3].add(hs.re);
+        sums[4].add(hs.im);
+        sums[5].add(ht.re);
+        sums[6].add(ht.im);
     });
-    RunSum<R> sums[3] = {tsr, tsi, tt};
-    double val[3];
-    if (grid_sum_run<3, NT, R>(sums, val, part, ticket)) {
-        KScal &s = sc[blockIdx.y];
-        if (val[2] == 0.0 || !(val[2] == val[2])) {
-            s.breakdown = 2;
-            s.active = 0;
-            s.omega = make_double2(0.0, 0.0);
-            return;
-        }
-        s.omega = make_double2(val[0] / val[2], val[1] / val[2]);
-    }
+    double val[7];
+    if (grid_sum_run<7, NT, R>(sums, val, part, ticket)) omega_beta(sc[blockIdx.y], val);
 }
 
-// x += alpha p + omega s;  r = s - omega t;  rho' = (rh, r), rr = (r, r);  beta = (rho'/rho)(alpha/omega)
+// x += alpha p + omega s;  r = s - omega t;  p = r + beta (p - omega v);  rr = (r, r)
 template <class P>
-__global__ void __launch_bounds__(NT) k_bicg_xr(VecArgs<P> va, typename P::SElem *x, const typename P::SElem *p,
-                                                typename P::SElem *r, const typename P::SElem *t,
-                                                const typename P::SElem *rh, KScal *sc, double *part,
-                                                unsigned *ticket)
+__global__ void __launch_bounds__(NT, 2) k_bicg_xrp(VecArgs<P> va, typename P::SElem *x, typename P::SElem *p,
+                                                    typename P::SElem *r, const typename P::SElem *t,
+                                                    const typename P::SElem *v, KScal *sc, double *part,
+                                                    unsigned *ticket)
 {
     using R = typename P::R;
     const KScal &s0 = sc[blockIdx.y];
     if (!s0.active) return;
     const cpx<R> al = {R(s0.alpha.x), R(s0.alpha.y)}, om = {R(s0.omega.x), R(s0.omega.y)};
+    const cpx<R> be = {R(s0.beta.x), R(s0.beta.y)};
     const long rb = (long)blockIdx.y * va.rs;
-    RunSum<R> rhre, rhim, rr;
+    RunSum<R> rr[1];
     for_chunks<P>(va.n, [&](long j, int k) {
-        cpx<R> xv[P::CW], pv[P::CW], sv[P::CW], tv[P::CW], hv[P::CW], a = {R(0), R(0)};
+        cpx<R> xv[P::CW], pv[P::CW], sv[P::CW], tv[P::CW], vv[P::CW];
         R b = 0;
         P::ld_chunk(x + rb, va.V, va.off + j, k, xv);
         P::ld_chunk(p + rb, va.V, va.off + j, k, pv);
         P::ld_chunk(r + rb, va.V, va.off + j, k, sv);
         P::ld_chunk(t + rb, va.V, va.off + j, k, tv);
-        P::ld_chunk(rh + rb, va.V, va.off + j, k, hv);
+        P::ld_chunk(v + rb, va.V, va.off + j, k, vv);
 #pragma unroll
         for (int q = 0; q < P::CW; q++) {
             cmac(xv[q], al, pv[q]);
             cmac(xv[q], om, sv[q]);
             cmsub(sv[q], om, tv[q]);
-            cmacc(a, hv[q], sv[q]);
             b = fmad(sv[q].re, sv[q].re, fmad(sv[q].im, sv[q].im, b));
+            cmsub(pv[q], om, vv[q]);
+            tv[q] = sv[q];
+            cmac(tv[q], be, pv[q]);
         }
         P::st_chunk(x + rb, va.V, va.off + j, k, xv);
         P::st_chunk(r + rb, va.V, va.off + j, k, sv);
-        rhre.add(a.re);
-        rhim.add(a.im);
-        rr.add(b);
+        P::st_chunk(p + rb, va.V, va.off + j, k, tv);
+        rr[0].add(b);
     });
-    RunSum<R> sums[3] = {rhre, rhim, rr};
-    double val[3];
-    if (grid_sum_run<3, NT, R>(sums, val, part, ticket)) {
+    double val[1];
+    if (grid_sum_run<1, NT, R>(rr, val, part, ticket)) {
         KScal &s = sc[blockIdx.y];
-        s.rr = val[2];
+        s.rr = val[0];
         s.iters += 1;
-        double2 rn = make_double2(val[0], val[1]);
-        // beta = (rn / rho) * (alpha / omega)
-        double d1 = s.rho.x * s.rho.x + s.rho.y * s.rho.y;
-        double d2 = s.omega.x * s.omega.x + s.omega.y * s.omega.y;
-        double2 q1 = make_double2((rn.x * s.rho.x + rn.y * s.rho.y) / d1, (rn.y * s.rho.x - rn.x * s.rho.y) / d1);
-        double2 q2 = make_double2((s.alpha.x * s.omega.x + s.alpha.y * s.omega.y) / d2,
-                                  (s.alpha.y * s.omega.x - s.alpha.x * s.omega.y) / d2);
-        s.beta = make_double2(q1.x * q2.x - q1.y * q2.y, q1.x * q2.y + q1.y * q2.x);
-        s.rho = rn;
-        if (!(val[2] == val[2])) {
+        if (!(val[0] == val[0])) {
             s.breakdown = 3;
             s.active = 0;
-        } else if (val[2] <= s.thresh || s.iters >= s.maxiter) {
+        } else if (val[0] <= s.thresh || s.iters >= s.maxiter) {
             s.active = 0;
-        } else if (rn.x * rn.x + rn.y * rn.y == 0.0 || d1 == 0.0) {
+        } else if (s.rho.x * s.rho.x + s.rho.y * s.rho.y == 0.0) {
             s.breakdown = 4;
             s.active = 0;
         }
     }
 }
 
-template <class P>
-__global__ void __launch_bounds__(NT) k_bicg_p(VecArgs<P> va, typename P::SElem *p, const typename P::SElem *r,
-                                               const typename P::SElem *v, const KScal *sc)
-{
-    using R = typename P::R;
-    const KScal &s = sc[blockIdx.y];
-    if (!s.active) return;
-    const cpx<R> be = {R(s.beta.x), R(s.beta.y)}, om = {R(s.omega.x), R(s.omega.y)};
-    const long rb = (long)blockIdx.y * va.rs;
-    for_chunks<P>(va.n, [&](long j, int k) {
-        cpx<R> pv[P::CW], rv[P::CW], vv[P::CW];
-        P::ld_chunk(p + rb, va.V, va.off + j, k, pv);
-        P::ld_chunk(r + rb, va.V, va.off + j, k, rv);
-        P::ld_chunk(v + rb, va.V, va.off + j, k, vv);
-#pragma unroll
-        for (int q = 0; q < P::CW; q++) {
-            cmsub(pv[q], om, vv[q]);
-            cmac(rv[q], be, pv[q]);
-        }
-        P::st_chunk(p + rb, va.V, va.off + j, k, rv);
-    });
-}
-
-// alpha (MODE 1) or omega (MODE 2) from the per-warp partial sums a fused stencil epilogue wrote:
-// part[(r * nwt + j) * 3 + k], summed in FP64 in a fixed order (one CTA per right-hand side)
+// alpha (MODE 1) or omega and beta (MODE 2) from the per-warp partial sums a fused stencil epilogue
+// wrote: part[(r * nwt + j) * RED_PARTS + k], summed in FP64 in a fixed order (one CTA per
+// right-hand side)
 template <int MODE>
 __global__ void __launch_bounds__(NT) k_bicg_fin(const double *part, long nwt, KScal *sc)
 {
-    __shared__ double sm[NT / 32][3];
+    constexpr int K = MODE == 1 ? 2 : RED_PARTS;
+    __shared__ double sm[NT / 32][K];
     const int r = blockIdx.x;
     if (!sc[r].active) return;
-    double v[3] = {0.0, 0.0, 0.0};
+    RunSum<double> v[K];
     for (long j = threadIdx.x; j < nwt; j += NT) {
-        const double *pp = part + ((long)r * nwt + j) * 3;
-        v[0] += pp[0];
-        v[1] += pp[1];
-        v[2] += pp[2];
+        const double *pp = part + ((long)r * nwt + j) * RED_PARTS;
+#pragma unroll
+        for (int k = 0; k < K; k++) v[k].add(pp[k]);
     }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < 3; k++) v[k] = warp_sum(v[k]);
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < 3; k++) sm[w][k] = v[k];
-    __syncthreads();
+    cta_sum_run<K, NT, double>(v, sm);
     if (threadIdx.x != 0) return;
-    double val[3] = {0.0, 0.0, 0.0};
-    for (int i = 0; i < NT / 32; i++)
+    double val[K];
 #pragma unroll
-        for (int k = 0; k < 3; k++) val[k] += sm[i][k];
+    for (int k = 0; k < K; k++) val[k] = v[k].value();
     KScal &s = sc[r];
-    if (MODE == 1) {  // alpha = rho / (rh, v)
+    if constexpr (MODE == 1) {  // alpha = rho / (rh, v)
         const double den = val[0] * val[0] + val[1] * val[1];
         if (den == 0.0 || !(den == den)) {
             s.breakdown = 1;
@@ -287,14 +273,8 @@ __global__ void __launch_bounds__(NT) k_bicg_fin(const double *part, long nwt, K
             return;
         }
         s.alpha = make_double2((s.rho.x * val[0] + s.rho.y * val[1]) / den, (s.rho.y * val[0] - s.rho.x * val[1]) / den);
-    } else {  // omega = (t, s) / (t, t)
-        if (val[2] == 0.0 || !(val[2] == val[2])) {
-            s.breakdown = 2;
-            s.active = 0;
-            s.omega = make_double2(0.0, 0.0);
-            return;
-        }
-        s.omega = make_double2(val[0] / val[2], val[1] / val[2]);
+    } else {
+        omega_beta(s, val);
     }
 }
 
@@ -445,7 +425,7 @@ static unsigned grid_for(long n, int nch, int nrhs)
 ddrw_status reduce_ws(ddrw_ctx *ctx, int nrhs, double **part, unsigned **ticket)
 {
     void *p;
-    ddrw_status st = workspace(ctx, "red_part", sizeof(double) * 4 * 608 * (size_t)nrhs, &p);
+    ddrw_status st = workspace(ctx, "red_part", sizeof(double) * 8 * 608 * (size_t)nrhs, &p);
     if (st) return st;
     *part = (double *)p;
     DevBuf &t = ctx->ws["red_ticket"];
@@ -502,7 +482,7 @@ void Blas<P>::bicg_s(ddrw_ctx *ctx, const VecRange &vr, E *r, const E *v, const 
 }
 
 template <class P>
-ddrw_status Blas<P>::bicg_omega(ddrw_ctx *ctx, const VecRange &vr, const E *t, const E *r, KScal *sc)
+ddrw_status Blas<P>::bicg_omega(ddrw_ctx *ctx, const VecRange &vr, const E *t, const E *r, const E *rh, KScal *sc)
 {
     double *part;
     unsigned *tk;
@@ -511,13 +491,12 @@ ddrw_status Blas<P>::bicg_omega(ddrw_ctx *ctx, const VecRange &vr, const E *t, c
     VecArgs<P> va{vr.V, vr.off, vr.n, vr.rs};
     ProfScope ps(ctx, PROF_BLAS, 0.0);
     ++ctx->launches;
-    k_bicg_omega<P><<<dim3(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(va, t, r, sc, part, tk);
+    k_bicg_omega<P><<<dim3(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(va, t, r, rh, sc, part, tk);
     return DDRW_OK;
 }
 
 template <class P>
-ddrw_status Blas<P>::bicg_xr(ddrw_ctx *ctx, const VecRange &vr, E *x, const E *p, E *r, const E *t, const E *rh,
-                             KScal *sc)
+ddrw_status Blas<P>::bicg_xrp(ddrw_ctx *ctx, const VecRange &vr, E *x, E *p, E *r, const E *t, const E *v, KScal *sc)
 {
     double *part;
     unsigned *tk;
@@ -526,17 +505,8 @@ ddrw_status Blas<P>::bicg_xr(ddrw_ctx *ctx, const VecRange &vr, E *x, const E *p
     VecArgs<P> va{vr.V, vr.off, vr.n, vr.rs};
     ProfScope ps(ctx, PROF_BLAS, 0.0);
     ++ctx->launches;
-    k_bicg_xr<P><<<dim3(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(va, x, p, r, t, rh, sc, part, tk);
+    k_bicg_xrp<P><<<dim3(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(va, x, p, r, t, v, sc, part, tk);
     return DDRW_OK;
-}
-
-template <class P>
-void Blas<P>::bicg_p(ddrw_ctx *ctx, const VecRange &vr, E *p, const E *r, const E *v, const KScal *sc)
-{
-    VecArgs<P> va{vr.V, vr.off, vr.n, vr.rs};
-    ProfScope ps(ctx, PROF_BLAS, 0.0);
-    ++ctx->launches;
-    k_bicg_p<P><<<dim3(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(va, p, r, v, sc);
 }
 
 template <class P>

@@ -28,10 +28,8 @@ template <class P> struct Blas {
     static ddrw_status bicg_init(ddrw_ctx *ctx, const VecRange &vr, E *r, E *rh, E *p, E *x, KScal *sc);
     static ddrw_status bicg_alpha(ddrw_ctx *ctx, const VecRange &vr, const E *rh, const E *v, KScal *sc);
     static void bicg_s(ddrw_ctx *ctx, const VecRange &vr, E *r, const E *v, const KScal *sc);
-    static ddrw_status bicg_omega(ddrw_ctx *ctx, const VecRange &vr, const E *t, const E *r, KScal *sc);
-    static ddrw_status bicg_xr(ddrw_ctx *ctx, const VecRange &vr, E *x, const E *p, E *r, const E *t, const E *rh,
-                               KScal *sc);
-    static void bicg_p(ddrw_ctx *ctx, const VecRange &vr, E *p, const E *r, const E *v, const KScal *sc);
+    static ddrw_status bicg_omega(ddrw_ctx *ctx, const VecRange &vr, const E *t, const E *r, const E *rh, KScal *sc);
+    static ddrw_status bicg_xrp(ddrw_ctx *ctx, const VecRange &vr, E *x, E *p, E *r, const E *t, const E *v, KScal *sc);
     static ddrw_status norm2(ddrw_ctx *ctx, const VecRange &vr, const E *f, double *out);
     static ddrw_status norm_dot(ddrw_ctx *ctx, const VecRange &vr, const E *d, const E *e, double *out);
     static void axpby(ddrw_ctx *ctx, const VecRange &vr, double a, const E *x, double b, E *y);
@@ -158,11 +156,11 @@ template <int K, int NT> __device__ bool grid_sum(double (&v)[K], double *part, 
 }
 
 // alpha (mode 1) or omega (mode 2) of the BiCGStab recurrence from the per-warp partial sums of a
-// fused stencil epilogue (DslashCall::red), nwt partials of 3 doubles per right-hand side
+// fused stencil epilogue (DslashCall::red), nwt partials of RED_PARTS doubles per right-hand side
 void bicg_fin(ddrw_ctx *ctx, int mode, int nrhs, const double *part, long nwt, KScal *sc);
 
 // partial-sum and ticket buffers of grid_sum for nrhs right-hand sides (at most 608 CTAs per
-// right-hand side and 4 doubles per CTA)
+// right-hand side and 8 doubles per CTA)
 ddrw_status reduce_ws(ddrw_ctx *ctx, int nrhs, double **part, unsigned **ticket);
 
 // FP64 fields <-> storage precision P (FP32, FP16, BF16) over a range, with a per-right-hand-side

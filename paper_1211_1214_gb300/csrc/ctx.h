@@ -328,8 +328,8 @@ struct DslashCall {
     int diag = 0, post = 0, hopsel = 0;
     int par0 = 0, npar = 2, blk0 = 0, nblk = 0;
     // fused inner products of the output (FP32 storage, all hops, one parity, one right-hand side
-    // per thread): red 1 -> conj(w) out, red 2 -> conj(out) x and |out|^2, per warp of 32 sites into
-    // red_part[(rhs * (n / 32) + warp) * 3 + k]
+    // per thread): red 1 -> conj(w) out, red 2 -> conj(out) x, |out|^2, conj(w) x and conj(w) out, per
+    // warp of 32 sites into red_part[(rhs * (n / 32) + warp) * RED_PARTS + k]
     int red = 0;
     const void *w = nullptr;
     double *red_part = nullptr;

@@ -44,8 +44,8 @@ template <class P> struct DsArgs {
     const typename P::UElem *Ubw;         // backward links U_mu(x - mu) stored at x (staged form)
     int *err;                             // device error flags (bit 0: a staging wait ran out)
     int stall_tx;                         // test switch: bytes announced on top of the staged copies
-    const typename P::SElem *w;           // fused inner products: the other vector of red 1
-    double *part;                         // per-warp partial sums [rhs][n / 32][3]
+    const typename P::SElem *w;           // fused inner products: the vector rh
+    double *part;                         // per-warp partial sums [rhs][n / 32][RED_PARTS]
     long nwt;                             // warps of 32 output sites per right-hand side (n / 32)
 };
 
@@ -226,7 +226,7 @@ constexpr size_t STAGED_SMEM_MAX = (size_t)62 * 128 * 16;
 // 6 / 7 as 5 / 4 with the neighbours read from the neighbour table instead of computed,
 // 11 fully rolled (one body for the eight hops; double-single storage only)
 // RED != 0 adds the inner products of the output to the epilogue (red 1: conj(w) out; red 2:
-// conj(out) x and |out|^2), one partial per warp of 32 sites, summed in FP64 by k_bicg_fin; the
+// conj(out) x, |out|^2, conj(w) x and conj(w) out), one partial per warp of 32 sites, summed in FP64 by k_bicg_fin; the
 // launcher only fuses launches whose output sites fill whole CTAs (no thread leaves early)
 template <class P, int BL, int HOPSEL, int NR, int ROLL = 0, int RED = 0>
 __global__ void __launch_bounds__(256, (ROLL == 4 || ROLL == 7) ? 3 : (ROLL == 5 || ROLL == 6) ? 2 : 1)
@@ -348,30 +348,38 @@ __global__ void __launch_bounds__(256, (ROLL == 4 || ROLL == 7) ? 3 : (ROLL == 5
     }
     if constexpr (RED != 0) {
         static_assert(NR == 1, "fused inner products take one right-hand side per thread");
-        Spinor<R> q;
-        P::load_spinor(RED == 1 ? a.w + roff : a.x + roff, g.V, s, q);
-        R d0 = 0, d1 = 0, d2 = 0;
+        constexpr int K = RED == 1 ? 2 : RED_PARTS;
+        Spinor<R> h, q;
+        P::load_spinor(a.w + roff, g.V, s, h);
+        if (RED == 2) P::load_spinor(a.x + roff, g.V, s, q);
+        R d[K] = {};
 #pragma unroll
         for (int sp = 0; sp < 4; sp++)
 #pragma unroll
             for (int c = 0; c < 3; c++) {
-                const cpx<R> z = RED == 1 ? cmulc(q.v[sp][c], acc[0].v[sp][c]) : cmulc(acc[0].v[sp][c], q.v[sp][c]);
-                d0 += z.re;
-                d1 += z.im;
-                d2 += acc[0].v[sp][c].re * acc[0].v[sp][c].re + acc[0].v[sp][c].im * acc[0].v[sp][c].im;
+                const cpx<R> o = acc[0].v[sp][c], hv = h.v[sp][c];
+                const cpx<R> ho = cmulc(hv, o);
+                if constexpr (RED == 1) {
+                    d[0] += ho.re;
+                    d[1] += ho.im;
+                } else {
+                    const cpx<R> os = cmulc(o, q.v[sp][c]), hs = cmulc(hv, q.v[sp][c]);
+                    d[0] += os.re;
+                    d[1] += os.im;
+                    d[2] += o.re * o.re + o.im * o.im;
+                    d[3] += hs.re;
+                    d[4] += hs.im;
+                    d[5] += ho.re;
+                    d[6] += ho.im;
+                }
             }
-        double e0 = d0, e1 = d1, e2 = d2;
+        double *pp = a.part + ((long)r0 * a.nwt + tile * (blockDim.x >> 5) + (threadIdx.x >> 5)) * RED_PARTS;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            e0 += __shfl_xor_sync(0xffffffffu, e0, o);
-            e1 += __shfl_xor_sync(0xffffffffu, e1, o);
-            e2 += __shfl_xor_sync(0xffffffffu, e2, o);
-        }
-        if ((threadIdx.x & 31) == 0) {
-            double *pp = a.part + ((long)r0 * a.nwt + tile * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 3;
-            pp[0] = e0;
-            pp[1] = e1;
-            pp[2] = e2;
+        for (int k = 0; k < K; k++) {
+            double e = d[k];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+            if ((threadIdx.x & 31) == 0) pp[k] = e;
         }
     }
 #pragma unroll
@@ -691,7 +699,7 @@ double compulsory_bytes(const DslashCall &c, long n)
     if (c.beta != 0.0) per += (c.npar == 1 ? 8.0 : 4.0) * Lk;
     if (c.diag == 1) per += Cb;
     if (c.post) per += Cb;
-    if (c.red == 1) per += S * c.nrhs;  // the fused inner product's second vector
+    if (c.red != 0) per += S * c.nrhs;  // the fused inner products' vector rh
     return per * (double)n;
 }
 

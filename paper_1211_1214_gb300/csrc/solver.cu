@@ -183,22 +183,20 @@ static ddrw_status bicg_iteration(ddrw_ctx *ctx, const MassSet &ms, int nrhs, lo
         // the inner products of alpha and omega in the epilogue of the stencil that writes v and t
         const long nwt = ctx->vh / 32;
         double *part;
-        if ((s2 = workspace(ctx, "eo_redpart", sizeof(double) * 3 * (size_t)nwt * nrhs, (void **)&part))) return s2;
+        if ((s2 = workspace(ctx, "eo_redpart", sizeof(double) * RED_PARTS * (size_t)nwt * nrhs, (void **)&part))) return s2;
         apply_mhat<P>(ctx, ms, nrhs, rs, p, tmp, v, colour, 1, rh, part);
         bicg_fin(ctx, 1, nrhs, part, nwt, sc);
         Blas<P>::bicg_s(ctx, ev, r, v, sc);
-        apply_mhat<P>(ctx, ms, nrhs, rs, r, tmp, t, colour, 2, nullptr, part);
+        apply_mhat<P>(ctx, ms, nrhs, rs, r, tmp, t, colour, 2, rh, part);
         bicg_fin(ctx, 2, nrhs, part, nwt, sc);
     } else {
         apply_mhat<P>(ctx, ms, nrhs, rs, p, tmp, v, colour);
         if ((s2 = Blas<P>::bicg_alpha(ctx, ev, rh, v, sc))) return s2;
         Blas<P>::bicg_s(ctx, ev, r, v, sc);
         apply_mhat<P>(ctx, ms, nrhs, rs, r, tmp, t, colour);
-        if ((s2 = Blas<P>::bicg_omega(ctx, ev, t, r, sc))) return s2;
+        if ((s2 = Blas<P>::bicg_omega(ctx, ev, t, r, rh, sc))) return s2;
     }
-    if ((s2 = Blas<P>::bicg_xr(ctx, ev, x, p, r, t, rh, sc))) return s2;
-    Blas<P>::bicg_p(ctx, ev, p, r, v, sc);
-    return DDRW_OK;
+    return Blas<P>::bicg_xrp(ctx, ev, x, p, r, t, v, sc);
 }
 
 // Inner even-odd BiCGStab in policy P: solve D x = b (full fields) until the even-odd residual of
@@ -301,9 +299,9 @@ ddrw_status eo_bicgstab(ddrw_ctx *ctx, const MassSet &ms, const typename P::SEle
         DDRW_CUDA_CHECK(cudaMemcpyAsync(&it, count, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
         DDRW_CUDA_CHECK(cudaMemcpyAsync(hs, sc, sizeof(KScal) * nrhs, cudaMemcpyDeviceToHost, ctx->stream));
         DDRW_SYNC(ctx);
-        // kernels the graph ran: 9 per iteration (4 stencil sweeps, 5 vector kernels) and one
+        // kernels the graph ran: 8 per iteration (4 stencil sweeps, 4 vector kernels) and one
         // condition kernel per `check` iterations
-        ctx->launches += (long)(it - it0) * 9 + (it - it0) / check;
+        ctx->launches += (long)(it - it0) * 8 + (it - it0) / check;
     } else {
         while (!done) {
             for (int k = 0; k < check; k++, it++)
@@ -491,7 +489,7 @@ static ddrw_status eo_bicgstab_reliable(ddrw_ctx *ctx, const MassSet &ms, const 
             DDRW_CUDA_CHECK(cudaMemcpyAsync(&it, count, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
             DDRW_CUDA_CHECK(cudaMemcpyAsync(hs, sc, sizeof(KScal) * nrhs, cudaMemcpyDeviceToHost, ctx->stream));
             DDRW_SYNC(ctx);  // (also keeps the host arrays above alive until the copies have run)
-            ctx->launches += (long)(it - it0) * 9 + (it - it0) / check;
+            ctx->launches += (long)(it - it0) * 8 + (it - it0) / check;
         } else {
             for (int k = 0; k < check; k++, it++)
                 if ((st = iteration())) return st;
@@ -797,7 +795,7 @@ ddrw_status full_solve_dc_prepare(ddrw_ctx *ctx, int nrhs)
     if ((st = workspace(ctx, "dcf_ctl", sizeof(int), &p))) return st;
     if ((st = workspace(ctx, "full_e64", sizeof(double2) * 12 * ctx->V * nrhs, &p))) return st;
     if ((st = workspace(ctx, "eo_graph_count", sizeof(int), &p))) return st;
-    if ((st = workspace(ctx, "eo_redpart", sizeof(double) * 3 * (size_t)(ctx->vh / 32) * nrhs, &p))) return st;
+    if ((st = workspace(ctx, "eo_redpart", sizeof(double) * RED_PARTS * (size_t)(ctx->vh / 32) * nrhs, &p))) return st;
     return DDRW_OK;
 }
 
