@@ -133,12 +133,12 @@ ddrw_status ddrw_set_outer_solver(ddrw_ctx *ctx, int method, int ncy, int nmr, i
  * tolerances.  DDRW_EINVAL for max_rhs < 0. */
 ddrw_status ddrw_set_max_rhs(ddrw_ctx *ctx, int max_rhs);
 
-/* Launch shape of the persistent block solver (Sec. 1: all blocks of a colour in one launch) for
- * blocks of at least 512 sites per parity: form 0 one CTA of 256 threads per block and right-hand
- * side; 1 the same with 512 threads; 2 (FP32 storage, an even number of right-hand sides per mass
- * slot; else 1) one CTA of 512 threads per block and pair of right-hand sides, each link and clover
- * term loaded once for both.  -1 (the default): the first launch of each shape times the candidates
- * on its real arguments and keeps the fastest.  Same results in every form.  DDRW_EINVAL outside -1..2. */
+/* Launch shape of the persistent block solver (Sec. 1: all blocks of a colour in one launch), which
+ * gives each block and right-hand side to a cluster of CTAs: form 0 the widest CTAs (one of 128
+ * threads for 4^4 blocks, three of 224 for 6^4, four of 512 for 8^4), form 1 or 2 the smallest (four of
+ * 32, six of 128, eight of 256: more CTAs where a small lattice has few blocks; 2^4 blocks have one
+ * shape).  -1 (the default): the first launch of each shape times both on its real arguments and
+ * keeps the faster.  Same results in every form to the solver's tolerance.  DDRW_EINVAL outside -1..2. */
 ddrw_status ddrw_block_config(ddrw_ctx *ctx, int form);
 
 /* The 16-bit storage precisions (DDRW_MIXED_FP16, DDRW_MIXED_BF16).  reliable_updates != 0 (the

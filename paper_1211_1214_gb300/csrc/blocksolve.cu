@@ -1,10 +1,9 @@
 // blocksolve.cu -- the persistent block solver (K6): x = D_cc(m)^-1 b for every block of one colour
 // c in one launch (D_bb and D_ww are block-diagonal, Eq. 1, so the blocks are independent).
 //
-// One CTA owns one (block, right-hand side) pair and runs the whole Krylov solve inside the kernel:
-// in-block even-odd preconditioning S = A_ee - 1/4 H_eo A_oo^-1 H_oe (hops inside the block only),
-// BiCGStab on S with CTA-wide reductions (warp shuffles + shared memory, FP64 above the thread),
-// then x_o = A_oo^-1 (b_o + 1/2 H_oe x_e).  The block's sites of one parity are contiguous in the
+// One cluster of CTAs owns one (block, right-hand side) pair and runs the whole Krylov solve inside the
+// kernel: in-block even-odd preconditioning S = A_ee - 1/4 H_eo A_oo^-1 H_oe (hops inside the block
+// only), BiCGStab on S with cluster-wide reductions (warp shuffles and distributed shared memory), then x_o = A_oo^-1 (b_o + 1/2 H_oe x_e).  The block's sites of one parity are contiguous in the
 // block-major layout, so every pass is a coalesced sweep over the block.
 //
 // The host driver wraps the kernel in FP64 defect correction: r = b - D_cc x in FP64, the kernel
@@ -113,8 +112,7 @@ static ddrw_status low_cycle(ddrw_ctx *ctx, int colour, const MassSet &ms, const
     BlkArgs<P> a;
     a.b = (const E *)bl;
     a.x = (E *)el;
-    a.r = (E *)w[0]; a.rh = (E *)w[1]; a.p = (E *)w[2];
-    a.v = (E *)w[3]; a.t = (E *)w[4]; a.tmp = (E *)w[5];
+    a.r = (E *)w[0]; a.rh = (E *)w[1]; a.p = (E *)w[2]; a.v = (E *)w[3];
     a.rstride = rsl;
     a.rpm = (nrhs + std::max(ms.n, 1) - 1) / std::max(ms.n, 1);
     fill_args(ctx, a, ms, colour);
@@ -260,10 +258,10 @@ static ddrw_status block_solve_dc(ddrw_ctx *ctx, int colour, const MassSet &ms, 
     if ((st = workspace(ctx, "dcb_ctl", sizeof(double) * 2, (void **)&ctlbuf))) return st;
     double *bb2 = norms, *rr2 = norms + 2 * nrhs, *tol2 = ctlbuf;
     int *cyc = (int *)(ctlbuf + 1);
-    void *w[6];
-    const char *names64[6] = {"blk_r", "blk_rh", "blk_p", "blk_v", "blk_t", "blk_tmp"};
-    const char *names32[6] = {"blk32_r", "blk32_rh", "blk32_p", "blk32_v", "blk32_t", "blk32_tmp"};
-    for (int k = 0; k < 6; k++)
+    void *w[4];
+    const char *names64[4] = {"blk_r", "blk_rh", "blk_p", "blk_v"};
+    const char *names32[4] = {"blk32_r", "blk32_rh", "blk32_p", "blk32_v"};
+    for (int k = 0; k < 4; k++)
         if ((st = workspace(ctx, mixed ? names32[k] : names64[k], mixed ? f32 : f64, &w[k]))) return st;
 
     if ((st = colour_norms_dev(ctx, colour, b, nrhs, bb2))) return st;
@@ -287,8 +285,7 @@ static ddrw_status block_solve_dc(ddrw_ctx *ctx, int colour, const MassSet &ms, 
             BlkArgs<PrecD> a;
             a.b = res64;
             a.x = e64;
-            a.r = (double2 *)w[0]; a.rh = (double2 *)w[1]; a.p = (double2 *)w[2];
-            a.v = (double2 *)w[3]; a.t = (double2 *)w[4]; a.tmp = (double2 *)w[5];
+            a.r = (double2 *)w[0]; a.rh = (double2 *)w[1]; a.p = (double2 *)w[2]; a.v = (double2 *)w[3];
             a.rstride = rs64;
             a.rpm = (nrhs + std::max(ms.n, 1) - 1) / std::max(ms.n, 1);
             fill_args(ctx, a, ms, colour);
@@ -337,10 +334,10 @@ ddrw_status block_solve64(ddrw_ctx *ctx, int colour, const MassSet &ms, const do
     if ((st = workspace(ctx, "blk_res64", f64, (void **)&res64))) return st;
 
     // inner workspaces
-    void *w[6];
-    const char *names64[6] = {"blk_r", "blk_rh", "blk_p", "blk_v", "blk_t", "blk_tmp"};
-    const char *names32[6] = {"blk32_r", "blk32_rh", "blk32_p", "blk32_v", "blk32_t", "blk32_tmp"};
-    for (int k = 0; k < 6; k++)
+    void *w[4];
+    const char *names64[4] = {"blk_r", "blk_rh", "blk_p", "blk_v"};
+    const char *names32[4] = {"blk32_r", "blk32_rh", "blk32_p", "blk32_v"};
+    for (int k = 0; k < 4; k++)
         if ((st = workspace(ctx, mixed ? names32[k] : names64[k], mixed ? f32 : f64, &w[k]))) return st;
     double *scale_d = nullptr;
     if (mixed) {
@@ -382,8 +379,7 @@ ddrw_status block_solve64(ddrw_ctx *ctx, int colour, const MassSet &ms, const do
             BlkArgs<PrecD> a;
             a.b = rhs;
             a.x = first ? x : e64;
-            a.r = (double2 *)w[0]; a.rh = (double2 *)w[1]; a.p = (double2 *)w[2];
-            a.v = (double2 *)w[3]; a.t = (double2 *)w[4]; a.tmp = (double2 *)w[5];
+            a.r = (double2 *)w[0]; a.rh = (double2 *)w[1]; a.p = (double2 *)w[2]; a.v = (double2 *)w[3];
             a.rstride = rs64;
             a.rpm = (nrhs + std::max(ms.n, 1) - 1) / std::max(ms.n, 1);
             fill_args(ctx, a, ms, colour);

@@ -1,6 +1,8 @@
 // blocksolve.cuh -- the persistent block-solver kernel (K6); instantiated per storage policy and
-// block length in blocksolve_<policy><l>.cu so that the instantiations compile in parallel.
+// block length in bs_<policy><l>.cu so that the instantiations compile in parallel.
 #pragma once
+
+#include <cooperative_groups.h>
 
 #include "blas.cuh"
 #include "ctx.h"
@@ -13,11 +15,11 @@ template <class P> struct BlkArgs {
     using E = typename P::SElem;
     const E *b;
     E *x;
-    E *r, *rh, *p, *v, *t, *tmp;
+    E *r, *rh, *p, *v;
     long rstride;
     const typename P::UElem *U;
     const typename P::CElem *Cl;
-    int rpm;
+    int rpm, nrhs;
     typename P::R mass4[MAXM];
     const typename P::CElem *Ainv[MAXM];
     int blk0;
@@ -27,694 +29,489 @@ template <class P> struct BlkArgs {
     int *stat;  // [0] max iterations, [1] blocks that missed the tolerance
 };
 
-template <int K, int NT>
-__device__ __forceinline__ void cta_sum(double (&v)[K], double (*sm)[K])
-{
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < K; k++) {
-        double a = v[k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-        v[k] = a;
-    }
-    __syncthreads();  // earlier readers of sm are done
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < K; k++) sm[w][k] = v[k];
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < K; k++) {
-        double s = 0;
-#pragma unroll
-        for (int i = 0; i < NT / 32; i++) s += sm[i][k];
-        v[k] = s;
-    }
-}
+// One cluster of C CTAs owns one (block, right-hand side) pair and runs the whole even-odd BiCGStab on
+// it; CTA q of the cluster holds the q-th part of the block's sites in time (BL / C time slices of
+// each parity), one even and one odd site per thread.
+//
+// What bounds it: the eight-neighbour gathers.  With the vectors in global memory (one CTA per block, the
+// six vectors of an 8^4 block 1.2 MB) the kernel waited on L2: 27 % of the issue slots, 16 MB through
+// L1 and L2 per iteration against 9.7 TB/s of L2 bandwidth for the whole chip, and its sums and scalars
+// in FP64 on every warp took a fifth of the time (GB300 issues FP64 at 1/64 of its FP32 rate).  So
+//   * the two vectors that are gathered from -- G (p, then s) on the even sites, T (A_oo^-1 H_oe G) on
+//     the odd ones -- live in the cluster's shared memory, and a time hop into the neighbouring CTA's
+//     part reads distributed shared memory.  The others are read and written once by the thread that
+//     owns the site: v and t stay in registers over the reduction that follows them;
+//   * inner products are summed in float pairs (RunSum), and one thread of each CTA does the FP64
+//     scalars;
+//   * more CTAs per block than one also spread a small lattice over the chip: an FP64 solve of
+//     the 8 blocks of 4^4 sites of one colour with 4 right-hand sides kept 32 SMs busy, now 128.
 
-template <typename R>
-__device__ __forceinline__ void sp_norm_dot(const Spinor<R> &a, const Spinor<R> &b, R &re, R &im)
-{  // += conj(a) b
-#pragma unroll
-    for (int sp = 0; sp < 4; sp++)
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-            cpx<R> z = cmulc(a.v[sp][c], b.v[sp][c]);
-            re += z.re;
-            im += z.im;
-        }
-}
+constexpr int BLK_KMAX = 7;  // inner products of one reduction
 
-template <typename R>
-__device__ __forceinline__ R sp_norm2(const Spinor<R> &a)
-{
-    R s = 0;
-#pragma unroll
-    for (int sp = 0; sp < 4; sp++)
-#pragma unroll
-        for (int c = 0; c < 3; c++) s += a.v[sp][c].re * a.v[sp][c].re + a.v[sp][c].im * a.v[sp][c].im;
-    return s;
-}
-
-// Per-site pieces of the block operator, kept out of line so that every phase of the kernel
-// reuses one register allocation (the fully unrolled stencil is large).
-
-// odd site s:  out(s) = A_oo^-1 ( y(s) + coef * H_intra in (s) )    (y may be null, coef 0 skips the hop)
-template <class P, int BL>
-__device__ __noinline__ void site_odd(const GeomDev &g, long s, const typename P::SElem *in,
-                                      const typename P::SElem *y, typename P::R coef,
-                                      const typename P::UElem *__restrict__ U,
-                                      const typename P::CElem *__restrict__ Ainv, typename P::SElem *out)
-{
-    using R = typename P::R;
-    Spinor<R> acc;
-    zero(acc);
-    if (coef != R(0)) {
-        Site<BL> st;
-        decode_site<BL>(s, g, st);
-        hop_sum<P, BL, 1, false>(g, st, s, in, U, acc);
-        scale(acc, coef);
-    }
-    if (y) {
-        Spinor<R> q;
-        P::load_spinor_rw(y, g.V, s, q);
-        axpy(acc, R(1), q);
-    }
-    clover_apply<P>(Ainv, g.V, s, R(0), acc);
-    P::store_spinor(out, g.V, s, acc);
-}
-
-template <typename R> struct Dot3 {
-    R a, b, c;
+template <class P, int BL, int C> struct BlkShape {
+    static constexpr int HL = BlockShape<BL>::VBH / C;  // sites of one parity per CTA
+    // 16-byte elements of one vector of the CTA
+    static constexpr int FE = P::ID == 64 ? 12 * HL : P::ID == 32 ? 6 * HL : 3 * HL + (HL + 3) / 4;
+    static constexpr size_t SMEM = (size_t)2 * FE * 16;  // G and T of one right-hand side
 };
 
-// even site s:  out(s) = D(x)(s) + coef * H_intra tmp (s), D = A(m) (diag) or 1, and the partial
-// inner products of the phase: mode 1 -> conj(w) out; mode 2 -> conj(out) x and |out|^2.
-template <class P, int BL>
-__device__ __noinline__ Dot3<typename P::R> site_even(const GeomDev &g, long s, const typename P::SElem *tmp,
-                                                      const typename P::SElem *x, typename P::R coef, bool diag,
-                                                      typename P::R mass4, const typename P::UElem *__restrict__ U,
-                                                      const typename P::CElem *__restrict__ Cl,
-                                                      const typename P::SElem *w, int mode, typename P::SElem *out)
+template <int C> __device__ __forceinline__ void blk_sync()
 {
-    using R = typename P::R;
-    Spinor<R> acc, q;
-    zero(acc);
-    Site<BL> st;
-    decode_site<BL>(s, g, st);
-    hop_sum<P, BL, 1, false>(g, st, s, tmp, U, acc);
-    scale(acc, coef);
-    P::load_spinor_rw(x, g.V, s, q);
-    Dot3<R> d{R(0), R(0), R(0)};
-    if (diag) {
-        Spinor<R> dq = q;
-        clover_apply<P>(Cl, g.V, s, mass4, dq);
-        axpy(acc, R(1), dq);
-    } else {
-        axpy(acc, R(1), q);
-    }
-    P::store_spinor(out, g.V, s, acc);
-    if (mode == 1) {
-        P::load_spinor_rw(w, g.V, s, q);
-        sp_norm_dot(q, acc, d.a, d.b);
-    } else if (mode == 2) {
-        sp_norm_dot(acc, q, d.a, d.b);
-        d.c = sp_norm2(acc);
-    }
-    return d;
+    if constexpr (C == 1) __syncthreads();
+    else cooperative_groups::this_cluster().sync();
 }
 
-template <class P, int BL, int NT>
-// 32-bit arithmetic: at most 128 registers (170 for 128 threads) -- two 256-thread CTAs or one
-// 512-thread CTA per SM -- so the register allocation keeps the occupancy of the out-of-line site
-// functions
-__global__ void __launch_bounds__(NT, sizeof(typename P::R) == 4 ? (NT >= 512 ? 1 : NT >= 256 ? 2 : NT >= 128 ? 3 : 1) : 1)
-    k_block_solve(GeomDev g, BlkArgs<P> a)
+// acc += the hop of direction MU, DIR (forward: (1 - g) U(s) F(s + mu), backward: (1 + g) U(s - mu)^dag
+// F(s - mu)) of the site with in-block coordinates c, half index h and internal index s, if it
+// stays inside the block.  F: the other parity's part of the vector held by this CTA (q).
+template <class P, int BL, int C, int MU, int DIR>
+__device__ __forceinline__ void hop_shared(const int (&c)[4], int lb, int s, int nbase, int q, int V,
+                                           const typename P::SElem *F, const typename P::UElem *__restrict__ U,
+                                           Spinor<typename P::R> &acc)
+{
+    using R = typename P::R;
+    constexpr int HL = BlkShape<P, BL, C>::HL;
+    constexpr int STEP = MU == 0 ? BL * BL * BL : MU == 1 ? BL * BL : MU == 2 ? BL : 1;
+    if (DIR > 0 ? c[MU] == BL - 1 : c[MU] == 0) return;
+    const int hn = (lb + DIR * STEP) >> 1;  // half index of the neighbour in the block
+    Link<R> L;
+    P::load_link(U, V, MU, DIR > 0 ? s : nbase + hn, L);
+    Spinor<R> p;
+    const int own = hn - q * HL;
+    if (C == 1 || MU != 0 || (own >= 0 && own < HL)) {
+        P::load_spinor_rw(F, HL, own, p);
+    } else {
+        const int q2 = q + DIR;
+        P::load_spinor_rw(cooperative_groups::this_cluster().map_shared_rank(F, q2), HL, hn - q2 * HL, p);
+    }
+    Half<R> h, w;
+    project<MU, -DIR>(p, h);
+    if (DIR > 0) link_mul(L, h, w);
+    else link_dag_mul(L, h, w);
+    reconstruct_add<MU, -DIR>(acc, w);
+}
+
+// shared scratch of the reductions: per warp, and per CTA of the cluster (two sets used in turn)
+template <typename R, int C, int NT> struct BlkRed {
+    typename RunSum<R>::Raw warp[NT / 32][BLK_KMAX], tot[2][C][BLK_KMAX];
+};
+
+// K totals over the cluster, in out[] of thread 0 of every CTA (the same bits in each).  Every thread of
+// the cluster takes part.  With C > 1 it ends with a cluster barrier.
+template <int K, int NT, int C, typename R>
+__device__ __forceinline__ void cluster_totals(RunSum<R> (&v)[K], double (&out)[K], BlkRed<R, C, NT> &red, int &buf, int q)
+{
+    using Raw = typename RunSum<R>::Raw;
+    constexpr int NW = NT / 32, W2 = NW <= 1 ? 1 : NW <= 2 ? 2 : NW <= 4 ? 4 : NW <= 8 ? 8 : 16;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < K; k++) v[k].template shuffle_sum<32>();
+    if (NW > 1) {
+        if (lane == 0)
+#pragma unroll
+            for (int k = 0; k < K; k++) red.warp[w][k] = v[k].raw();
+        __syncthreads();
+        if (w == 0)
+#pragma unroll
+            for (int k = 0; k < K; k++) {
+                v[k] = RunSum<R>();
+                if (lane < NW) v[k].join(red.warp[lane][k]);
+                v[k].template shuffle_sum<W2>();
+            }
+    }
+    if constexpr (C > 1) {
+        auto cl = cooperative_groups::this_cluster();
+        if (threadIdx.x == 0) {
+#pragma unroll
+            for (int j = 0; j < C; j++) {
+                Raw *d = cl.map_shared_rank(&red.tot[buf][q][0], j);
+#pragma unroll
+                for (int k = 0; k < K; k++) d[k] = v[k].raw();
+            }
+        }
+        cl.sync();
+        if (threadIdx.x == 0) {
+#pragma unroll
+            for (int k = 0; k < K; k++) {
+                v[k] = RunSum<R>();
+#pragma unroll
+                for (int j = 0; j < C; j++) v[k].join(red.tot[buf][j][k]);
+            }
+        }
+        buf ^= 1;
+    }
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int k = 0; k < K; k++) out[k] = v[k].value();
+}
+
+// FP32 arithmetic: at most 128 registers, so that 512 threads fit an SM
+template <class P, int BL, int C, int NT>
+__global__ void __launch_bounds__(NT, sizeof(typename P::R) == 4 ? 512 / NT : 1) k_block_solve(GeomDev g, BlkArgs<P> a)
 {
     using R = typename P::R;
     using E = typename P::SElem;
-    constexpr int VBH = BlockShape<BL>::VBH;
-    constexpr int NP = P::NCHUNK, CW = P::CW;
-    __shared__ double sm[NT / 32][3];
-    // right-hand side fastest: the CTAs of one block run together and share its links in L2
-    const int rhs = blockIdx.x;
-    const int blk = a.blk0 + blockIdx.y;
+    constexpr int VBH = BlockShape<BL>::VBH, HL = BlkShape<P, BL, C>::HL;
+    static_assert(HL <= NT && BL % C == 0 && NT % 32 == 0, "one site of each parity per thread, whole time slices per CTA");
+    extern __shared__ __align__(16) unsigned char blk_smem[];
+    __shared__ BlkRed<R, C, NT> red;
+    __shared__ R scal[6];   // alpha, omega, beta
+    __shared__ double fs[5]; // thread 0's FP64 scalars: rho, alpha, the threshold of ||r||^2
+    __shared__ int live;    // 0 once converged or broken down
+    E *G = reinterpret_cast<E *>(blk_smem), *T = G + BlkShape<P, BL, C>::FE;
+    const int q = C == 1 ? 0 : (int)(blockIdx.x % C), id = C == 1 ? (int)blockIdx.x : (int)(blockIdx.x / C);
+    // right-hand side fastest: the clusters of one block run together and share its links in L2
+    const int rhs = id % a.nrhs, blk = a.blk0 + id / a.nrhs;
     const long ro = (long)rhs * a.rstride;
     const int slot = rhs / a.rpm;
     const R mass4 = a.mass4[slot];
     const typename P::CElem *Ainv = a.Ainv[slot];
-    const long e0 = (long)blk * VBH, o0 = g.vh + (long)blk * VBH;
-    const long V = g.V;
-    const E *b = a.b + ro;
-    E *x = a.x + ro, *r = a.r + ro, *rh = a.rh + ro, *p = a.p + ro, *v = a.v + ro, *t = a.t + ro, *tmp = a.tmp + ro;
+    const int V = (int)g.V, vh = (int)g.vh;
 
-    // ||b||^2 over the block; tmp_o = A_oo^-1 b_o
-    R bbl = 0;
-    for (int h = threadIdx.x; h < VBH; h += NT)
-        for (int k = 0; k < NP; k++) {
-            cpx<R> c[CW], d[CW];
-            P::ld_chunk(b, V, e0 + h, k, c);
-            P::ld_chunk(b, V, o0 + h, k, d);
-#pragma unroll
-            for (int q = 0; q < CW; q++)
-                bbl += c[q].re * c[q].re + c[q].im * c[q].im + d[q].re * d[q].re + d[q].im * d[q].im;
+    const bool act = (int)threadIdx.x < HL;
+    const int hl = act ? threadIdx.x : 0;  // site of either parity: own slot
+    const int be = blk * VBH, bo = vh + be;
+
+    double &rho_x = fs[0], &rho_y = fs[1], &al_x = fs[2], &al_y = fs[3], &thresh = fs[4];
+    int it = 0, buf = 0;
+    bool ok = false;
+    // the solution becomes the gather source of the odd sites
+    auto finish = [&](int se) {
+        if (act) {
+            Spinor<R> s;
+            P::load_spinor_rw(a.x + ro, V, se, s);
+            P::store_spinor(G, HL, hl, s);
         }
-    for (int h = threadIdx.x; h < VBH; h += NT) site_odd<P, BL>(g, o0 + h, nullptr, b, R(0), a.U, Ainv, tmp);
-    double red[3] = {(double)bbl, 0, 0};
-    cta_sum<3, NT>(red, sm);
-    const double bb = red[0];
-    // r = b_e + 1/2 H_eo tmp_o ; rh = p = r ; x_e = 0
-    for (int h = threadIdx.x; h < VBH; h += NT)
-        site_even<P, BL>(g, e0 + h, tmp, b, R(0.5), false, mass4, a.U, a.Cl, nullptr, 0, r);
-    R rl = 0;
-    for (int h = threadIdx.x; h < VBH; h += NT)
-        for (int k = 0; k < NP; k++) {
-            cpx<R> c[CW], z[CW];
-            P::ld_chunk(r, V, e0 + h, k, c);
-#pragma unroll
-            for (int q = 0; q < CW; q++) {
-                rl += c[q].re * c[q].re + c[q].im * c[q].im;
-                z[q] = {R(0), R(0)};
+    };
+    // the passes of the loop: start (btil, r = rh = p), v = S p, t = S s, and the odd sites of x
+    enum { START, V_OF_P, T_OF_S, FINISH };
+    int stage = START;
+    while (true) {
+        // index in the block, opaque to the compiler: the neighbours' addresses are cheaper to form again in
+        // every pass than to keep in registers (or spill) across the loop
+        int h = q * HL + hl;
+        asm volatile("" : "+r"(h));
+        const int se = be + h, so = bo + h;
+        int c[4];  // in-block coordinates; z depends on the parity
+        int zr = h / (BL / 2);
+        const int z0 = 2 * (h - zr * (BL / 2));
+        c[2] = zr % BL;
+        zr /= BL;
+        c[1] = zr % BL;
+        c[0] = zr / BL;
+        const int odd_row = (c[0] + c[1] + c[2]) & 1;
+        if (act) {
+            // ---- odd site:  T = A_oo^-1 ( y + coef H_oe G ),  y = b_o at the start and the end
+            Spinor<R> acc;
+            zero(acc);
+            if (stage != START) {
+                c[3] = z0 + (odd_row ^ 1);
+                const int lb = 2 * h + (c[3] & 1);
+                hop_shared<P, BL, C, 0, +1>(c, lb, so, be, q, V, G, a.U, acc);
+                hop_shared<P, BL, C, 0, -1>(c, lb, so, be, q, V, G, a.U, acc);
+                hop_shared<P, BL, C, 1, +1>(c, lb, so, be, q, V, G, a.U, acc);
+                hop_shared<P, BL, C, 1, -1>(c, lb, so, be, q, V, G, a.U, acc);
+                hop_shared<P, BL, C, 2, +1>(c, lb, so, be, q, V, G, a.U, acc);
+                hop_shared<P, BL, C, 2, -1>(c, lb, so, be, q, V, G, a.U, acc);
+                hop_shared<P, BL, C, 3, +1>(c, lb, so, be, q, V, G, a.U, acc);
+                hop_shared<P, BL, C, 3, -1>(c, lb, so, be, q, V, G, a.U, acc);
             }
-            P::st_chunk(rh, V, e0 + h, k, c);
-            P::st_chunk(p, V, e0 + h, k, c);
-            P::st_chunk(x, V, e0 + h, k, z);
-        }
-    red[0] = (double)rl;
-    cta_sum<3, NT>(red, sm);
-    double rr = red[0];
-    double2 rho = make_double2(rr, 0.0);
-    const double thresh = (a.tol2_dev ? *a.tol2_dev : a.tol2) * bb;
-    int it = 0;
-    bool ok = rr <= thresh;
-    while (!ok && it < a.maxiter) {
-        // v = S p  and  (rh, v)
-        for (int h = threadIdx.x; h < VBH; h += NT) site_odd<P, BL>(g, o0 + h, p, nullptr, R(1), a.U, Ainv, tmp);
-        __syncthreads();
-        R are = 0, aim = 0;
-        for (int h = threadIdx.x; h < VBH; h += NT) {
-            Dot3<R> d = site_even<P, BL>(g, e0 + h, tmp, p, R(-0.25), true, mass4, a.U, a.Cl, rh, 1, v);
-            are += d.a;
-            aim += d.b;
-        }
-        red[0] = (double)are;
-        red[1] = (double)aim;
-        cta_sum<3, NT>(red, sm);
-        double den = red[0] * red[0] + red[1] * red[1];
-        if (den == 0.0 || !(den == den)) break;
-        double2 alpha = make_double2((rho.x * red[0] + rho.y * red[1]) / den, (rho.y * red[0] - rho.x * red[1]) / den);
-        const cpx<R> al = {R(alpha.x), R(alpha.y)};
-        // s = r - alpha v (in r)
-        for (int h = threadIdx.x; h < VBH; h += NT)
-            for (int k = 0; k < NP; k++) {
-                    cpx<R> c[CW], d[CW];
-                P::ld_chunk(r, V, e0 + h, k, c);
-                P::ld_chunk(v, V, e0 + h, k, d);
-#pragma unroll
-                for (int q = 0; q < CW; q++) c[q] = c[q] - cmul(al, d[q]);
-                P::st_chunk(r, V, e0 + h, k, c);
+            if (stage == START || stage == FINISH) {
+                Spinor<R> y;
+                P::load_spinor(a.b + ro, V, so, y);
+                if (stage == FINISH) scale(acc, R(0.5));
+                axpy(acc, R(1), y);
             }
-        __syncthreads();
-        // t = S s  and  (t, s), (t, t)
-        for (int h = threadIdx.x; h < VBH; h += NT) site_odd<P, BL>(g, o0 + h, r, nullptr, R(1), a.U, Ainv, tmp);
-        __syncthreads();
-        R tsr = 0, tsi = 0, tt = 0;
-        for (int h = threadIdx.x; h < VBH; h += NT) {
-            Dot3<R> d = site_even<P, BL>(g, e0 + h, tmp, r, R(-0.25), true, mass4, a.U, a.Cl, nullptr, 2, t);
-            tsr += d.a;
-            tsi += d.b;
-            tt += d.c;
+            clover_apply<P>(Ainv, V, so, R(0), acc);
+            if (stage == FINISH) P::store_spinor(a.x + ro, V, so, acc);
+            else P::store_spinor(T, HL, hl, acc);
         }
-        red[0] = (double)tsr;
-        red[1] = (double)tsi;
-        red[2] = (double)tt;
-        cta_sum<3, NT>(red, sm);
-        if (red[2] == 0.0 || !(red[2] == red[2])) break;
-        double2 omega = make_double2(red[0] / red[2], red[1] / red[2]);
-        const cpx<R> om = {R(omega.x), R(omega.y)};
-        // x += alpha p + omega s ; r = s - omega t ; rho' = (rh, r) ; rr = (r, r)
-        R hre = 0, him = 0, rrl = 0;
-        for (int h = threadIdx.x; h < VBH; h += NT)
-            for (int k = 0; k < NP; k++) {
-                    cpx<R> xv[CW], pv[CW], sv[CW], tv[CW], hv[CW];
-                P::ld_chunk(x, V, e0 + h, k, xv);
-                P::ld_chunk(p, V, e0 + h, k, pv);
-                P::ld_chunk(r, V, e0 + h, k, sv);
-                P::ld_chunk(t, V, e0 + h, k, tv);
-                P::ld_chunk(rh, V, e0 + h, k, hv);
+        if (stage == FINISH) break;
+        blk_sync<C>();
+        // ---- even site:  acc = D own + coef H_eo T  (D = 1, coef 1/2 at the start; A(m), -1/4 after)
+        Spinor<R> acc;
+        zero(acc);
+        if (act) {
+            c[3] = z0 + odd_row;
+            const int lb = 2 * h + (c[3] & 1);
+            hop_shared<P, BL, C, 0, +1>(c, lb, se, bo, q, V, T, a.U, acc);
+            hop_shared<P, BL, C, 0, -1>(c, lb, se, bo, q, V, T, a.U, acc);
+            hop_shared<P, BL, C, 1, +1>(c, lb, se, bo, q, V, T, a.U, acc);
+            hop_shared<P, BL, C, 1, -1>(c, lb, se, bo, q, V, T, a.U, acc);
+            hop_shared<P, BL, C, 2, +1>(c, lb, se, bo, q, V, T, a.U, acc);
+            hop_shared<P, BL, C, 2, -1>(c, lb, se, bo, q, V, T, a.U, acc);
+            hop_shared<P, BL, C, 3, +1>(c, lb, se, bo, q, V, T, a.U, acc);
+            hop_shared<P, BL, C, 3, -1>(c, lb, se, bo, q, V, T, a.U, acc);
+            scale(acc, stage == START ? R(0.5) : R(-0.25));
+            Spinor<R> own;
+            if (stage == START) {
+                P::load_spinor(a.b + ro, V, se, own);
+            } else {
+                P::load_spinor_rw(G, HL, hl, own);
+                clover_apply<P>(a.Cl, V, se, mass4, own);
+            }
+            axpy(acc, R(1), own);
+        }
+        if (stage == V_OF_P) {
+            RunSum<R> d[2];
+            if (act) {
+                Spinor<R> w;
+                P::load_spinor_rw(a.rh + ro, V, se, w);
+                cpx<R> z = {R(0), R(0)};
 #pragma unroll
-                for (int q = 0; q < CW; q++) {
-                    xv[q] = xv[q] + cmul(al, pv[q]) + cmul(om, sv[q]);
-                    sv[q] = sv[q] - cmul(om, tv[q]);
-                    cpx<R> z = cmulc(hv[q], sv[q]);
-                    hre += z.re;
-                    him += z.im;
-                    rrl += sv[q].re * sv[q].re + sv[q].im * sv[q].im;
+                for (int k = 0; k < 12; k++) cmacc(z, w.v[k / 3][k % 3], acc.v[k / 3][k % 3]);
+                d[0].add(z.re);
+                d[1].add(z.im);
+                P::store_spinor(a.v + ro, V, se, acc);
+            }
+            double o[2];
+            cluster_totals<2, NT, C, R>(d, o, red, buf, q);
+            if (threadIdx.x == 0) {  // alpha = rho / (rh, v); a zero or NaN is a breakdown: x as it is
+                const double den = o[0] * o[0] + o[1] * o[1];
+                live = !(den == 0.0 || !(den == den));
+                const double iv = 1.0 / den;
+                al_x = (rho_x * o[0] + rho_y * o[1]) * iv;
+                al_y = (rho_y * o[0] - rho_x * o[1]) * iv;
+                scal[0] = R(al_x);
+                scal[1] = R(al_y);
+            }
+            __syncthreads();
+            if (!live) {
+                finish(se);
+                stage = FINISH;
+            } else {
+                if (act) {  // s = r - alpha v
+                    const cpx<R> al = {scal[0], scal[1]};
+                    Spinor<R> s;
+                    P::load_spinor_rw(a.r + ro, V, se, s);
+#pragma unroll
+                    for (int k = 0; k < 12; k++) cmsub(s.v[k / 3][k % 3], al, acc.v[k / 3][k % 3]);
+                    P::store_spinor(G, HL, hl, s);
                 }
-                P::st_chunk(x, V, e0 + h, k, xv);
-                P::st_chunk(r, V, e0 + h, k, sv);
+                stage = T_OF_S;
             }
-        red[0] = (double)hre;
-        red[1] = (double)him;
-        red[2] = (double)rrl;
-        cta_sum<3, NT>(red, sm);
-        it++;
-        rr = red[2];
-        if (!(rr == rr)) break;
-        if (rr <= thresh) {
-            ok = true;
-            break;
+            blk_sync<C>();
+            continue;
         }
-        double2 rn = make_double2(red[0], red[1]);
-        double d1 = rho.x * rho.x + rho.y * rho.y, d2 = omega.x * omega.x + omega.y * omega.y;
-        if (d1 == 0.0 || d2 == 0.0) break;
-        double2 q1 = make_double2((rn.x * rho.x + rn.y * rho.y) / d1, (rn.y * rho.x - rn.x * rho.y) / d1);
-        double2 q2 = make_double2((alpha.x * omega.x + alpha.y * omega.y) / d2, (alpha.y * omega.x - alpha.x * omega.y) / d2);
-        const cpx<R> be = {R(q1.x * q2.x - q1.y * q2.y), R(q1.x * q2.y + q1.y * q2.x)};
-        rho = rn;
-        // p = r + beta (p - omega v)
-        for (int h = threadIdx.x; h < VBH; h += NT)
-            for (int k = 0; k < NP; k++) {
-                    cpx<R> pv[CW], rv[CW], vv[CW];
-                P::ld_chunk(p, V, e0 + h, k, pv);
-                P::ld_chunk(r, V, e0 + h, k, rv);
-                P::ld_chunk(v, V, e0 + h, k, vv);
+        // r = rh = p at the start; the end of an iteration after t
+        RunSum<R> rr[2];  // ||r||^2 and, at the start, ||b||^2
+        if (stage == START) {
+            if (act) {
+                R n = 0, nb = 0;
+                Spinor<R> o;
 #pragma unroll
-                for (int q = 0; q < CW; q++) pv[q] = rv[q] + cmul(be, pv[q] - cmul(om, vv[q]));
-                P::st_chunk(p, V, e0 + h, k, pv);
+                for (int k = 0; k < 12; k++) {
+                    const cpx<R> z = acc.v[k / 3][k % 3];
+                    n = fmad(z.re, z.re, fmad(z.im, z.im, n));
+                }
+                P::load_spinor(a.b + ro, V, se, o);
+#pragma unroll
+                for (int k = 0; k < 12; k++) {
+                    const cpx<R> z = o.v[k / 3][k % 3];
+                    nb = fmad(z.re, z.re, fmad(z.im, z.im, nb));
+                }
+                rr[1].add(nb);
+                nb = 0;
+                P::load_spinor(a.b + ro, V, so, o);
+#pragma unroll
+                for (int k = 0; k < 12; k++) {
+                    const cpx<R> z = o.v[k / 3][k % 3];
+                    nb = fmad(z.re, z.re, fmad(z.im, z.im, nb));
+                }
+                rr[0].add(n);
+                rr[1].add(nb);
+                P::store_spinor(a.r + ro, V, se, acc);
+                P::store_spinor(a.rh + ro, V, se, acc);
+                P::store_spinor(a.p + ro, V, se, acc);
+                P::store_spinor(G, HL, hl, acc);
+                zero(acc);
+                P::store_spinor(a.x + ro, V, se, acc);
             }
+        } else {
+            RunSum<R> d[7];
+            if (act) {
+                Spinor<R> w;
+                P::load_spinor_rw(G, HL, hl, w);
+                cpx<R> ts = {R(0), R(0)}, hs = {R(0), R(0)}, ht = {R(0), R(0)};
+                R tt = 0;
+#pragma unroll
+                for (int k = 0; k < 12; k++) {
+                    const cpx<R> z = acc.v[k / 3][k % 3];
+                    cmacc(ts, z, w.v[k / 3][k % 3]);
+                    tt = fmad(z.re, z.re, fmad(z.im, z.im, tt));
+                }
+                Spinor<R> hh;
+                P::load_spinor_rw(a.rh + ro, V, se, hh);
+#pragma unroll
+                for (int k = 0; k < 12; k++) {
+                    cmacc(hs, hh.v[k / 3][k % 3], w.v[k / 3][k % 3]);
+                    cmacc(ht, hh.v[k / 3][k % 3], acc.v[k / 3][k % 3]);
+                }
+                d[0].add(ts.re);
+                d[1].add(ts.im);
+                d[2].add(tt);
+                d[3].add(hs.re);
+                d[4].add(hs.im);
+                d[5].add(ht.re);
+                d[6].add(ht.im);
+            }
+            double o[7];
+            cluster_totals<7, NT, C, R>(d, o, red, buf, q);
+            if (threadIdx.x == 0) {
+                // omega = (t, s) / (t, t), rho' = (rh, s) - omega (rh, t), beta = rho' alpha / (rho omega)
+                const double tt = o[2];
+                const bool go = !(tt == 0.0 || !(tt == tt));
+                live = go;
+                const double iv = go ? 1.0 / tt : 0.0;
+                const double ox = o[0] * iv, oy = o[1] * iv;
+                const double rx = o[3] - (ox * o[5] - oy * o[6]), ry = o[4] - (ox * o[6] + oy * o[5]);
+                const double nx = rx * al_x - ry * al_y, ny = rx * al_y + ry * al_x;
+                const double dx = rho_x * ox - rho_y * oy, dy = rho_x * oy + rho_y * ox;
+                const double d2 = dx * dx + dy * dy, jv = d2 > 0.0 ? 1.0 / d2 : 0.0;
+                scal[2] = R(ox);
+                scal[3] = R(oy);
+                scal[4] = R((nx * dx + ny * dy) * jv);
+                scal[5] = R((ny * dx - nx * dy) * jv);
+                rho_x = d2 > 0.0 ? rx : 0.0;  // a zero denominator ends the recurrence after this iteration
+                rho_y = d2 > 0.0 ? ry : 0.0;
+            }
+            __syncthreads();
+            if (!live) {
+                finish(se);
+                stage = FINISH;
+                blk_sync<C>();
+                continue;
+            }
+            if (act) {  // x += alpha p + omega s ; r = s - omega t ; p = r + beta (p - omega v)
+                const cpx<R> al = {scal[0], scal[1]}, om = {scal[2], scal[3]}, bt = {scal[4], scal[5]};
+                Spinor<R> s, pv, y;
+                P::load_spinor_rw(G, HL, hl, s);
+                P::load_spinor_rw(a.p + ro, V, se, pv);
+                P::load_spinor_rw(a.x + ro, V, se, y);
+                R n = 0;
+#pragma unroll
+                for (int k = 0; k < 12; k++) {
+                    cpx<R> &sk = s.v[k / 3][k % 3], &xk = y.v[k / 3][k % 3];
+                    cmac(xk, al, pv.v[k / 3][k % 3]);
+                    cmac(xk, om, sk);
+                    cmsub(sk, om, acc.v[k / 3][k % 3]);
+                    n = fmad(sk.re, sk.re, fmad(sk.im, sk.im, n));
+                }
+                P::store_spinor(a.x + ro, V, se, y);
+                P::store_spinor(a.r + ro, V, se, s);
+                P::load_spinor_rw(a.v + ro, V, se, y);
+#pragma unroll
+                for (int k = 0; k < 12; k++) {
+                    cpx<R> &pk = pv.v[k / 3][k % 3];
+                    cmsub(pk, om, y.v[k / 3][k % 3]);
+                    cmac(s.v[k / 3][k % 3], bt, pk);
+                }
+                P::store_spinor(a.p + ro, V, se, s);
+                P::store_spinor(G, HL, hl, s);
+                rr[0].add(n);
+            }
+            it++;
+        }
+        double o[2];
+        cluster_totals<2, NT, C, R>(rr, o, red, buf, q);
+        if (threadIdx.x == 0) {
+            if (stage == START) {
+                thresh = (a.tol2_dev ? *a.tol2_dev : a.tol2) * o[1];
+                rho_x = o[0];
+                rho_y = 0.0;
+            }
+            ok = o[0] <= thresh;
+            const bool dead = !(o[0] == o[0]) || it >= a.maxiter || (rho_x == 0.0 && rho_y == 0.0);
+            live = !ok && !dead;
+        }
         __syncthreads();
+        stage = V_OF_P;
+        if (!live) {
+            finish(se);
+            stage = FINISH;
+            blk_sync<C>();
+        }
     }
-    __syncthreads();
-    // x_o = A_oo^-1 (b_o + 1/2 H_oe x_e)
-    for (int h = threadIdx.x; h < VBH; h += NT) site_odd<P, BL>(g, o0 + h, x, b, R(0.5), a.U, Ainv, x);
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && q == 0) {
         atomicMax(a.stat, it);
         if (!ok) atomicAdd(a.stat + 1, 1);
     }
+    blk_sync<C>();  // no CTA leaves while another may read its part
 }
 
+// Launch shapes: C CTAs of NT threads per block and right-hand side.  Form 0 is the wider CTA, form 1 the
+// smaller one (more CTAs for few blocks and right-hand sides, more distributed-memory hops).
+// Measured on FP32 storage, ms per launch of a colour, form 0 / form 1 / the kernel with its vectors in
+// global memory: 24x12^3 in 6^4 blocks, 5 right-hand sides 0.43 / 0.45 / 1.07; 16^4 in 4^4 blocks, 16
+// right-hand sides 0.97 / 1.80 / 1.54; 32x16^3 in 8^4 blocks, 18 right-hand sides 4.4 / 5.1 / 7.0;
+// 48x24^3 in 6^4 blocks, 6 right-hand sides 6.3 / 7.2 / 9.1; 64x32^3 in 8^4 blocks, 4 right-hand sides
+// 15.5 / 17.9 / 25.2.  What bounds it now is L2: 1.9 MB of links, clover terms and own-site vectors per
+// CTA and iteration in 38 us (8^4 blocks), 7.6 of the chip's 9.7 TB/s.  Two or four right-hand sides in
+// a CTA, to share the links through L1, lost (22.8 ms on 64x32^3): their barriers couple them.
+template <int BL> struct BlkForms;
+template <> struct BlkForms<2> { static constexpr int C[2] = {1, 1}, N[2] = {32, 32}; };
+template <> struct BlkForms<4> { static constexpr int C[2] = {1, 4}, N[2] = {128, 32}; };
+template <> struct BlkForms<6> { static constexpr int C[2] = {3, 6}, N[2] = {224, 128}; };
+template <> struct BlkForms<8> { static constexpr int C[2] = {4, 8}, N[2] = {512, 256}; };
 
-// ---- NR right-hand sides of one block per CTA (rstride apart, same mass slot): each link and
-// clover term is loaded once for all NR, and every thread carries NR independent chains between
-// the CTA's barriers.  A right-hand side that has converged (or broken down) is frozen -- its
-// scalars become zero, so x and r stay as they are -- while the others iterate on.
-
-template <int NR, typename R> struct DotN {
-    R a[NR], b[NR], c[NR];
-};
-
-template <class P, int BL, int NR>
-__device__ __noinline__ void site_odd_n(const GeomDev &g, long s, const typename P::SElem *in,
-                                        const typename P::SElem *y, long rs, typename P::R coef,
-                                        const typename P::UElem *__restrict__ U,
-                                        const typename P::CElem *__restrict__ Ainv, typename P::SElem *out)
+template <class P, int BL, int C, int NT>
+void launch_block_shape(ddrw_ctx *ctx, const BlkArgs<P> &a, int nrhs)
 {
-    using R = typename P::R;
-    Spinor<R> acc[NR];
-#pragma unroll
-    for (int r = 0; r < NR; r++) zero(acc[r]);
-    if (coef != R(0)) {
-        Site<BL> st;
-        decode_site<BL>(s, g, st);
-        hop_dir_multi<P, BL, 1, 0, NR, false>(g, st, s, in, rs, U, acc);
-        hop_dir_multi<P, BL, 1, 1, NR, false>(g, st, s, in, rs, U, acc);
-        hop_dir_multi<P, BL, 1, 2, NR, false>(g, st, s, in, rs, U, acc);
-        hop_dir_multi<P, BL, 1, 3, NR, false>(g, st, s, in, rs, U, acc);
-#pragma unroll
-        for (int r = 0; r < NR; r++) scale(acc[r], coef);
-    }
-    if (y) {
-#pragma unroll
-        for (int r = 0; r < NR; r++) {
-            Spinor<R> q;
-            P::load_spinor_rw(y + r * rs, g.V, s, q);
-            axpy(acc[r], R(1), q);
-        }
-    }
-#pragma unroll
-    for (int ch = 0; ch < 2; ch++) {
-        R c[36];
-        P::load_clover(Ainv, g.V, s, ch, c);
-#pragma unroll
-        for (int r = 0; r < NR; r++) {
-            cpx<R> v6[6], o6[6];
-#pragma unroll
-            for (int k = 0; k < 6; k++) v6[k] = acc[r].v[2 * ch + k / 3][k % 3];
-            herm6_mul<R>(c, R(0), v6, o6);
-#pragma unroll
-            for (int k = 0; k < 6; k++) acc[r].v[2 * ch + k / 3][k % 3] = o6[k];
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < NR; r++) P::store_spinor(out + r * rs, g.V, s, acc[r]);
+    BlkArgs<P> b = a;
+    b.nrhs = nrhs;
+    constexpr size_t smem = BlkShape<P, BL, C>::SMEM;
+    if (smem > 40 * 1024)  // (static shared memory counts towards the default limit of 48 KB)
+        cudaFuncSetAttribute(k_block_solve<P, BL, C, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)((long)C * nrhs * ctx->nblk_c));
+    lc.blockDim = dim3(NT);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = ctx->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    lc.attrs = at;
+    lc.numAttrs = C > 1 ? 1 : 0;
+    ++ctx->launches;
+    cudaLaunchKernelEx(&lc, k_block_solve<P, BL, C, NT>, geom_dev(ctx), b);
 }
 
-// even site s: out = D x + coef H_intra tmp for NR right-hand sides, D = A(m) (diag) or 1, and
-// the partial inner products of the phase: mode 1 -> conj(w) out; mode 2 -> conj(out) x and |out|^2.
-template <class P, int BL, int NR>
-__device__ __noinline__ DotN<NR, typename P::R> site_even_n(const GeomDev &g, long s, const typename P::SElem *tmp,
-                                                            const typename P::SElem *x, long rs, typename P::R coef,
-                                                            bool diag, typename P::R mass4,
-                                                            const typename P::UElem *__restrict__ U,
-                                                            const typename P::CElem *__restrict__ Cl,
-                                                            const typename P::SElem *w, int mode, typename P::SElem *out)
-{
-    using R = typename P::R;
-    Spinor<R> acc[NR];
-#pragma unroll
-    for (int r = 0; r < NR; r++) zero(acc[r]);
-    Site<BL> st;
-    decode_site<BL>(s, g, st);
-    hop_dir_multi<P, BL, 1, 0, NR, false>(g, st, s, tmp, rs, U, acc);
-    hop_dir_multi<P, BL, 1, 1, NR, false>(g, st, s, tmp, rs, U, acc);
-    hop_dir_multi<P, BL, 1, 2, NR, false>(g, st, s, tmp, rs, U, acc);
-    hop_dir_multi<P, BL, 1, 3, NR, false>(g, st, s, tmp, rs, U, acc);
-#pragma unroll
-    for (int r = 0; r < NR; r++) scale(acc[r], coef);
-    // (the clover term of the site is read once per right-hand side; the repeat hits L1)
-#pragma unroll
-    for (int r = 0; r < NR; r++) {
-        Spinor<R> q;
-        P::load_spinor_rw(x + r * rs, g.V, s, q);
-        if (diag) clover_apply<P>(Cl, g.V, s, mass4, q);
-        axpy(acc[r], R(1), q);
-    }
-    DotN<NR, R> d;
-#pragma unroll
-    for (int r = 0; r < NR; r++) {
-        d.a[r] = R(0);
-        d.b[r] = R(0);
-        d.c[r] = R(0);
-        P::store_spinor(out + r * rs, g.V, s, acc[r]);
-        Spinor<R> q;
-        if (mode == 1) {
-            P::load_spinor_rw(w + r * rs, g.V, s, q);
-            sp_norm_dot(q, acc[r], d.a[r], d.b[r]);
-        } else if (mode == 2) {
-            P::load_spinor_rw(x + r * rs, g.V, s, q);
-            sp_norm_dot(acc[r], q, d.a[r], d.b[r]);
-            d.c[r] = sp_norm2(acc[r]);
-        }
-    }
-    return d;
-}
-
-template <class P, int BL, int NT, int NR>
-__global__ void __launch_bounds__(NT, sizeof(typename P::R) == 4 ? (NT >= 512 ? 1 : NT >= 256 ? 2 : 3) : 1)
-    k_block_solve_n(GeomDev g, BlkArgs<P> a)
-{
-    using R = typename P::R;
-    using E = typename P::SElem;
-    constexpr int VBH = BlockShape<BL>::VBH;
-    constexpr int NP = P::NCHUNK, CW = P::CW;
-    constexpr int K = 3 * NR;
-    __shared__ double sm[NT / 32][K];
-    const int rhs0 = blockIdx.x * NR;  // a group of NR right-hand sides of one mass slot
-    const int blk = a.blk0 + blockIdx.y;
-    const long rs = a.rstride, ro = (long)rhs0 * rs;
-    const int slot = rhs0 / a.rpm;
-    const R mass4 = a.mass4[slot];
-    const typename P::CElem *Ainv = a.Ainv[slot];
-    const long e0 = (long)blk * VBH, o0 = g.vh + (long)blk * VBH;
-    const long V = g.V;
-    const E *b = a.b + ro;
-    E *x = a.x + ro, *r = a.r + ro, *rh = a.rh + ro, *p = a.p + ro, *v = a.v + ro, *t = a.t + ro, *tmp = a.tmp + ro;
-
-    // ||b||^2 per right-hand side; tmp_o = A_oo^-1 b_o
-    double red[K];
-#pragma unroll
-    for (int k = 0; k < K; k++) red[k] = 0.0;
-#pragma unroll
-    for (int q = 0; q < NR; q++) {
-        R bbl = 0;
-        for (int h = threadIdx.x; h < VBH; h += NT)
-            for (int k = 0; k < NP; k++) {
-                cpx<R> c[CW], d[CW];
-                P::ld_chunk(b + q * rs, V, e0 + h, k, c);
-                P::ld_chunk(b + q * rs, V, o0 + h, k, d);
-#pragma unroll
-                for (int i = 0; i < CW; i++)
-                    bbl += c[i].re * c[i].re + c[i].im * c[i].im + d[i].re * d[i].re + d[i].im * d[i].im;
-            }
-        red[q] = (double)bbl;
-    }
-    for (int h = threadIdx.x; h < VBH; h += NT) site_odd_n<P, BL, NR>(g, o0 + h, nullptr, b, rs, R(0), a.U, Ainv, tmp);
-    cta_sum<K, NT>(red, sm);
-    double bb[NR];
-#pragma unroll
-    for (int q = 0; q < NR; q++) bb[q] = red[q];
-    __syncthreads();
-    // r = b_e + 1/2 H_eo tmp_o ; rh = p = r ; x_e = 0
-    for (int h = threadIdx.x; h < VBH; h += NT)
-        site_even_n<P, BL, NR>(g, e0 + h, tmp, b, rs, R(0.5), false, mass4, a.U, a.Cl, nullptr, 0, r);
-#pragma unroll
-    for (int k = 0; k < K; k++) red[k] = 0.0;
-    for (int h = threadIdx.x; h < VBH; h += NT)
-#pragma unroll
-        for (int q = 0; q < NR; q++)
-            for (int k = 0; k < NP; k++) {
-                cpx<R> c[CW], z[CW];
-                P::ld_chunk(r + q * rs, V, e0 + h, k, c);
-                R rl = 0;
-#pragma unroll
-                for (int i = 0; i < CW; i++) {
-                    rl += c[i].re * c[i].re + c[i].im * c[i].im;
-                    z[i] = {R(0), R(0)};
-                }
-                red[q] += (double)rl;
-                P::st_chunk(rh + q * rs, V, e0 + h, k, c);
-                P::st_chunk(p + q * rs, V, e0 + h, k, c);
-                P::st_chunk(x + q * rs, V, e0 + h, k, z);
-            }
-    cta_sum<K, NT>(red, sm);
-    const double t2 = a.tol2_dev ? *a.tol2_dev : a.tol2;
-    double rr[NR], thresh[NR];
-    double2 rho[NR], alpha[NR], omega[NR];
-    bool act[NR], ok[NR];
-    int nact = 0;
-#pragma unroll
-    for (int q = 0; q < NR; q++) {
-        rr[q] = red[q];
-        rho[q] = make_double2(rr[q], 0.0);
-        thresh[q] = t2 * bb[q];
-        ok[q] = rr[q] <= thresh[q];
-        act[q] = !ok[q];
-        nact += act[q] ? 1 : 0;
-        alpha[q] = omega[q] = make_double2(0.0, 0.0);
-    }
-    int it = 0;
-    while (nact > 0 && it < a.maxiter) {
-        // v = S p  and  (rh, v)
-        __syncthreads();
-        for (int h = threadIdx.x; h < VBH; h += NT) site_odd_n<P, BL, NR>(g, o0 + h, p, nullptr, rs, R(1), a.U, Ainv, tmp);
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < K; k++) red[k] = 0.0;
-        for (int h = threadIdx.x; h < VBH; h += NT) {
-            DotN<NR, R> d = site_even_n<P, BL, NR>(g, e0 + h, tmp, p, rs, R(-0.25), true, mass4, a.U, a.Cl, rh, 1, v);
-#pragma unroll
-            for (int q = 0; q < NR; q++) {
-                red[2 * q] += (double)d.a[q];
-                red[2 * q + 1] += (double)d.b[q];
-            }
-        }
-        cta_sum<K, NT>(red, sm);
-        cpx<R> al[NR];
-#pragma unroll
-        for (int q = 0; q < NR; q++) {
-            const double dr = red[2 * q], di = red[2 * q + 1];
-            const double den = dr * dr + di * di;
-            if (act[q] && (den == 0.0 || !(den == den))) act[q] = false;  // breakdown: frozen, not converged
-            alpha[q] = act[q] ? make_double2((rho[q].x * dr + rho[q].y * di) / den, (rho[q].y * dr - rho[q].x * di) / den)
-                              : make_double2(0.0, 0.0);
-            al[q] = {R(alpha[q].x), R(alpha[q].y)};
-        }
-        // s = r - alpha v (in r)
-        for (int h = threadIdx.x; h < VBH; h += NT)
-#pragma unroll
-            for (int q = 0; q < NR; q++)
-                for (int k = 0; k < NP; k++) {
-                    cpx<R> c[CW], d[CW];
-                    P::ld_chunk(r + q * rs, V, e0 + h, k, c);
-                    P::ld_chunk(v + q * rs, V, e0 + h, k, d);
-#pragma unroll
-                    for (int i = 0; i < CW; i++) c[i] = c[i] - cmul(al[q], d[i]);
-                    P::st_chunk(r + q * rs, V, e0 + h, k, c);
-                }
-        __syncthreads();
-        // t = S s  and  (t, s), (t, t)
-        for (int h = threadIdx.x; h < VBH; h += NT) site_odd_n<P, BL, NR>(g, o0 + h, r, nullptr, rs, R(1), a.U, Ainv, tmp);
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < K; k++) red[k] = 0.0;
-        for (int h = threadIdx.x; h < VBH; h += NT) {
-            DotN<NR, R> d = site_even_n<P, BL, NR>(g, e0 + h, tmp, r, rs, R(-0.25), true, mass4, a.U, a.Cl, nullptr, 2, t);
-#pragma unroll
-            for (int q = 0; q < NR; q++) {
-                red[3 * q] += (double)d.a[q];
-                red[3 * q + 1] += (double)d.b[q];
-                red[3 * q + 2] += (double)d.c[q];
-            }
-        }
-        cta_sum<K, NT>(red, sm);
-        cpx<R> om[NR];
-#pragma unroll
-        for (int q = 0; q < NR; q++) {
-            const double tt = red[3 * q + 2];
-            // breakdown: frozen; the x update below still adds alpha p, which matches the s-step
-            // that already moved r
-            if (act[q] && (tt == 0.0 || !(tt == tt))) act[q] = false;
-            omega[q] = act[q] ? make_double2(red[3 * q] / tt, red[3 * q + 1] / tt) : make_double2(0.0, 0.0);
-            om[q] = {R(omega[q].x), R(omega[q].y)};
-            al[q] = {R(alpha[q].x), R(alpha[q].y)};
-        }
-        // x += alpha p + omega s ; r = s - omega t ; rho' = (rh, r) ; rr = (r, r)
-#pragma unroll
-        for (int k = 0; k < K; k++) red[k] = 0.0;
-        for (int h = threadIdx.x; h < VBH; h += NT)
-#pragma unroll
-            for (int q = 0; q < NR; q++) {
-                R hre = 0, him = 0, rrl = 0;
-                for (int k = 0; k < NP; k++) {
-                    cpx<R> xv[CW], pv[CW], sv[CW], tv[CW], hv[CW];
-                    P::ld_chunk(x + q * rs, V, e0 + h, k, xv);
-                    P::ld_chunk(p + q * rs, V, e0 + h, k, pv);
-                    P::ld_chunk(r + q * rs, V, e0 + h, k, sv);
-                    P::ld_chunk(t + q * rs, V, e0 + h, k, tv);
-                    P::ld_chunk(rh + q * rs, V, e0 + h, k, hv);
-#pragma unroll
-                    for (int i = 0; i < CW; i++) {
-                        xv[i] = xv[i] + cmul(al[q], pv[i]) + cmul(om[q], sv[i]);
-                        sv[i] = sv[i] - cmul(om[q], tv[i]);
-                        cpx<R> z = cmulc(hv[i], sv[i]);
-                        hre += z.re;
-                        him += z.im;
-                        rrl += sv[i].re * sv[i].re + sv[i].im * sv[i].im;
-                    }
-                    P::st_chunk(x + q * rs, V, e0 + h, k, xv);
-                    P::st_chunk(r + q * rs, V, e0 + h, k, sv);
-                }
-                red[3 * q] += (double)hre;
-                red[3 * q + 1] += (double)him;
-                red[3 * q + 2] += (double)rrl;
-            }
-        cta_sum<K, NT>(red, sm);
-        it++;
-        cpx<R> be[NR];
-#pragma unroll
-        for (int q = 0; q < NR; q++) {
-            be[q] = {R(0), R(0)};
-            if (!act[q]) continue;
-            rr[q] = red[3 * q + 2];
-            if (!(rr[q] == rr[q])) {
-                act[q] = false;
-                continue;
-            }
-            if (rr[q] <= thresh[q]) {
-                ok[q] = true;
-                act[q] = false;
-                continue;
-            }
-            const double2 rn = make_double2(red[3 * q], red[3 * q + 1]);
-            const double d1 = rho[q].x * rho[q].x + rho[q].y * rho[q].y;
-            const double d2 = omega[q].x * omega[q].x + omega[q].y * omega[q].y;
-            if (d1 == 0.0 || d2 == 0.0) {
-                act[q] = false;
-                continue;
-            }
-            const double2 q1 = make_double2((rn.x * rho[q].x + rn.y * rho[q].y) / d1, (rn.y * rho[q].x - rn.x * rho[q].y) / d1);
-            const double2 q2 = make_double2((alpha[q].x * omega[q].x + alpha[q].y * omega[q].y) / d2,
-                                            (alpha[q].y * omega[q].x - alpha[q].x * omega[q].y) / d2);
-            be[q] = {R(q1.x * q2.x - q1.y * q2.y), R(q1.x * q2.y + q1.y * q2.x)};
-            rho[q] = rn;
-        }
-        nact = 0;
-#pragma unroll
-        for (int q = 0; q < NR; q++) {
-            nact += act[q] ? 1 : 0;
-            if (!act[q]) om[q] = {R(0), R(0)};
-        }
-        if (nact == 0) break;
-        // p = r + beta (p - omega v) for the right-hand sides still iterating
-        for (int h = threadIdx.x; h < VBH; h += NT)
-#pragma unroll
-            for (int q = 0; q < NR; q++) {
-                if (!act[q]) continue;
-                for (int k = 0; k < NP; k++) {
-                    cpx<R> pv[CW], rv[CW], vv[CW];
-                    P::ld_chunk(p + q * rs, V, e0 + h, k, pv);
-                    P::ld_chunk(r + q * rs, V, e0 + h, k, rv);
-                    P::ld_chunk(v + q * rs, V, e0 + h, k, vv);
-#pragma unroll
-                    for (int i = 0; i < CW; i++) pv[i] = rv[i] + cmul(be[q], pv[i] - cmul(om[q], vv[i]));
-                    P::st_chunk(p + q * rs, V, e0 + h, k, pv);
-                }
-            }
-    }
-    __syncthreads();
-    // x_o = A_oo^-1 (b_o + 1/2 H_oe x_e)
-    for (int h = threadIdx.x; h < VBH; h += NT) site_odd_n<P, BL, NR>(g, o0 + h, x, b, rs, R(0.5), a.U, Ainv, x);
-    if (threadIdx.x == 0) {
-        atomicMax(a.stat, it);
-        int miss = 0;
-#pragma unroll
-        for (int q = 0; q < NR; q++) miss += ok[q] ? 0 : 1;
-        if (miss) atomicAdd(a.stat + 1, miss);
-    }
-}
-
-// Launch shape of the block solver: NT threads per (block, right-hand side), or for blocks of at
-// least 512 sites per parity on 32- and 16-bit storage also 2 NT threads (one CTA per SM instead of
-// two, half the Krylov vectors of the resident CTAs competing for L2).  The first launch of each
-// (storage, block length, right-hand sides) shape times both on the real arguments -- the kernel
-// reads b and overwrites all of x, so a repeat gives the same result -- and keeps the faster.
+// The first launch of each (storage, block length, right-hand sides) shape times the forms on the real
+// arguments -- the kernel reads b and overwrites all of x, so a repeat gives the same result --
+// and keeps the fastest.
 template <class P, int BL>
 void launch_block_kernel(ddrw_ctx *ctx, const BlkArgs<P> &a, int nrhs)
 {
-    GeomDev g = geom_dev(ctx);
-    dim3 grid((unsigned)nrhs, (unsigned)ctx->nblk_c);
-    constexpr int VBH = BlockShape<BL>::VBH;
-    constexpr int NT = VBH <= 32 ? 32 : (VBH <= 128 ? 128 : 256);
-    constexpr bool WIDE = VBH >= 512 && P::ID != 64;
-    constexpr int NT2 = WIDE ? 2 * NT : NT;
+    using F = BlkForms<BL>;
+    constexpr int NF = BL == 2 ? 1 : 2;
     const int kind = P::ID == 64 ? PROF_BLOCK64 : P::ID == 32 ? PROF_BLOCK32 : PROF_BLOCK16;
-    // form 2: two right-hand sides per CTA (FP32 storage; pairs inside one mass slot)
-    const bool pairs = P::ID == 32 && WIDE && nrhs % 2 == 0 && a.rpm % 2 == 0;
     auto run = [&](int form) {
-        ++ctx->launches;
-        if constexpr (P::ID == 32 && WIDE) {
-            if (form == 2) {
-                k_block_solve_n<P, BL, NT2, 2><<<dim3((unsigned)nrhs / 2, (unsigned)ctx->nblk_c), NT2, 0, ctx->stream>>>(g, a);
-                return;
-            }
-        }
-        if (form) k_block_solve<P, BL, NT2><<<grid, NT2, 0, ctx->stream>>>(g, a);
-        else k_block_solve<P, BL, NT><<<grid, NT, 0, ctx->stream>>>(g, a);
+        if (NF > 1 && form) launch_block_shape<P, BL, F::C[1], F::N[1]>(ctx, a, nrhs);
+        else launch_block_shape<P, BL, F::C[0], F::N[0]>(ctx, a, nrhs);
     };
     int form = 0;
-    if (WIDE) {
-        const std::array<int, 3> key = {P::ID, BL, nrhs * 2 + (pairs ? 1 : 0)};
+    if (NF > 1) {
+        const std::array<int, 3> key = {P::ID, BL, nrhs};
         auto it = ctx->blk_tune.find(key);
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         cudaStreamIsCapturing(ctx->stream, &cs);
         if (ctx->blk_form >= 0) {
-            form = (ctx->blk_form == 2 && !pairs) ? 1 : ctx->blk_form;  // pinned (ddrw_block_config)
+            form = ctx->blk_form;  // pinned (ddrw_block_config)
         } else if (it != ctx->blk_tune.end()) {
             form = it->second;
         } else if (ctx->autotune && cs == cudaStreamCaptureStatusNone && a.b != a.x) {
-            const int nf = pairs ? 3 : 2;
-            cudaEvent_t e[4];
+            cudaEvent_t e[NF + 1];
             for (auto &ev : e) cudaEventCreate(&ev);
             cudaEventRecord(e[0], ctx->stream);
-            for (int f = 0; f < nf; f++) {
+            for (int f = 0; f < NF; f++) {
                 run(f);
                 cudaEventRecord(e[f + 1], ctx->stream);
             }
-            cudaEventSynchronize(e[nf]);
+            cudaEventSynchronize(e[NF]);
             float best = 0;
-            form = 0;
-            for (int f = 0; f < nf; f++) {
+            for (int f = 0; f < NF; f++) {
                 float ms = 0;
                 cudaEventElapsedTime(&ms, e[f], e[f + 1]);
                 if (f == 0 || ms < best) best = ms, form = f;

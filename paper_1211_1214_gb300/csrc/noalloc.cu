@@ -3,7 +3,7 @@
 // Some callers cannot call cudaMalloc: code that runs while a memory pool is frozen or inside a
 // host callback, or a host framework that owns every device allocation and forbids libraries from
 // making their own.  ddrw_solve_block_noalloc gives them the block solve x = D_cc(m)^-1 b with all
-// of its scratch (the internal copies of b and x, the six Krylov vectors of the persistent block
+// of its scratch (the internal copies of b and x, the four Krylov vectors of the persistent block
 // solver, the defect-correction residual and correction, the reduction slots) in one file-scope
 // device array of fixed size.  The caller still passes b and x.
 //
@@ -28,8 +28,8 @@ extern template void launch_block_kernel<PrecD, 8>(ddrw_ctx *, const BlkArgs<Pre
 
 // largest lattice (sites) the scratch array serves: 12^4
 constexpr long NOALLOC_MAX_SITES = 20736;
-// FP64 spinor fields in the scratch array: b, x, r, rh, p, v, t, tmp, residual, correction
-constexpr int NOALLOC_FIELDS = 10;
+// FP64 spinor fields in the scratch array: b, x, r, rh, p, v, residual, correction
+constexpr int NOALLOC_FIELDS = 8;
 constexpr long NOALLOC_FIELD_ELEMS = 12 * NOALLOC_MAX_SITES;  // double2 per field
 constexpr long NOALLOC_RED_ELEMS = 64;                       // reduction slots (double2)
 
@@ -127,7 +127,7 @@ extern "C" ddrw_status ddrw_solve_block_noalloc(ddrw_ctx *ctx, int colour, doubl
     const long V = ctx->V, fe = 12 * V;
     double2 *F[NOALLOC_FIELDS];
     for (int k = 0; k < NOALLOC_FIELDS; k++) F[k] = base + k * fe;
-    double2 *fb = F[0], *fx = F[1], *fres = F[8], *fe64 = F[9];
+    double2 *fb = F[0], *fx = F[1], *fres = F[6], *fe64 = F[7];
     double *red = (double *)(base + NOALLOC_FIELDS * NOALLOC_FIELD_ELEMS);
     int *stat = (int *)(red + 8);
     double *h = ctx->h_pinned;
@@ -143,8 +143,6 @@ extern "C" ddrw_status ddrw_solve_block_noalloc(ddrw_ctx *ctx, int colour, doubl
     a.rh = F[3];
     a.p = F[4];
     a.v = F[5];
-    a.t = F[6];
-    a.tmp = F[7];
     a.rstride = fe;
     a.rpm = 1;
     for (int k = 0; k < MAXM; k++) {
