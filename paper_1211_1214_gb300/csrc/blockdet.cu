@@ -14,6 +14,7 @@
 //     a unit vector at the same even site and component of every block gives that column of every
 //     S_k at once, because the blocks do not couple (k_unit_fields, two stencil launches,
 //     k_scatter_cols);
+//     For 2^4 blocks one kernel assembles the matrix in shared memory and factorises it there;
 //   * det S_k: a batched LU with partial pivoting in FP64, one CTA per matrix, blocked right-looking
 //     (panels of NB columns factorised in place, the trailing matrix updated once per panel with
 //     the panel's multipliers held in registers and the panel's U rows staged in shared memory).
@@ -320,31 +321,291 @@ __global__ void __launch_bounds__(LU_NT) k_lu_logdet(int n, double2 *mats, doubl
     }
 }
 
+// ----------------------------------------------------------------------------- 2^4 blocks, in shared memory
+
+// S_k of a 2^4 block is 96 x 96 (147 KB): one CTA assembles it straight from the links and the in-block
+// inverses into shared memory and factorises it there.
+//
+// Assembly.  With H_xy = R V P, where (1 + s g_mu) = R P, P = [1, s e_mu], R = [1; s e_mu^dag] in 2x2 spin
+// blocks and V the link of the hop (or its adjoint), the term of the odd site k between even sites i, j is
+//   -1/4 H_ik A_k^-1 H_kj = -1/4 R_ik (V_ik M V_kj) P_kj,  M = P_ik A_k^-1 R_kj = A+ + (s e_i) A- (s' e_j^dag),
+// a 6x6 product spread over the 12x12 entries by signed permutations.  In a 2^4 block every site has one
+// neighbour per direction, so flipping coordinates mu and nu of i gives j: 4 odd sites for i = j, two for
+// each of the 6 other i ^ j that occur.  A thread takes one (i, i ^ j) and one 3x3 spin block of M.
+//
+// LU with partial pivoting on rows that stay where they are (a list of rows not yet used as pivots
+// replaces the swaps; their order's parity enters the sign), in panels of SNB columns: one thread per row
+// holds its panel entries in registers, then all warps update the remaining columns of the remaining
+// rows.  What bounds it: FP64 issue (GB300: one warp instruction per 20 clocks and SM), 0.36 ms per matrix
+// for the 8/3 n^3 flop, and the panels' chains of pivot searches and divisions.  Measured on the 4096
+// blocks of 16^4: 17.5 ms, against 40.1 ms for the LU in global memory plus 12.9 ms for assembling S_k's
+// columns with the block stencil on unit fields.
+constexpr int SN = 96, SNB = 8, S_NT = 256;
+constexpr size_t SMALL_SMEM = (size_t)(SN * SN + SNB * SN) * sizeof(double2);
+
+// e_mu as a signed permutation of the two spins: row sp has its entry ph in column sp ^ flip
+__device__ __forceinline__ double2 spin_phase(int mu, int sp)
+{
+    if (mu == 0) return make_double2(-1.0, 0.0);
+    if (mu == 1) return make_double2(0.0, -1.0);
+    if (mu == 2) return make_double2(sp == 0 ? -1.0 : 1.0, 0.0);
+    return make_double2(0.0, sp == 0 ? -1.0 : 1.0);
+}
+__device__ __forceinline__ int spin_flip(int mu) { return mu == 1 || mu == 2; }
+__device__ __forceinline__ double2 conj2(double2 a) { return make_double2(a.x, -a.y); }
+__device__ __forceinline__ void cmac2(double2 &acc, double2 a, double2 b)
+{
+    acc.x = fma(a.x, b.x, fma(-a.y, b.y, acc.x));
+    acc.y = fma(a.x, b.y, fma(a.y, b.x, acc.y));
+}
+__device__ __forceinline__ void cmsub2(double2 &acc, double2 a, double2 b)
+{
+    acc.x = fma(-a.x, b.x, fma(a.y, b.y, acc.x));
+    acc.y = fma(-a.x, b.y, fma(-a.y, b.x, acc.y));
+}
+
+// entry (i, j) of the Hermitian 6x6 block of chirality ch at site s (packed planes, see herm6_mul)
+__device__ __forceinline__ double2 herm_entry(const double2 *__restrict__ A, long V, long s, int ch, int i, int j)
+{
+    const double2 *b = A + (long)ch * 18 * V + s;
+    if (i == j) {
+        const double2 v = b[(long)(i >> 1) * V];
+        return make_double2((i & 1) ? v.y : v.x, 0.0);
+    }
+    const double2 v = b[(long)(3 + (i < j ? herm_off(i, j) : herm_off(j, i))) * V];
+    return i < j ? v : conj2(v);
+}
+
+// the 3x3 link of the hop into site x from its in-block neighbour y in direction mu: U_mu(x) forward
+// (y = x + mu), U_mu(y)^dag backward
+__device__ __forceinline__ void hop_link(const double2 *__restrict__ U, long V, int mu, bool fwd, long x, long y,
+                                         double2 (&L)[9])
+{
+    const double2 *b = U + (long)mu * 9 * V + (fwd ? x : y);
+#pragma unroll
+    for (int a = 0; a < 3; a++)
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            const double2 v = b[(long)(fwd ? a * 3 + c : c * 3 + a) * V];
+            L[a * 3 + c] = fwd ? v : conj2(v);
+        }
+}
+
+__global__ void __launch_bounds__(S_NT) k_small_logdet(const double2 *__restrict__ U64, const double2 *__restrict__ C64,
+                                                      const double2 *__restrict__ Ainv, long V, long vh, double mass4,
+                                                      double *lg_out, double *ang_out)
+{
+    extern __shared__ __align__(16) unsigned char small_smem[];
+    double2 *A = reinterpret_cast<double2 *>(small_smem);  // column-major: entry (i, j) at A[j SN + i]
+    double2 *U12 = A + SN * SN;                            // [SNB][SN]
+    __shared__ double2 piv[SN], prow[SNB];
+    __shared__ double bestv[3];
+    __shared__ int besti[3], order[SN], rows[SN];
+    __shared__ int nrows;
+    __shared__ double rlg[3], rang[3];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const long e0 = (long)blockIdx.x * 8, o0 = vh + e0;
+
+    for (int t = tid; t < SN * SN; t += S_NT) A[t] = make_double2(0.0, 0.0);
+    __syncthreads();
+    if (tid < 224) {
+        const int i = tid / 28, x = (tid / 4) % 7, sp = (tid >> 1) & 1, sq = tid & 1;
+        const int flip[4] = {4, 2, 1, 0};  // index of the neighbour in direction mu: index ^ flip[mu]
+        const int j = i ^ x;
+        const int ci[4] = {(i >> 2) & 1, (i >> 1) & 1, i & 1, ((i >> 2) + (i >> 1) + i) & 1};
+#pragma unroll 1
+        for (int mu = 0; mu < 4; mu++) {
+            int nu = -1;  // the direction from k to j
+            for (int d = 0; d < 4; d++)
+                if ((flip[mu] ^ flip[d]) == x) nu = d;
+            const int k = i ^ flip[mu];
+            if (nu >= 0) {
+                const bool fi = ci[mu] == 0;  // k = i + mu
+                const int ck = nu == 3 ? ((k >> 2) + (k >> 1) + k + 1) & 1 : (k >> (2 - nu)) & 1;
+                const bool fk = ck == 0;      // j = k + nu
+                const double s1 = fi ? -1.0 : 1.0, s2 = fk ? -1.0 : 1.0;
+                const double2 p1 = spin_phase(mu, sp), p2 = spin_phase(nu, sq);
+                const double2 ph = cmul2(make_double2(s1 * s2 * p1.x, s1 * s2 * p1.y), conj2(p2));
+                const int tp = sp ^ spin_flip(mu), tq = sq ^ spin_flip(nu);  // lower spins
+                double2 L[9], Q[9];
+                hop_link(U64, V, mu, fi, e0 + i, o0 + k, L);
+#pragma unroll
+                for (int q = 0; q < 9; q++) Q[q] = make_double2(0.0, 0.0);
+#pragma unroll
+                for (int a = 0; a < 3; a++)  // Q = L M
+#pragma unroll
+                    for (int b = 0; b < 3; b++) {
+                        double2 m = herm_entry(Ainv, V, o0 + k, 0, 3 * sp + a, 3 * sq + b);
+                        cmac2(m, ph, herm_entry(Ainv, V, o0 + k, 1, 3 * tp + a, 3 * tq + b));
+#pragma unroll
+                        for (int r = 0; r < 3; r++) cmac2(Q[r * 3 + b], L[r * 3 + a], m);
+                    }
+                hop_link(U64, V, nu, fk, o0 + k, e0 + j, L);
+                const double2 rl = make_double2(s1 * p1.x, -s1 * p1.y), cl = make_double2(s2 * p2.x, s2 * p2.y);
+#pragma unroll
+                for (int a = 0; a < 3; a++)
+#pragma unroll
+                    for (int b = 0; b < 3; b++) {
+                        double2 v = make_double2(0.0, 0.0);
+#pragma unroll
+                        for (int r = 0; r < 3; r++) cmac2(v, Q[a * 3 + r], L[r * 3 + b]);
+                        v = make_double2(-0.25 * v.x, -0.25 * v.y);
+                        const int iu = i * 12 + 3 * sp + a, il = i * 12 + 6 + 3 * tp + a;
+                        const int ju = j * 12 + 3 * sq + b, jl = j * 12 + 6 + 3 * tq + b;
+                        const double2 vc = cmul2(v, cl);
+                        double2 *d0 = A + ju * SN, *d1 = A + jl * SN;
+                        d0[iu] = make_double2(d0[iu].x + v.x, d0[iu].y + v.y);
+                        d1[iu] = make_double2(d1[iu].x + vc.x, d1[iu].y + vc.y);
+                        cmac2(d0[il], rl, v);
+                        cmac2(d1[il], rl, vc);
+                    }
+            }
+            // the four spin blocks of an (i, j) are lanes of one warp; the next direction maps the lower
+            // spins differently
+            __syncwarp();
+        }
+        if (x == 0) {  // A_ee = (4 + m) + C on the diagonal blocks: this thread's spin block of both chiralities
+            for (int ch = 0; ch < 2; ch++)
+                for (int a = 0; a < 3; a++)
+                    for (int b = 0; b < 3; b++) {
+                        double2 v = herm_entry(C64, V, e0 + i, ch, 3 * sp + a, 3 * sq + b);
+                        if (sp == sq && a == b) v.x += mass4;
+                        double2 *d = A + (i * 12 + 6 * ch + 3 * sq + b) * SN + i * 12 + 6 * ch + 3 * sp + a;
+                        *d = make_double2(d->x + v.x, d->y + v.y);
+                    }
+        }
+    }
+    bool used = false;  // of row tid (tid < SN)
+    __syncthreads();
+    for (int k0 = 0; k0 < SN; k0 += SNB) {
+        // ---- panel: one thread per row, its SNB entries in registers
+        if (tid < SN) {
+            double2 a[SNB];
+#pragma unroll
+            for (int q = 0; q < SNB; q++) a[q] = A[(k0 + q) * SN + tid];
+#pragma unroll
+            for (int kk = 0; kk < SNB; kk++) {
+                // the largest entry of the unused rows (a NaN counts as less than any number, a used row
+                // as less than that), ties to the lowest row
+                const double m = a[kk].x * a[kk].x + a[kk].y * a[kk].y;
+                double bv = used ? -2.0 : (m >= 0.0 ? m : -1.0);
+                int bi = tid;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    const double v2 = __shfl_xor_sync(0xffffffffu, bv, o);
+                    const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
+                    if (v2 > bv || (v2 == bv && i2 < bi)) bv = v2, bi = i2;
+                }
+                if (lane == 0) bestv[w] = bv, besti[w] = bi;
+                asm volatile("bar.sync 1, 96;" ::: "memory");
+                int p = besti[0];
+                bv = bestv[0];
+#pragma unroll
+                for (int q = 1; q < 3; q++)
+                    if (bestv[q] > bv) bv = bestv[q], p = besti[q];
+                if (tid == p) {
+#pragma unroll
+                    for (int q = 0; q < SNB; q++) prow[q] = a[q];
+                    piv[k0 + kk] = a[kk];
+                    order[k0 + kk] = p;
+                    used = true;
+                }
+                asm volatile("bar.sync 1, 96;" ::: "memory");
+                if (!used) {
+                    const double2 pv = prow[kk];
+                    const double id = 1.0 / (pv.x * pv.x + pv.y * pv.y);
+                    a[kk] = cmul2(a[kk], make_double2(pv.x * id, -pv.y * id));
+#pragma unroll
+                    for (int q = kk + 1; q < SNB; q++) cmsub2(a[q], a[kk], prow[q]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < SNB; q++) A[(k0 + q) * SN + tid] = a[q];
+            // the rows still to be eliminated, in order
+            const unsigned act = __ballot_sync(0xffffffffu, !used);
+            if (lane == 0) besti[w] = __popc(act);
+            asm volatile("bar.sync 1, 96;" ::: "memory");
+            int at = __popc(act & ((1u << lane) - 1));
+            for (int q = 0; q < w; q++) at += besti[q];
+            if (!used) rows[at] = tid;
+            if (tid == 0) nrows = besti[0] + besti[1] + besti[2];
+        }
+        __syncthreads();
+        const int j1 = k0 + SNB;
+        // ---- U12 = L11^-1 (pivot rows of the remaining columns), one thread per column
+        if (j1 + tid < SN) {
+            const int j = j1 + tid;
+            double2 u[SNB];
+#pragma unroll
+            for (int r = 0; r < SNB; r++) {
+                const int pr = order[k0 + r];
+                u[r] = A[j * SN + pr];
+#pragma unroll
+                for (int q = 0; q < r; q++) cmsub2(u[r], A[(k0 + q) * SN + pr], u[q]);
+                U12[r * SN + j] = u[r];
+            }
+        }
+        __syncthreads();
+        // ---- remaining rows -= L21 U12: lanes over rows, warps over columns
+        const int nr = nrows;
+        for (int rb = 0; rb < nr; rb += 32) {
+            const bool in = rb + lane < nr;
+            const int row = rows[in ? rb + lane : 0];
+            double2 l[SNB];
+#pragma unroll
+            for (int q = 0; q < SNB; q++) l[q] = A[(k0 + q) * SN + row];
+            for (int j = j1 + w; j < SN; j += S_NT / 32) {
+                double2 v = A[j * SN + row];
+#pragma unroll
+                for (int q = 0; q < SNB; q++) cmsub2(v, l[q], U12[q * SN + j]);
+                if (in) A[j * SN + row] = v;
+            }
+        }
+        __syncthreads();
+    }
+    // log |det| and phase: the pivots, and pi if the pivot rows' order is an odd permutation
+    if (tid < SN) {
+        const double2 pv = piv[tid];
+        double lg = 0.5 * log(pv.x * pv.x + pv.y * pv.y), ang = atan2(pv.y, pv.x);
+        int inv = 0;
+        for (int q = tid + 1; q < SN; q++) inv += order[q] < order[tid];
+        if (inv & 1) ang += M_PI;
+        for (int o = 16; o > 0; o >>= 1) {
+            lg += __shfl_down_sync(0xffffffffu, lg, o);
+            ang += __shfl_down_sync(0xffffffffu, ang, o);
+        }
+        if (lane == 0) rlg[w] = lg, rang[w] = ang;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        lg_out[blockIdx.x] = rlg[0] + rlg[1] + rlg[2];
+        ang_out[blockIdx.x] = rang[0] + rang[1] + rang[2];
+    }
+}
+
+static ddrw_status launch_small_logdet(ddrw_ctx *ctx, const MassInv *mi, double m, double *lg, double *ang)
+{
+    DDRW_CUDA_CHECK(cudaFuncSetAttribute(k_small_logdet, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMALL_SMEM));
+    ++ctx->launches;
+    k_small_logdet<<<ctx->nblk, S_NT, SMALL_SMEM, ctx->stream>>>(ctx->U64, ctx->C64, mi->A64, ctx->V, ctx->vh, 4.0 + m, lg,
+                                                                 ang);
+    DDRW_CUDA_CHECK(cudaGetLastError());
+    return DDRW_OK;
+}
+
 }  // namespace
 
 void cut_links(ddrw_ctx *ctx) { DISPATCH_L(ctx, k_cut_links, geom_dev(ctx), ctx->cut, ctx->U64, ctx->U32); }
 
-// log |det D_k(m)| and sign for all blocks (host vectors, library block numbering)
-static ddrw_status block_logdets(ddrw_ctx *ctx, double m, std::vector<double> &logdet, std::vector<double> &sign)
+// the Schur determinants of blocks whose matrices do not fit in shared memory (l = 4, 6): columns of S_k from
+// the FP64 block stencil, one CTA per matrix for the LU
+static ddrw_status dense_logdets(ddrw_ctx *ctx, const MassInv *mi, double m, double *dslg, double *dsang)
 {
-    if (ctx->l > 6) return set_error(ctx, DDRW_EINVAL, "block determinants need blocks of at most 6^4 sites");
-    ddrw_status st;
-    MassInv *mi;
-    if ((st = mass_inverse(ctx, m, &mi))) return st;
     const long V = ctx->V;
     const int vbh = ctx->l * ctx->l * ctx->l * ctx->l / 2, nblk = ctx->nblk;
     const int n = 12 * vbh;
     const size_t mat = (size_t)n * n * sizeof(double2);
-
-    // det A_oo per block
-    double *dlg, *dang;
-    if ((st = workspace(ctx, "bdet_site", sizeof(double) * 4 * nblk, (void **)&dlg))) return st;
-    dang = dlg + nblk;
-    double *dslg = dlg + 2 * nblk, *dsang = dlg + 3 * nblk;
-    ++ctx->launches;
-    k_site_logdet<<<nblk, SITE_NT, 0, ctx->stream>>>(ctx->C64, V, ctx->vh, vbh, 4.0 + m, dlg, dang);
-    DDRW_CUDA_CHECK(cudaGetLastError());
-
+    ddrw_status st;
     // batches of blocks whose matrices fit in a fraction of the free memory
     size_t fre = 0, tot = 0;
     DDRW_CUDA_CHECK(cudaMemGetInfo(&fre, &tot));
@@ -402,6 +663,30 @@ static ddrw_status block_logdets(ddrw_ctx *ctx, double m, std::vector<double> &l
         k_lu_logdet<<<nb, LU_NT, 0, ctx->stream>>>(n, S, dslg + k0, dsang + k0);
         DDRW_CUDA_CHECK(cudaGetLastError());
     }
+    return DDRW_OK;
+}
+
+// log |det D_k(m)| and sign for all blocks (host vectors, library block numbering)
+static ddrw_status block_logdets(ddrw_ctx *ctx, double m, std::vector<double> &logdet, std::vector<double> &sign)
+{
+    if (ctx->l > 6) return set_error(ctx, DDRW_EINVAL, "block determinants need blocks of at most 6^4 sites");
+    ddrw_status st;
+    MassInv *mi;
+    if ((st = mass_inverse(ctx, m, &mi))) return st;
+    const long V = ctx->V;
+    const int vbh = ctx->l * ctx->l * ctx->l * ctx->l / 2, nblk = ctx->nblk;
+    // det A_oo per block
+    double *dlg, *dang;
+    if ((st = workspace(ctx, "bdet_site", sizeof(double) * 4 * nblk, (void **)&dlg))) return st;
+    dang = dlg + nblk;
+    double *dslg = dlg + 2 * nblk, *dsang = dlg + 3 * nblk;
+    ++ctx->launches;
+    k_site_logdet<<<nblk, SITE_NT, 0, ctx->stream>>>(ctx->C64, V, ctx->vh, vbh, 4.0 + m, dlg, dang);
+    DDRW_CUDA_CHECK(cudaGetLastError());
+
+    if (ctx->l == 2) st = launch_small_logdet(ctx, mi, m, dslg, dsang);
+    else st = dense_logdets(ctx, mi, m, dslg, dsang);
+    if (st) return st;
     std::vector<double> h(4 * nblk);
     DDRW_CUDA_CHECK(cudaMemcpyAsync(h.data(), dlg, sizeof(double) * 4 * nblk, cudaMemcpyDeviceToHost, ctx->stream));
     DDRW_CUDA_CHECK(cudaStreamSynchronize(ctx->stream));
