@@ -100,73 +100,13 @@ __device__ __forceinline__ M3c load_link64(const double2 *U64, long V, int mu, l
     return r;
 }
 
-// chiral-basis gamma matrices (same convention as the operator): row a has one non-zero entry
-__device__ __forceinline__ void gamma_entry(int mu, int a, int *col, cpx<double> *val)
-{
-    // g0: [[0,-1],[-1,0]];  g_k: [[0, -i s_k], [i s_k, 0]] in 2x2 spin blocks
-    const int cols[4][4] = {{2, 3, 0, 1}, {3, 2, 1, 0}, {3, 2, 1, 0}, {2, 3, 0, 1}};
-    *col = cols[mu][a];
-    double re = 0, im = 0;
-    if (mu == 0) re = -1;
-    else if (mu == 1) im = (a < 2) ? -1 : 1;
-    else if (mu == 2) re = (a == 0 || a == 3) ? -1 : 1;
-    else im = (a == 0 || a == 3) ? -1 : 1;
-    *val = {re, im};
-}
-
-// (1 + s g_mu) psi, full 4-spin result
-__device__ __forceinline__ void one_pm_gamma(int mu, double s, const Spinor<double> &p, Spinor<double> &o)
+// K += a (x) b^dag for the colour vectors of one spin component
+__device__ __forceinline__ void outer_mac(M3c &K, const cpx<double> *a, const cpx<double> *b)
 {
 #pragma unroll
-    for (int a = 0; a < 4; a++) {
-        int b;
-        cpx<double> g;
-        gamma_entry(mu, a, &b, &g);
+    for (int i = 0; i < 3; i++)
 #pragma unroll
-        for (int c = 0; c < 3; c++) o.v[a][c] = p.v[a][c] + s * cmul(g, p.v[b][c]);
-    }
-}
-
-// sigma_{mu nu} = (i/2)[g_mu, g_nu] as a dense 4x4
-__device__ void sigma_matrix(int mu, int nu, cpx<double> S[4][4])
-{
-    cpx<double> G1[4][4], G2[4][4];
-    for (int a = 0; a < 4; a++)
-        for (int b = 0; b < 4; b++) G1[a][b] = G2[a][b] = {0.0, 0.0};
-    for (int a = 0; a < 4; a++) {
-        int b;
-        cpx<double> g;
-        gamma_entry(mu, a, &b, &g);
-        G1[a][b] = g;
-        gamma_entry(nu, a, &b, &g);
-        G2[a][b] = g;
-    }
-    for (int a = 0; a < 4; a++)
-        for (int b = 0; b < 4; b++) {
-            cpx<double> t = {0.0, 0.0};
-            for (int k = 0; k < 4; k++) t = t + cmul(G1[a][k], G2[k][b]) - cmul(G2[a][k], G1[k][b]);
-            S[a][b] = timesI(0.5 * t);
-        }
-}
-
-__device__ __forceinline__ void load_sp64(const double2 *f, long V, long s, Spinor<double> &p)
-{
-#pragma unroll
-    for (int k = 0; k < 12; k++) {
-        double2 v = f[(long)k * V + s];
-        p.v[k / 3][k % 3] = {v.x, v.y};
-    }
-}
-
-// K += c * (sum_spin a_spin (x) b_spin^dag)
-__device__ __forceinline__ void outer_acc(M3c &K, const Spinor<double> &a, const Spinor<double> &b, double c)
-{
-#pragma unroll
-    for (int sp = 0; sp < 4; sp++)
-#pragma unroll
-        for (int i = 0; i < 3; i++)
-#pragma unroll
-            for (int j = 0; j < 3; j++) K.m[i][j] = K.m[i][j] + c * cmulc(b.v[sp][j], a.v[sp][i]);
+        for (int j = 0; j < 3; j++) cmacc(K.m[i][j], b[j], a[i]);
 }
 
 struct ForceArgs {
@@ -176,40 +116,69 @@ struct ForceArgs {
     long rs;
     const double2 *U64;
     double2 *omega;  // [6 planes][9][V]
+    double *plaq;    // [6 planes][4 links of the loop][8][V]
     double csw;
     double *out;     // [V lexicographic][4][8]
 };
 
-// Omega_{mu nu}(x) = Lambda + Lambda^dag, Lambda = sum_rhs c sum_pairs sigma_{mu nu} R L^dag
-template <int BL>
-__global__ void k_omega(GeomDev g, ForceArgs a)
+// Omega_{mu nu}(x) = Lambda + Lambda^dag, Lambda = sum_rhs c sum_pairs sigma_{mu nu} R L^dag.  In the chiral
+// basis sigma_{0l} = diag(s_l, -s_l) and sigma_{jk} = -eps_{jkl} diag(s_l, s_l), so the six planes are
+// combinations of X_l = sum s_l R L^dag per chirality, l = 1..3: 36 colour outer products per pair of
+// spinors instead of a dense spin product and 4 outer products for each plane.  Bound by FP64
+// issue (about 5000 FP64 instructions per site at 8 right-hand sides).
+__global__ void __launch_bounds__(64) k_omega(long V, ForceArgs a)
 {
-    long s = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= g.V) return;
-    int pl = 0;
-    for (int mu = 0; mu < 4; mu++)
-        for (int nu = mu + 1; nu < 4; nu++, pl++) {
-            cpx<double> S[4][4];
-            sigma_matrix(mu, nu, S);
-            M3c Lam = m3_zero();
-            for (int r = 0; r < a.nrhs; r++) {
-                for (int pr = 0; pr < 2; pr++) {
-                    const double2 *L = (pr ? a.L2 : a.L1) + r * a.rs, *R = (pr ? a.R2 : a.R1) + r * a.rs;
-                    Spinor<double> lv, rv, sr;
-                    load_sp64(L, g.V, s, lv);
-                    load_sp64(R, g.V, s, rv);
-                    for (int al = 0; al < 4; al++)
-                        for (int c = 0; c < 3; c++) {
-                            cpx<double> t = {0.0, 0.0};
-                            for (int be = 0; be < 4; be++) t = t + cmul(S[al][be], rv.v[be][c]);
-                            sr.v[al][c] = t;
-                        }
-                    outer_acc(Lam, sr, lv, a.c[r]);
-                }
+    const long s = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= V) return;
+    M3c Lam[6];  // planes 01 02 03 12 13 23; the first chirality's X_l wait in the electric planes
+#pragma unroll 1
+    for (int ch = 0; ch < 2; ch++) {
+        M3c D = m3_zero(), T01 = m3_zero(), T10 = m3_zero();  // T_ab = sum c R_a L_b^dag, D = T00 - T11
+#pragma unroll 1
+        for (int r = 0; r < 2 * a.nrhs; r++) {
+            const int rr = r >> 1;
+            const double2 *L = ((r & 1) ? a.L2 : a.L1) + rr * a.rs + (long)6 * ch * V + s;
+            const double2 *R = ((r & 1) ? a.R2 : a.R1) + rr * a.rs + (long)6 * ch * V + s;
+            const double c = a.c[rr];
+            cpx<double> l[2][3], q[2][3];
+#pragma unroll
+            for (int k = 0; k < 6; k++) {
+                const double2 u = L[(long)k * V], v = R[(long)k * V];
+                l[k / 3][k % 3] = {u.x, u.y};
+                q[k / 3][k % 3] = {c * v.x, c * v.y};
             }
-            M3c Om = Lam;
-            m3_acc(Om, m3_dag(Lam), 1.0);
-            for (int k = 0; k < 9; k++) a.omega[((long)pl * 9 + k) * g.V + s] = make_double2(Om.m[k / 3][k % 3].re, Om.m[k / 3][k % 3].im);
+            outer_mac(D, q[0], l[0]);
+            outer_mac(T01, q[0], l[1]);
+            outer_mac(T10, q[1], l[0]);
+#pragma unroll
+            for (int k = 0; k < 3; k++) q[1][k] = -q[1][k];
+            outer_mac(D, q[1], l[1]);
+        }
+        // X_1 = T10 + T01, X_2 = -i T10 + i T01, X_3 = D
+#pragma unroll
+        for (int k = 0; k < 9; k++) {
+            const int i = k / 3, j = k % 3;
+            const cpx<double> x1 = T10.m[i][j] + T01.m[i][j], x2 = timesI(T01.m[i][j] - T10.m[i][j]), x3 = D.m[i][j];
+            if (ch == 0) {
+                Lam[0].m[i][j] = x1;
+                Lam[1].m[i][j] = x2;
+                Lam[2].m[i][j] = x3;
+            } else {
+                Lam[5].m[i][j] = -(Lam[0].m[i][j] + x1);
+                Lam[4].m[i][j] = Lam[1].m[i][j] + x2;
+                Lam[3].m[i][j] = -(Lam[2].m[i][j] + x3);
+                Lam[0].m[i][j] = Lam[0].m[i][j] - x1;
+                Lam[1].m[i][j] = Lam[1].m[i][j] - x2;
+                Lam[2].m[i][j] = Lam[2].m[i][j] - x3;
+            }
+        }
+    }
+#pragma unroll
+    for (int pl = 0; pl < 6; pl++)
+#pragma unroll
+        for (int k = 0; k < 9; k++) {
+            const cpx<double> u = Lam[pl].m[k / 3][k % 3], v = Lam[pl].m[k % 3][k / 3];
+            a.omega[((long)pl * 9 + k) * V + s] = make_double2(u.re + v.re, u.im - v.im);
         }
 }
 
@@ -218,121 +187,187 @@ __device__ __forceinline__ M3c load_omega(const double2 *om, long V, int pl, lon
     M3c r;
 #pragma unroll
     for (int k = 0; k < 9; k++) {
-        double2 v = om[((long)pl * 9 + k) * V + s];
+        double2 v = __ldg(om + ((long)pl * 9 + k) * V + s);
         r.m[k / 3][k % 3] = {v.x, v.y};
     }
     return r;
 }
 
-__device__ __forceinline__ int plane_index(int mu, int nu)  // mu < nu
+// Re tr(lambda_a M) (IM = false) or Im tr(lambda_a M), a = 1..8
+template <bool IM> __device__ __forceinline__ void gell_mann_traces(const M3c &M, double *o)
 {
-    const int idx[4][4] = {{-1, 0, 1, 2}, {-1, -1, 3, 4}, {-1, -1, -1, 5}, {-1, -1, -1, -1}};
-    return idx[mu][nu];
+    const double r3 = 0.57735026918962576;
+    auto p = [](cpx<double> z) { return IM ? z.im : z.re; };
+    auto pi = [](cpx<double> z) { return IM ? z.re : -z.im; };  // of i z
+#pragma unroll
+    for (int k = 0; k < 3; k++) {  // (i, j) = 01, 02, 12: lambda 1, 2; 4, 5; 6, 7
+        const int i = k < 2 ? 0 : 1, j = k == 0 ? 1 : 2, n = k == 0 ? 0 : k == 1 ? 3 : 5;
+        o[n] = p(M.m[i][j]) + p(M.m[j][i]);
+        o[n + 1] = pi(M.m[i][j]) - pi(M.m[j][i]);
+    }
+    o[2] = p(M.m[0][0]) - p(M.m[1][1]);
+    o[7] = r3 * (p(M.m[0][0]) + p(M.m[1][1]) - 2.0 * p(M.m[2][2]));
 }
 
+__device__ __forceinline__ long shifted(const int *x, const GeomDev &g, int mu, int dmu, int nu, int dnu, long (*index)(const GeomDev &, int, int, int, int))
+{
+    int c[4];
+#pragma unroll
+    for (int d = 0; d < 4; d++) {
+        int v = x[d] + (d == mu ? dmu : 0) + (d == nu ? dnu : 0);
+        c[d] = v < 0 ? v + g.L[d] : v >= g.L[d] ? v - g.L[d] : v;
+    }
+    return index(g, c[0], c[1], c[2], c[3]);
+}
+
+// The clover insertions of one plaquette loop W_0 W_1 W_2 W_3 = U_al(x) U_be(x+al) U_al(x+be)^dag U_be(x)^dag,
+// Omega O_j at the corner before W_j, for its four links at once: with G_j = O_j W_j + W_j O_{j+1} and
+// S_j = W_j W_{j+1},  E_k = G_{k+1} S_{k+2} + S_{k+1} G_{k+3}.  Thread row j forms G_j and S_j, shares
+// them through shared memory, and then does E_j and the link's eight traces: 6 matrix products per link,
+// against 10 when every link forms its six loops alone.  plaq[pl][j][a][x] = Im tr(lambda_a / 2 K).
 template <int BL>
-__device__ long site_shift(const GeomDev &g, const int *x, int mu, int dmu, int nu, int dnu)
+__global__ void __launch_bounds__(128) k_plaq(GeomDev g, ForceArgs a)
 {
-    int c[4] = {x[0], x[1], x[2], x[3]};
-    c[mu] = (c[mu] + dmu + g.L[mu]) % g.L[mu];
-    c[nu] = (c[nu] + dnu + g.L[nu]) % g.L[nu];
-    return internal_index<BL>(g, c[0], c[1], c[2], c[3]);
-}
-
-// E_k of a plaquette loop W0 W1 W2 W3 with Omega O_j at the corner before W_j (k: position of the link)
-__device__ M3c loop_env(const M3c *W, const M3c *O, int k)
-{
-    const M3c &A = W[(k + 1) & 3], &B = W[(k + 2) & 3], &C = W[(k + 3) & 3];
-    M3c AB = m3_mul(A, B), BC = m3_mul(B, C), ABC = m3_mul(AB, C);
-    M3c E = m3_mul(O[(k + 1) & 3], ABC);
-    m3_acc(E, m3_mul(m3_mul(A, O[(k + 2) & 3]), BC), 1.0);
-    m3_acc(E, m3_mul(m3_mul(AB, O[(k + 3) & 3]), C), 1.0);
-    m3_acc(E, m3_mul(ABC, O[k & 3]), 1.0);
-    return E;
-}
-
-// per link: K from the hopping bilinears and the clover insertions, then de_a = Im tr(T_a K)
-template <int BL>
-__global__ void k_force(GeomDev g, ForceArgs a, const double *lam /* 8 Gell-Mann matrices, [8][3][3][2] */)
-{
-    long s = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= g.V) return;
-    int mu = blockIdx.y;
+    __shared__ double2 sh[2][4][9][32];  // G, S
+    const int j = threadIdx.y, t = threadIdx.x;
+    const long s0 = (long)blockIdx.x * 32 + t;
+    const long s = s0 < g.V ? s0 : g.V - 1;  // (V is a multiple of 16: a last half warp repeats a site)
+    const int pl = blockIdx.y;
+    const int al = pl < 3 ? 0 : pl < 5 ? 1 : 2, be = pl < 3 ? pl + 1 : pl < 5 ? pl - 1 : 3;
     Site<BL> st;
     decode_site<BL>(s, g, st);
     const int *o = g.blk_org + st.blk * 4;
-    int x[4] = {o[0] + st.c[0], o[1] + st.c[1], o[2] + st.c[2], o[3] + st.c[3]};
+    const int x[4] = {o[0] + st.c[0], o[1] + st.c[1], o[2] + st.c[2], o[3] + st.c[3]};
+    // corner j and the next one, the site and direction of link j
+    const int j1 = (j + 1) & 3;
+    const long cj = shifted(x, g, al, j == 1 || j == 2, be, j >= 2, internal_index<BL>);
+    const long cn = shifted(x, g, al, j1 == 1 || j1 == 2, be, j1 >= 2, internal_index<BL>);
+    const int dir = (j & 1) ? be : al;
+    M3c W = load_link64(a.U64, g.V, dir, j < 2 ? cj : cn);
+    if (j >= 2) W = m3_dag(W);
+    {
+        M3c G = m3_mul(load_omega(a.omega, g.V, pl, cj), W);
+        m3_acc(G, m3_mul(W, load_omega(a.omega, g.V, pl, cn)), 1.0);
+#pragma unroll
+        for (int k = 0; k < 9; k++) {
+            sh[0][j][k][t] = make_double2(G.m[k / 3][k % 3].re, G.m[k / 3][k % 3].im);
+            sh[1][j][k][t] = make_double2(W.m[k / 3][k % 3].re, W.m[k / 3][k % 3].im);
+        }
+    }
+    auto get = [&](int f, int q) {
+        M3c r;
+#pragma unroll
+        for (int k = 0; k < 9; k++) {
+            const double2 v = sh[f][q & 3][k][t];
+            r.m[k / 3][k % 3] = {v.x, v.y};
+        }
+        return r;
+    };
+    __syncthreads();
+    const M3c S = m3_mul(W, get(1, j + 1));
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 9; k++) sh[1][j][k][t] = make_double2(S.m[k / 3][k % 3].re, S.m[k / 3][k % 3].im);
+    __syncthreads();
+    M3c E = m3_mul(get(0, j + 1), get(1, j + 2));
+    m3_acc(E, m3_mul(get(1, j + 1), get(0, j + 3)), 1.0);
+    // K = -f i U E (link held as U, j < 2) or +f i E U^dag (held as U^dag), f = csw / 8; Im tr(lambda/2 K)
+    const M3c T = j < 2 ? m3_mul(W, E) : m3_mul(E, W);
+    double tr[8];
+    gell_mann_traces<false>(T, tr);
+    const double f = 0.5 * a.csw / 8.0 * (j < 2 ? -1.0 : 1.0);
+    if (s0 < g.V)
+#pragma unroll
+        for (int k = 0; k < 8; k++) a.plaq[(((long)pl * 4 + j) * 8 + k) * g.V + s] = f * tr[k];
+}
+
+// h = (1 + sg g_mu) psi restricted to its two independent spin components, psi_u + sg e_mu psi_d
+__device__ __forceinline__ void load_projected(const double2 *f, long V, long s, int mu, double sg, cpx<double> (&h)[2][3])
+{
+    cpx<double> d[2][3];
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        const double2 u = f[(long)k * V + s], v = f[(long)(6 + k) * V + s];
+        h[k / 3][k % 3] = {u.x, u.y};
+        d[k / 3][k % 3] = {v.x, v.y};
+    }
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        cpx<double> e0, e1;  // e_mu psi_d
+        switch (mu) {
+        case 0: e0 = -d[0][c]; e1 = -d[1][c]; break;
+        case 1: e0 = timesMinusI(d[1][c]); e1 = timesMinusI(d[0][c]); break;
+        case 2: e0 = -d[1][c]; e1 = d[0][c]; break;
+        default: e0 = timesMinusI(d[0][c]); e1 = timesI(d[1][c]); break;
+        }
+        h[0][c] = {fma(sg, e0.re, h[0][c].re), fma(sg, e0.im, h[0][c].im)};
+        h[1][c] = {fma(sg, e1.re, h[1][c].re), fma(sg, e1.im, h[1][c].im)};
+    }
+}
+
+// per link: K from the hopping bilinears, de_a = Im tr(T_a K), plus the traces of the six plaquettes that
+// hold the link.  (1 -+ g_mu) = P^dag P with P psi the half spinor, so the spin sum of
+// [(1 - g) R] L^dag has two outer products of half spinors.
+template <int BL>
+__global__ void __launch_bounds__(64) k_force(GeomDev g, ForceArgs a)
+{
+    const long s = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= g.V) return;
+    const int mu = blockIdx.y;
+    Site<BL> st;
+    decode_site<BL>(s, g, st);
+    const int *o = g.blk_org + st.blk * 4;
+    const int x[4] = {o[0] + st.c[0], o[1] + st.c[1], o[2] + st.c[2], o[3] + st.c[3]};
     bool cross;
     int ph;
-    long sf = neighbour<BL>(st, mu, +1, g, &cross, &ph);
-    M3c U = load_link64(a.U64, g.V, mu, s);
-
-    // hopping: Y = sum c [(1-g)R(x+mu)] L(x)^dag, Z = sum c [(1+g)R(x)] L(x+mu)^dag
+    const long sf = neighbour<BL>(st, mu, +1, g, &cross, &ph);
+    // Y = sum c [(1-g)R(x+mu)] L(x)^dag, Z = sum c [(1+g)R(x)] L(x+mu)^dag
     M3c Y = m3_zero(), Z = m3_zero();
-    for (int r = 0; r < a.nrhs; r++)
-        for (int pr = 0; pr < 2; pr++) {
-            const double2 *L = (pr ? a.L2 : a.L1) + r * a.rs, *R = (pr ? a.R2 : a.R1) + r * a.rs;
-            Spinor<double> l0, l1, r0, r1, t;
-            load_sp64(L, g.V, s, l0);
-            load_sp64(L, g.V, sf, l1);
-            load_sp64(R, g.V, s, r0);
-            load_sp64(R, g.V, sf, r1);
-            one_pm_gamma(mu, -1.0, r1, t);
-            outer_acc(Y, t, l0, a.c[r] * ph);
-            one_pm_gamma(mu, +1.0, r0, t);
-            outer_acc(Z, t, l1, a.c[r] * ph);
+#pragma unroll 1
+    for (int r = 0; r < 2 * a.nrhs; r++) {
+        const int rr = r >> 1;
+        const double2 *L = ((r & 1) ? a.L2 : a.L1) + rr * a.rs, *R = ((r & 1) ? a.R2 : a.R1) + rr * a.rs;
+        const double c = a.c[rr] * ph;
+        cpx<double> l[2][3], q[2][3];
+        load_projected(R, g.V, sf, mu, -1.0, q);
+        load_projected(L, g.V, s, mu, -1.0, l);
+#pragma unroll
+        for (int sp = 0; sp < 2; sp++) {
+#pragma unroll
+            for (int k = 0; k < 3; k++) q[sp][k] = c * q[sp][k];
+            outer_mac(Y, q[sp], l[sp]);
         }
+        load_projected(R, g.V, s, mu, +1.0, q);
+        load_projected(L, g.V, sf, mu, +1.0, l);
+#pragma unroll
+        for (int sp = 0; sp < 2; sp++) {
+#pragma unroll
+            for (int k = 0; k < 3; k++) q[sp][k] = c * q[sp][k];
+            outer_mac(Z, q[sp], l[sp]);
+        }
+    }
+    const M3c U = load_link64(a.U64, g.V, mu, s);
     M3c K = m3_mul(U, Y);
     m3_acc(K, m3_mul(Z, m3_dag(U)), -1.0);
-
-    // clover: the six plaquettes that contain U_mu(x)
-    if (a.csw != 0.0) {
-        const double f = a.csw / 8.0;
+    double de[8];
+    gell_mann_traces<true>(K, de);
+#pragma unroll
+    for (int k = 0; k < 8; k++) de[k] *= 0.5;
+    if (a.csw != 0.0)
         for (int nu = 0; nu < 4; nu++) {
             if (nu == mu) continue;
-            int al = mu < nu ? mu : nu, be = mu < nu ? nu : mu;
-            int pl = plane_index(al, be);
-            for (int side = 0; side < 2; side++) {
-                // lower-left corner zc of the plaquette in the (al, be) plane holding the link
-                int zc[4] = {x[0], x[1], x[2], x[3]};
-                int k;  // position of the link in the loop
-                if (mu == al) {  // the link runs along the first direction: W0 (side 0) or W2^dag (side 1)
-                    if (side == 1) zc[be] = (zc[be] - 1 + g.L[be]) % g.L[be];
-                    k = side == 0 ? 0 : 2;
-                } else {          // along the second direction: W1 (side 0, corner x - al) or W3^dag (side 1, corner x)
-                    if (side == 0) zc[al] = (zc[al] - 1 + g.L[al]) % g.L[al];
-                    k = side == 0 ? 1 : 3;
-                }
-                long c0 = site_shift<BL>(g, zc, al, 0, be, 0), c1 = site_shift<BL>(g, zc, al, 1, be, 0);
-                long c2 = site_shift<BL>(g, zc, al, 1, be, 1), c3 = site_shift<BL>(g, zc, al, 0, be, 1);
-                M3c W[4], O[4];
-                W[0] = load_link64(a.U64, g.V, al, c0);
-                W[1] = load_link64(a.U64, g.V, be, c1);
-                W[2] = m3_dag(load_link64(a.U64, g.V, al, c3));
-                W[3] = m3_dag(load_link64(a.U64, g.V, be, c0));
-                O[0] = load_omega(a.omega, g.V, pl, c0);
-                O[1] = load_omega(a.omega, g.V, pl, c1);
-                O[2] = load_omega(a.omega, g.V, pl, c2);
-                O[3] = load_omega(a.omega, g.V, pl, c3);
-                M3c E = loop_env(W, O, k);
-                // K += -f i U E (link held as U) or +f i E U^dag (held as U^dag)
-                M3c T = (k < 2) ? m3_mul(U, E) : m3_mul(E, m3_dag(U));
-                double sg = (k < 2) ? -f : f;
-                for (int i = 0; i < 9; i++) K.m[i / 3][i % 3] = K.m[i / 3][i % 3] + sg * timesI(T.m[i / 3][i % 3]);
-            }
+            const int al = mu < nu ? mu : nu, be = mu < nu ? nu : mu;
+            const int pl = al == 0 ? be - 1 : al == 1 ? be + 1 : 5;
+            // link 0 of the loop at x and 2 of the one at x - nu (mu = al), 3 at x and 1 at x - nu (mu = be)
+            const long sn = shifted(x, g, nu, -1, mu, 0, internal_index<BL>);
+            const double *p0 = a.plaq + ((long)pl * 4 + (mu == al ? 0 : 3)) * 8 * g.V + s;
+            const double *p1 = a.plaq + ((long)pl * 4 + (mu == al ? 2 : 1)) * 8 * g.V + sn;
+#pragma unroll
+            for (int k = 0; k < 8; k++) de[k] += p0[(long)k * g.V] + p1[(long)k * g.V];
         }
-    }
-    // de_a = Im tr(T_a K), T_a = lambda_a / 2
-    long lx = (((long)x[0] * g.L[1] + x[1]) * g.L[2] + x[2]) * g.L[3] + x[3];
-    for (int aa = 0; aa < 8; aa++) {
-        cpx<double> tr = {0.0, 0.0};
-        for (int i = 0; i < 3; i++)
-            for (int j = 0; j < 3; j++) {
-                cpx<double> l = {0.5 * lam[((aa * 3 + i) * 3 + j) * 2], 0.5 * lam[((aa * 3 + i) * 3 + j) * 2 + 1]};
-                tr = tr + cmul(l, K.m[j][i]);
-            }
-        a.out[(lx * 4 + mu) * 8 + aa] = tr.im;
-    }
+    const long lx = (((long)x[0] * g.L[1] + x[1]) * g.L[2] + x[2]) * g.L[3] + x[3];
+#pragma unroll
+    for (int k = 0; k < 8; k++) a.out[(lx * 4 + mu) * 8 + k] = de[k];
 }
 
 // y = g5 x on every site (flip spins 2, 3)
@@ -381,36 +416,7 @@ void gamma5(ddrw_ctx *ctx, const double2 *x, double2 *y, int nrhs)
     k_gamma5<<<(unsigned)((n * nrhs + 255) / 256), 256, 0, ctx->stream>>>(n, ctx->V, nrhs, n, x, y);
 }
 
-void hop_between_rows64(ddrw_ctx *ctx, int rows, const double2 *in, double2 *out, int nrhs)
-{
-    DslashCall c;
-    c.in = in;
-    c.out = out;
-    c.rstride = 12 * ctx->V;
-    c.nrhs = nrhs;
-    c.beta = -0.5;
-    c.hopsel = 2;
-    c.par0 = 0;
-    c.npar = 2;
-    c.blk0 = rows == DDRW_BLACK ? 0 : ctx->nblk_c;
-    c.nblk = ctx->nblk_c;
-    dslash64(ctx, c);
-}
-
 }  // namespace
-
-static const double GELL_MANN[8][3][3][2] = {
-    {{{0, 0}, {1, 0}, {0, 0}}, {{1, 0}, {0, 0}, {0, 0}}, {{0, 0}, {0, 0}, {0, 0}}},
-    {{{0, 0}, {0, -1}, {0, 0}}, {{0, 1}, {0, 0}, {0, 0}}, {{0, 0}, {0, 0}, {0, 0}}},
-    {{{1, 0}, {0, 0}, {0, 0}}, {{0, 0}, {-1, 0}, {0, 0}}, {{0, 0}, {0, 0}, {0, 0}}},
-    {{{0, 0}, {0, 0}, {1, 0}}, {{0, 0}, {0, 0}, {0, 0}}, {{1, 0}, {0, 0}, {0, 0}}},
-    {{{0, 0}, {0, 0}, {0, -1}}, {{0, 0}, {0, 0}, {0, 0}}, {{0, 1}, {0, 0}, {0, 0}}},
-    {{{0, 0}, {0, 0}, {0, 0}}, {{0, 0}, {0, 0}, {1, 0}}, {{0, 0}, {1, 0}, {0, 0}}},
-    {{{0, 0}, {0, 0}, {0, 0}}, {{0, 0}, {0, 0}, {0, -1}}, {{0, 0}, {0, 1}, {0, 0}}},
-    {{{0.57735026918962576, 0}, {0, 0}, {0, 0}},
-     {{0, 0}, {0.57735026918962576, 0}, {0, 0}},
-     {{0, 0}, {0, 0}, {-1.1547005383792515, 0}}},
-};
 
 }  // namespace ddrw
 
@@ -427,7 +433,6 @@ extern "C" ddrw_status ddrw_force(ddrw_ctx *ctx, int nhit, uint64_t seed, uint64
     const long V = ctx->V, rs = 12 * V;
     const int R2 = 2 * nhit;
     const size_t f1 = sizeof(double2) * rs * nhit, f2 = sizeof(double2) * rs * R2;
-    const bool mixed = ctx->prec != DDRW_FP64;
     ddrw_status st;
     // fields: eta, delta (nhit) from the forward chain
     double2 *eta, *delta;
@@ -464,7 +469,7 @@ extern "C" ddrw_status ddrw_force(ddrw_ctx *ctx, int nhit, uint64_t seed, uint64
     if (st == DDRW_ENOCONV) conv = st;
     else if (st) return st;
     DDRW_CUDA_CHECK(cudaMemsetAsync(T1, 0, f1, ctx->stream));
-    hop_between_rows64(ctx, DDRW_BLACK, T2, T1, nhit);
+    hop_between64(ctx, DDRW_BLACK, T2, T1, nhit, -0.5);
     GeomDev g = geom_dev(ctx);
     {
         dim3 grid((unsigned)((V + 127) / 128), (unsigned)nhit);
@@ -479,10 +484,10 @@ extern "C" ddrw_status ddrw_force(ddrw_ctx *ctx, int nhit, uint64_t seed, uint64
         return DDRW_OK;
     };
     DDRW_CUDA_CHECK(cudaMemsetAsync(T1, 0, f2, ctx->stream));
-    hop_between_rows64(ctx, DDRW_WHITE, V2, T1, R2);  // E v
+    hop_between64(ctx, DDRW_WHITE, V2, T1, R2, -0.5);  // E v
     if ((st = bsolve(DDRW_WHITE, T1, A))) return st;  // a = W^-1 E v
     DDRW_CUDA_CHECK(cudaMemsetAsync(T1, 0, f2, ctx->stream));
-    hop_between_rows64(ctx, DDRW_BLACK, A, T1, R2);  // C a
+    hop_between64(ctx, DDRW_BLACK, A, T1, R2, -0.5);  // C a
     if ((st = bsolve(DDRW_BLACK, T1, Q))) return st;  // q = B^-1 C a
     // g5 z in both slots
     gamma5(ctx, Zf, T1, nhit);
@@ -490,7 +495,7 @@ extern "C" ddrw_status ddrw_force(ddrw_ctx *ctx, int nhit, uint64_t seed, uint64
     if ((st = bsolve(DDRW_BLACK, T1, T2))) return st;  // B^-1 g5 z
     gamma5(ctx, T2, ZT, R2);                            // zt = g5 B^-1 g5 z
     DDRW_CUDA_CHECK(cudaMemsetAsync(T1, 0, f2, ctx->stream));
-    hop_between_rows64(ctx, DDRW_WHITE, T2, T1, R2);  // E g5 zt
+    hop_between64(ctx, DDRW_WHITE, T2, T1, R2, -0.5);  // E g5 zt
     if ((st = bsolve(DDRW_WHITE, T1, T2))) return st;
     gamma5(ctx, T2, WT, R2);  // wt = g5 W^-1 E g5 zt
     // rho = q - a (into Q), sigma = a - v (into A)
@@ -504,12 +509,10 @@ extern "C" ddrw_status ddrw_force(ddrw_ctx *ctx, int nhit, uint64_t seed, uint64
         c[j] = w;
         c[nhit + j] = -w;
     }
-    double *cd, *lamd, *red;
-    if ((st = workspace(ctx, "frc_c", sizeof(double) * (R2 + 144 + 12 * R2), (void **)&cd))) return st;
-    lamd = cd + R2;
-    red = lamd + 144;
+    double *cd, *red;
+    if ((st = workspace(ctx, "frc_c", sizeof(double) * (R2 + 12 * R2), (void **)&cd))) return st;
+    red = cd + R2;
     DDRW_CUDA_CHECK(cudaMemcpyAsync(cd, c.data(), sizeof(double) * R2, cudaMemcpyHostToDevice, ctx->stream));
-    DDRW_CUDA_CHECK(cudaMemcpyAsync(lamd, GELL_MANN, sizeof(GELL_MANN), cudaMemcpyHostToDevice, ctx->stream));
 
     // de/dm2 = -2 Re[<zt_2, q_2> + <wt_2, a_2>] = -2 Re[<L1, rho> + <L2, sigma>] on the m2 slot
     if (dm2) {
@@ -523,21 +526,25 @@ extern "C" ddrw_status ddrw_force(ddrw_ctx *ctx, int nhit, uint64_t seed, uint64
     }
     if (dU) {
         double2 *omega;
+        double *plaq;
         if ((st = workspace(ctx, "frc_omega", sizeof(double2) * 54 * V, (void **)&omega))) return st;
+        if ((st = workspace(ctx, "frc_plaq", sizeof(double) * 192 * V, (void **)&plaq))) return st;
         double *out;
         void *dout;
         bool host;
         size_t ob = sizeof(double) * 32 * V;
         if ((st = stage_out(ctx, dU, ob, "stage_force", &dout, &host))) return st;
         out = (double *)dout;
-        ForceArgs fa{ZT, Q, WT, A, cd, R2, rs, ctx->U64, omega, ctx->csw, out};
-        {
-            dim3 grid((unsigned)((V + 63) / 64));
-            DISPATCH_BL(ctx, k_omega, grid, 64, g, fa);
+        ForceArgs fa{ZT, Q, WT, A, cd, R2, rs, ctx->U64, omega, plaq, ctx->csw, out};
+        if (ctx->csw != 0.0) {
+            ++ctx->launches;
+            k_omega<<<(unsigned)((V + 63) / 64), 64, 0, ctx->stream>>>(V, fa);
+            dim3 grid((unsigned)((V + 31) / 32), 6u);
+            DISPATCH_BL(ctx, k_plaq, grid, dim3(32, 4), g, fa);
         }
         {
             dim3 grid((unsigned)((V + 63) / 64), 4u);
-            DISPATCH_BL(ctx, k_force, grid, 64, g, fa, lamd);
+            DISPATCH_BL(ctx, k_force, grid, 64, g, fa);
         }
         if ((st = finish_out(ctx, dU, out, ob, host))) return st;
     }
