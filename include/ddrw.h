@@ -137,8 +137,8 @@ ddrw_status ddrw_set_max_rhs(ddrw_ctx *ctx, int max_rhs);
  * gives each block and right-hand side to a cluster of CTAs: form 0 the widest CTAs (one of 128
  * threads for 4^4 blocks, three of 224 for 6^4, four of 512 for 8^4), form 1 or 2 the smallest (four of
  * 32, six of 128, eight of 256: more CTAs where a small lattice has few blocks; 2^4 blocks have one
- * shape).  -1 (the default): the first launch of each shape times both on its real arguments and
- * keeps the faster.  Same results in every form to the solver's tolerance.  DDRW_EINVAL outside -1..2. */
+ * shape), form 2 in FP64 with 4^4 blocks eight threads per site (four CTAs of 256).  -1 (the
+ * default): the first launch of each shape times them on its real arguments and keeps the fastest.  Same results in every form to the solver's tolerance.  DDRW_EINVAL outside -1..2. */
 ddrw_status ddrw_block_config(ddrw_ctx *ctx, int form);
 
 /* The 16-bit storage precisions (DDRW_MIXED_FP16, DDRW_MIXED_BF16).  reliable_updates != 0 (the

@@ -249,7 +249,7 @@ template <int MODE>
 __global__ void __launch_bounds__(NT) k_bicg_fin(const double *part, long nwt, KScal *sc)
 {
     constexpr int K = MODE == 1 ? 2 : RED_PARTS;
-    __shared__ double sm[NT / 32][K];
+    __shared__ double sm[NT / 32][K], tot[K];
     const int r = blockIdx.x;
     if (!sc[r].active) return;
     RunSum<double> v[K];
@@ -258,11 +258,13 @@ __global__ void __launch_bounds__(NT) k_bicg_fin(const double *part, long nwt, K
 #pragma unroll
         for (int k = 0; k < K; k++) v[k].add(pp[k]);
     }
-    cta_sum_run<K, NT, double>(v, sm);
+    cta_sum_run<K, NT, double>(v, sm, tot);
+    if (threadIdx.x >= 32) return;
+    __syncwarp();
     if (threadIdx.x != 0) return;
     double val[K];
 #pragma unroll
-    for (int k = 0; k < K; k++) val[k] = v[k].value();
+    for (int k = 0; k < K; k++) val[k] = tot[k];
     KScal &s = sc[r];
     if constexpr (MODE == 1) {  // alpha = rho / (rh, v)
         const double den = val[0] * val[0] + val[1] * val[1];
@@ -418,7 +420,10 @@ static unsigned grid_for(long n, int nch, int nrhs)
 {
     const long units = std::max(1L, (n + NT - 1) / NT) * nch;
     const long most = std::min(608L, std::max(1L, (1216L + nrhs - 1) / nrhs));
-    const long per = (units + most - 1) / most;
+    long per = (units + most - 1) / most;
+    // FP64 fields (12 chunks): two units per CTA once every SM has work, the sums of a warp cost as much
+    // FP64 time as a unit
+    if (nch == 12) per = std::max(per, std::min(2L, units * nrhs / 152));
     return (unsigned)((units + per - 1) / per);
 }
 

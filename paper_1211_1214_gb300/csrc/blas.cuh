@@ -38,13 +38,6 @@ template <class P> struct Blas {
 // ----------------------------------------------------------------------------- reductions
 // (deterministic grid-wide sums shared by the vector kernels of blas.cu and sap.cu)
 
-__device__ __forceinline__ double warp_sum(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-
 // A running sum: FP64 for FP64 fields; for FP32 arithmetic an unevaluated pair hi + lo (Knuth's
 // two-sum, about 48 significant bits against the 24 of the terms).  GB300 adds FP64 at 1/64 of its FP32
 // rate: with FP64 shuffle steps in every warp and FP64 sums over the warps, the reductions took longer
@@ -89,23 +82,70 @@ template <> struct RunSum<float> {
     }
 };
 
-// CTA totals of v[0..K) in thread 0 (the caller's other threads may go on; sm is reused only after a barrier)
+// Warp totals of K running sums at once: while several sums are left, each exchange step also halves the
+// sums a lane keeps, so K = 7 takes 9 additions per lane instead of 35 (FP64 additions are what these
+// reductions wait for).  Afterwards lane l holds the total of sum l >> SHIFT.
+template <int K, typename R> struct WarpSums {
+    static constexpr int M = K <= 1 ? 1 : K <= 2 ? 2 : K <= 4 ? 4 : 8;
+    static constexpr int SHIFT = M == 1 ? 5 : M == 2 ? 4 : M == 4 ? 3 : 2;
+    __device__ static __forceinline__ typename RunSum<R>::Raw xchg(typename RunSum<R>::Raw a, int o)
+    {
+        if constexpr (sizeof(R) == 8) {
+            return __shfl_xor_sync(0xffffffffu, a, o);
+        } else {
+            a.x = __shfl_xor_sync(0xffffffffu, a.x, o);
+            a.y = __shfl_xor_sync(0xffffffffu, a.y, o);
+            return a;
+        }
+    }
+    __device__ static __forceinline__ RunSum<R> total(const RunSum<R> (&v)[K])
+    {
+        RunSum<R> t[M];
+#pragma unroll
+        for (int k = 0; k < K; k++) t[k] = v[k];
+#pragma unroll
+        for (int o = 16, m = M; o > 0; o >>= 1) {
+            if (m > 1) {
+                m >>= 1;
+                const bool up = (threadIdx.x & o) != 0;
+#pragma unroll
+                for (int k = 0; k < M / 2; k++)
+                    if (k < m) {
+                        const RunSum<R> keep = up ? t[k + m] : t[k], send = up ? t[k] : t[k + m];
+                        t[k] = keep;
+                        t[k].join(xchg(send.raw(), o));
+                    }
+            } else {
+                t[0].join(xchg(t[0].raw(), o));
+            }
+        }
+        return t[0];
+    }
+};
+
+// CTA totals of v[0..K): sum k in out[k] (shared memory), complete after the caller's next __syncwarp of
+// warp 0 (whose lanes write it) or a barrier; sm and out are used again only after a barrier
 template <int K, int NT, typename R>
-__device__ __forceinline__ void cta_sum_run(RunSum<R> (&v)[K], typename RunSum<R>::Raw (*sm)[K])
+__device__ __forceinline__ void cta_sum_run(RunSum<R> (&v)[K], typename RunSum<R>::Raw (*sm)[K],
+                                            typename RunSum<R>::Raw (&out)[K])
 {
+    using WS = WarpSums<K, R>;
+    constexpr int NW = NT / 32;
+    static_assert(NW == 8, "eight warps");
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < K; k++) v[k].template shuffle_sum<32>();
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < K; k++) sm[w][k] = v[k].raw();
+    const RunSum<R> t = WS::total(v);
+    const int k = lane >> WS::SHIFT;
+    if ((lane & ((1 << WS::SHIFT) - 1)) == 0 && k < K) sm[w][k] = t.raw();
     __syncthreads();
     if (w == 0)
 #pragma unroll
-        for (int k = 0; k < K; k++) {
-            v[k] = RunSum<R>();
-            if (lane < NT / 32) v[k].join(sm[lane][k]);
-            v[k].template shuffle_sum<NT / 32>();
+        for (int k0 = 0; k0 < K; k0 += 4) {  // four sums at a time, eight lanes each
+            const int kk = k0 + (lane >> 3);
+            RunSum<R> q;
+            if (kk < K) q.join(sm[lane & 7][kk]);
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) q.join(WS::xchg(q.raw(), o));
+            if ((lane & 7) == 0 && kk < K) out[kk] = q.raw();
         }
 }
 
@@ -116,17 +156,20 @@ template <int K, int NT, typename R>
 __device__ bool grid_sum_run(RunSum<R> (&v)[K], double (&out)[K], double *part, unsigned *ticket)
 {
     using Raw = typename RunSum<R>::Raw;
-    __shared__ Raw sm[NT / 32][K];
+    __shared__ Raw sm[NT / 32][K], tot[K];
     __shared__ bool last;
     const int r = blockIdx.y, G = gridDim.x;
     Raw *pp = reinterpret_cast<Raw *>(part) + (long)r * G * K;
-    cta_sum_run<K, NT, R>(v, sm);
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < K; k++) pp[(long)blockIdx.x * K + k] = v[k].raw();
+    cta_sum_run<K, NT, R>(v, sm, tot);
+    if (threadIdx.x < 32) {
+        __syncwarp();
+        if (threadIdx.x < K) pp[(long)blockIdx.x * K + threadIdx.x] = tot[threadIdx.x];
         __threadfence();
-        unsigned t = atomicAdd(ticket + r, 1u);
-        last = (t == (unsigned)(G - 1));
+        __syncwarp();
+        if (threadIdx.x == 0) {
+            unsigned t = atomicAdd(ticket + r, 1u);
+            last = (t == (unsigned)(G - 1));
+        }
     }
     __syncthreads();
     if (!last) return false;
@@ -136,14 +179,19 @@ __device__ bool grid_sum_run(RunSum<R> (&v)[K], double (&out)[K], double *part, 
     for (int i = threadIdx.x; i < G; i += NT)
 #pragma unroll
         for (int k = 0; k < K; k++) v[k].join(__ldcg(pp + (long)i * K + k));
-    cta_sum_run<K, NT, R>(v, sm);
-    if (threadIdx.x == 0) {
+    cta_sum_run<K, NT, R>(v, sm, tot);
+    if (threadIdx.x >= 32) return false;
+    __syncwarp();
+    if (threadIdx.x != 0) return false;
+    RunSum<R> q;
 #pragma unroll
-        for (int k = 0; k < K; k++) out[k] = v[k].value();
-        ticket[r] = 0;
-        return true;
+    for (int k = 0; k < K; k++) {
+        q = RunSum<R>();
+        q.join(tot[k]);
+        out[k] = q.value();
     }
-    return false;
+    ticket[r] = 0;
+    return true;
 }
 
 // the same from per-thread FP64 values, in place

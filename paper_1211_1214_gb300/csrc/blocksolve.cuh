@@ -7,6 +7,7 @@
 #include "blas.cuh"
 #include "ctx.h"
 #include "lowprec.cuh"
+#include "split64.cuh"
 #include "stencil.cuh"
 
 namespace ddrw {
@@ -104,12 +105,21 @@ __device__ __forceinline__ void cluster_totals(RunSum<R> (&v)[K], double (&out)[
     using Raw = typename RunSum<R>::Raw;
     constexpr int NW = NT / 32, W2 = NW <= 1 ? 1 : NW <= 2 ? 2 : NW <= 4 ? 4 : NW <= 8 ? 8 : 16;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < K; k++) v[k].template shuffle_sum<32>();
-    if (NW > 1) {
+    using WS = WarpSums<K, R>;
+    {
+        const RunSum<R> t = WS::total(v);
+        const int k = lane >> WS::SHIFT;
+        if ((lane & ((1 << WS::SHIFT) - 1)) == 0 && k < K) red.warp[w][k] = t.raw();
+    }
+    if (NW == 1) {
+        __syncwarp();
         if (lane == 0)
 #pragma unroll
-            for (int k = 0; k < K; k++) red.warp[w][k] = v[k].raw();
+            for (int k = 0; k < K; k++) {
+                v[k] = RunSum<R>();
+                v[k].join(red.warp[0][k]);
+            }
+    } else {
         __syncthreads();
         if (w == 0)
 #pragma unroll
@@ -439,6 +449,281 @@ __global__ void __launch_bounds__(NT, sizeof(typename P::R) == 4 ? 512 / NT : 1)
     blk_sync<C>();  // no CTA leaves while another may read its part
 }
 
+// ---- FP64, eight lanes per site (split64.cuh), for 2^4 and 4^4 blocks.  With one thread per site a warp's
+// chain of FP64 instructions takes 180 us per iteration, whether it has an SM to itself (8 blocks of 4^4
+// sites and 4 right-hand sides: 128 CTAs of one warp) or shares it with three others; a 2^4 block fills
+// 8 of a warp's 32 lanes.  Here lane u does hop u, then its share of spin u & 3; the Krylov vectors stay in
+// registers for the whole solve (lane (al, q) owns colours 0, 1 of spin al for q = 0, colour 2 for q = 1).
+// ms per launch of a colour, one thread per site / split: 8^4 in 4^4 blocks, 4 right-hand sides 3.47 / 1.42,
+// 16 right-hand sides 3.64 / 5.58, 16^4, 4 right-hand sides 13.1 / 20.5 (the tuner chooses).
+template <int BL, int C> struct SplitShape {
+    static constexpr int HL = BlockShape<BL>::VBH / C, NT = 8 * HL;
+    static constexpr size_t SMEM = (size_t)HL * (2 * 12 + 48) * sizeof(double2);  // G, T, the half spinors
+};
+
+template <int BL, int C>
+__global__ void __launch_bounds__(SplitShape<BL, C>::NT) k_block_split(GeomDev g, BlkArgs<PrecD> a)
+{
+    constexpr int VBH = BlockShape<BL>::VBH, HL = SplitShape<BL, C>::HL, NT = SplitShape<BL, C>::NT;
+    static_assert(HL % 4 == 0 && BL % C == 0, "whole warps, whole time slices per CTA");
+    extern __shared__ __align__(16) unsigned char blk_smem[];
+    __shared__ BlkRed<double, C, NT> red;
+    __shared__ double scal[6], fs[5];
+    __shared__ int live;
+    double2 *G = reinterpret_cast<double2 *>(blk_smem), *T = G + 12 * HL;  // [site][12]
+    const int q = C == 1 ? 0 : (int)(blockIdx.x % C), id = C == 1 ? (int)blockIdx.x : (int)(blockIdx.x / C);
+    const int rhs = id % a.nrhs, blk = a.blk0 + id / a.nrhs;
+    const long ro = (long)rhs * a.rstride, V = g.V;
+    const int slot = rhs / a.rpm;
+    const double mass4 = a.mass4[slot];
+    const double2 *Ainv = a.Ainv[slot];
+
+    const int u = threadIdx.x & 7, al = u & 3, hf = u >> 2, hl = threadIdx.x >> 3, h = q * HL + hl;
+    double2 *w = T + 12 * HL + hl * 48;  // [hop][6]
+    const long be = (long)blk * VBH, bo = g.vh + be, se = be + h, so = bo + h;
+    const int mu = u >> 1;
+    const bool fwd = (u & 1) == 0;
+    // coordinate and half-index step of this lane's hop, for each parity of the output site
+    int zr = h / (BL / 2);
+    const int z0 = 2 * (h - zr * (BL / 2)), cy = zr % BL, cx = (zr / BL) % BL, ct = zr / (BL * BL);
+    const int odd_row = (ct + cx + cy) & 1;
+
+    // this lane's hop into the site of parity par, gathered from F, then its share of the hop sum
+    auto hops = [&](int par, const double2 *F, cpx<double> (&o)[3]) {
+        const int cz = z0 + (odd_row ^ par), cm = mu == 0 ? ct : mu == 1 ? cx : mu == 2 ? cy : cz;
+        const int step = mu == 0 ? BL * BL * BL : mu == 1 ? BL * BL : mu == 2 ? BL : 1;
+        Half<double> hw;
+        if (fwd ? cm < BL - 1 : cm > 0) {
+            const int hn = (2 * h + (cz & 1) + (fwd ? step : -step)) >> 1;
+            const long s = par ? so : se, sn = (par ? be : bo) + hn;
+            const int own = hn - q * HL;
+            const double2 *src = F + 12 * own;
+            if (C > 1 && (own < 0 || own >= HL)) {
+                const int q2 = own < 0 ? q - 1 : q + 1;
+                src = cooperative_groups::this_cluster().map_shared_rank(F, q2) + 12 * (hn - q2 * HL);
+            }
+            split_hop(src, 1, a.U + (long)mu * 9 * V + (fwd ? s : sn), V, mu, fwd, hw);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 6; k++) hw.v[k / 3][k % 3] = {0.0, 0.0};
+        }
+#pragma unroll
+        for (int k = 0; k < 6; k++) w[u * 6 + k] = make_double2(hw.v[k / 3][k % 3].re, hw.v[k / 3][k % 3].im);
+        __syncwarp();
+        split_sum(w, al, hf, o);
+        __syncwarp();
+    };
+    // the two components a lane owns (the second is zero for hf = 1), and back to shared memory
+    const int k0 = 3 * al + 2 * hf;
+    auto own2 = [&](const cpx<double> (&o)[3], cpx<double> (&e)[2]) {
+        e[0] = hf ? o[2] : o[0];
+        e[1] = hf ? cpx<double>{0.0, 0.0} : o[1];
+    };
+    auto put = [&](double2 *F, const cpx<double> (&e)[2]) {
+        F[12 * hl + k0] = make_double2(e[0].re, e[0].im);
+        if (!hf) F[12 * hl + k0 + 1] = make_double2(e[1].re, e[1].im);
+    };
+    auto put_global = [&](double2 *f, long s, const cpx<double> (&e)[2]) {
+        f[(long)k0 * V + s] = make_double2(e[0].re, e[0].im);
+        if (!hf) f[(long)(k0 + 1) * V + s] = make_double2(e[1].re, e[1].im);
+    };
+    auto add_b = [&](long s, cpx<double> (&o)[3]) {  // by one lane of a spin, before the halves join
+        if (hf == 0)
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                const double2 t = __ldg(a.b + ro + (long)(3 * al + c) * V + s);
+                o[c].re += t.x;
+                o[c].im += t.y;
+            }
+    };
+
+    double &rho_x = fs[0], &rho_y = fs[1], &al_x = fs[2], &al_y = fs[3], &thresh = fs[4];
+    int it = 0, buf = 0;
+    bool ok = false;
+    cpx<double> x[2] = {{0.0, 0.0}, {0.0, 0.0}}, r[2], rh[2], p[2], v[2], s[2];
+    enum { START, V_OF_P, T_OF_S, FINISH };
+    int stage = START;
+    while (true) {
+        cpx<double> o[3] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}}, f3[3], e[2];
+        // ---- odd site:  T = A_oo^-1 ( y + coef H_oe G )
+        if (stage != START) hops(1, G, o);
+        if (stage == FINISH)
+#pragma unroll
+            for (int c = 0; c < 3; c++) o[c] = 0.5 * o[c];
+        if (stage == START || stage == FINISH) add_b(so, o);
+        split_join(o);
+        split_fetch(o, al, hf, f3);
+        split_herm(Ainv + so, V, al, hf, 0.0, f3, o);
+        split_join(o);
+        own2(o, e);
+        if (stage == FINISH) {
+            put_global(a.x + ro, so, e);
+            break;
+        }
+        put(T, e);
+        blk_sync<C>();
+        // ---- even site
+        hops(0, T, o);
+        const double coef = stage == START ? 0.5 : -0.25;
+#pragma unroll
+        for (int c = 0; c < 3; c++) o[c] = coef * o[c];
+        if (stage == START) {
+            add_b(se, o);
+        } else {
+            cpx<double> d[3];
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                const double2 t = G[12 * hl + 3 * ((al & 2) + hf) + c];
+                f3[c] = {t.x, t.y};
+            }
+            split_herm(a.Cl + se, V, al, hf, mass4, f3, d);
+#pragma unroll
+            for (int c = 0; c < 3; c++) o[c] = o[c] + d[c];
+        }
+        split_join(o);
+        own2(o, e);
+        if (stage == V_OF_P) {
+            RunSum<double> d[2];
+            cpx<double> z = {0.0, 0.0};
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                v[k] = e[k];
+                cmacc(z, rh[k], v[k]);
+            }
+            d[0].s = z.re;
+            d[1].s = z.im;
+            double t[2];
+            cluster_totals<2, NT, C, double>(d, t, red, buf, q);
+            if (threadIdx.x == 0) {  // alpha = rho / (rh, v); a zero or NaN is a breakdown: x as it is
+                const double den = t[0] * t[0] + t[1] * t[1];
+                live = !(den == 0.0 || !(den == den));
+                const double iv = 1.0 / den;
+                scal[0] = al_x = (rho_x * t[0] + rho_y * t[1]) * iv;
+                scal[1] = al_y = (rho_y * t[0] - rho_x * t[1]) * iv;
+            }
+            __syncthreads();
+            if (!live) {
+                put(G, x);
+                stage = FINISH;
+            } else {  // s = r - alpha v
+                const cpx<double> alp = {scal[0], scal[1]};
+#pragma unroll
+                for (int k = 0; k < 2; k++) {
+                    s[k] = r[k];
+                    cmsub(s[k], alp, v[k]);
+                }
+                put(G, s);
+                stage = T_OF_S;
+            }
+            blk_sync<C>();
+            continue;
+        }
+        RunSum<double> rr[2];  // ||r||^2 and, at the start, ||b||^2
+        if (stage == START) {
+            double n = 0, nb = 0;
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                r[k] = rh[k] = p[k] = e[k];
+                n = fma(e[k].re, e[k].re, fma(e[k].im, e[k].im, n));
+                if (k == 0 || !hf) {
+                    const double2 t0 = __ldg(a.b + ro + (long)(k0 + k) * V + se), t1 = __ldg(a.b + ro + (long)(k0 + k) * V + so);
+                    nb = fma(t0.x, t0.x, fma(t0.y, t0.y, fma(t1.x, t1.x, fma(t1.y, t1.y, nb))));
+                }
+            }
+            rr[0].s = n;
+            rr[1].s = nb;
+            put(G, p);
+        } else {
+            RunSum<double> d[7];
+            cpx<double> ts = {0.0, 0.0}, hs = {0.0, 0.0}, ht = {0.0, 0.0};
+            double tt = 0;
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                cmacc(ts, e[k], s[k]);
+                tt = fma(e[k].re, e[k].re, fma(e[k].im, e[k].im, tt));
+                cmacc(hs, rh[k], s[k]);
+                cmacc(ht, rh[k], e[k]);
+            }
+            d[0].s = ts.re;
+            d[1].s = ts.im;
+            d[2].s = tt;
+            d[3].s = hs.re;
+            d[4].s = hs.im;
+            d[5].s = ht.re;
+            d[6].s = ht.im;
+            double t[7];
+            cluster_totals<7, NT, C, double>(d, t, red, buf, q);
+            if (threadIdx.x == 0) {  // as in k_block_solve
+                const double n2 = t[2];
+                const bool go = !(n2 == 0.0 || !(n2 == n2));
+                live = go;
+                const double iv = go ? 1.0 / n2 : 0.0;
+                const double ox = t[0] * iv, oy = t[1] * iv;
+                const double rx = t[3] - (ox * t[5] - oy * t[6]), ry = t[4] - (ox * t[6] + oy * t[5]);
+                const double nx = rx * al_x - ry * al_y, ny = rx * al_y + ry * al_x;
+                const double dx = rho_x * ox - rho_y * oy, dy = rho_x * oy + rho_y * ox;
+                const double d2 = dx * dx + dy * dy, jv = d2 > 0.0 ? 1.0 / d2 : 0.0;
+                scal[2] = ox;
+                scal[3] = oy;
+                scal[4] = (nx * dx + ny * dy) * jv;
+                scal[5] = (ny * dx - nx * dy) * jv;
+                rho_x = d2 > 0.0 ? rx : 0.0;
+                rho_y = d2 > 0.0 ? ry : 0.0;
+            }
+            __syncthreads();
+            if (!live) {
+                put(G, x);
+                stage = FINISH;
+                blk_sync<C>();
+                continue;
+            }
+            // x += alpha p + omega s ; r = s - omega t ; p = r + beta (p - omega v)
+            const cpx<double> alp = {scal[0], scal[1]}, om = {scal[2], scal[3]}, bt = {scal[4], scal[5]};
+            double n = 0;
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                cmac(x[k], alp, p[k]);
+                cmac(x[k], om, s[k]);
+                r[k] = s[k];
+                cmsub(r[k], om, e[k]);
+                n = fma(r[k].re, r[k].re, fma(r[k].im, r[k].im, n));
+                cmsub(p[k], om, v[k]);
+                cpx<double> pn = r[k];
+                cmac(pn, bt, p[k]);
+                p[k] = pn;
+            }
+            put(G, p);
+            rr[0].s = n;
+            it++;
+        }
+        double t[2];
+        cluster_totals<2, NT, C, double>(rr, t, red, buf, q);
+        if (threadIdx.x == 0) {
+            if (stage == START) {
+                thresh = (a.tol2_dev ? *a.tol2_dev : a.tol2) * t[1];
+                rho_x = t[0];
+                rho_y = 0.0;
+            }
+            ok = t[0] <= thresh;
+            const bool dead = !(t[0] == t[0]) || it >= a.maxiter || (rho_x == 0.0 && rho_y == 0.0);
+            live = !ok && !dead;
+        }
+        __syncthreads();
+        stage = V_OF_P;
+        if (!live) {
+            put(G, x);
+            stage = FINISH;
+            blk_sync<C>();
+        }
+    }
+    put_global(a.x + ro, se, x);
+    if (threadIdx.x == 0 && q == 0) {
+        atomicMax(a.stat, it);
+        if (!ok) atomicAdd(a.stat + 1, 1);
+    }
+    blk_sync<C>();  // no CTA leaves while another may read its part
+}
+
 // Launch shapes: C CTAs of NT threads per block and right-hand side.  Form 0 is the wider CTA, form 1 the
 // smaller one (more CTAs for few blocks and right-hand sides, more distributed-memory hops).
 // Measured on FP32 storage, ms per launch of a colour, form 0 / form 1 / the kernel with its vectors in
@@ -454,14 +739,14 @@ template <> struct BlkForms<4> { static constexpr int C[2] = {1, 4}, N[2] = {128
 template <> struct BlkForms<6> { static constexpr int C[2] = {3, 6}, N[2] = {224, 128}; };
 template <> struct BlkForms<8> { static constexpr int C[2] = {4, 8}, N[2] = {512, 256}; };
 
-template <class P, int BL, int C, int NT>
-void launch_block_shape(ddrw_ctx *ctx, const BlkArgs<P> &a, int nrhs)
+template <class P>
+void launch_clusters(ddrw_ctx *ctx, void (*kernel)(GeomDev, BlkArgs<P>), int C, int NT, size_t smem, const BlkArgs<P> &a,
+                     int nrhs)
 {
     BlkArgs<P> b = a;
     b.nrhs = nrhs;
-    constexpr size_t smem = BlkShape<P, BL, C>::SMEM;
     if (smem > 40 * 1024)  // (static shared memory counts towards the default limit of 48 KB)
-        cudaFuncSetAttribute(k_block_solve<P, BL, C, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute((const void *)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)((long)C * nrhs * ctx->nblk_c));
     lc.blockDim = dim3(NT);
@@ -475,7 +760,13 @@ void launch_block_shape(ddrw_ctx *ctx, const BlkArgs<P> &a, int nrhs)
     lc.attrs = at;
     lc.numAttrs = C > 1 ? 1 : 0;
     ++ctx->launches;
-    cudaLaunchKernelEx(&lc, k_block_solve<P, BL, C, NT>, geom_dev(ctx), b);
+    cudaLaunchKernelEx(&lc, kernel, geom_dev(ctx), b);
+}
+
+template <class P, int BL, int C, int NT>
+void launch_block_shape(ddrw_ctx *ctx, const BlkArgs<P> &a, int nrhs)
+{
+    launch_clusters<P>(ctx, k_block_solve<P, BL, C, NT>, C, NT, BlkShape<P, BL, C>::SMEM, a, nrhs);
 }
 
 // The first launch of each (storage, block length, right-hand sides) shape times the forms on the real
@@ -485,11 +776,23 @@ template <class P, int BL>
 void launch_block_kernel(ddrw_ctx *ctx, const BlkArgs<P> &a, int nrhs)
 {
     using F = BlkForms<BL>;
-    constexpr int NF = BL == 2 ? 1 : 2;
+    // FP64 solves of 4^4 blocks have the split kernel as a third form, those of 2^4 blocks as the only one
+    constexpr bool SPLIT = P::ID == 64 && BL == 4;
+    constexpr int NF = BL == 2 ? 1 : SPLIT ? 3 : 2;
     const int kind = P::ID == 64 ? PROF_BLOCK64 : P::ID == 32 ? PROF_BLOCK32 : PROF_BLOCK16;
     auto run = [&](int form) {
-        if (NF > 1 && form) launch_block_shape<P, BL, F::C[1], F::N[1]>(ctx, a, nrhs);
-        else launch_block_shape<P, BL, F::C[0], F::N[0]>(ctx, a, nrhs);
+        if constexpr (P::ID == 64 && BL == 2) {
+            launch_clusters<P>(ctx, k_block_split<2, 1>, 1, SplitShape<2, 1>::NT, SplitShape<2, 1>::SMEM, a, nrhs);
+        } else {
+            if constexpr (SPLIT) {
+                if (form == 2) {
+                    launch_clusters<P>(ctx, k_block_split<4, 4>, 4, SplitShape<4, 4>::NT, SplitShape<4, 4>::SMEM, a, nrhs);
+                    return;
+                }
+            }
+            if (NF > 1 && form) launch_block_shape<P, BL, F::C[1], F::N[1]>(ctx, a, nrhs);
+            else launch_block_shape<P, BL, F::C[0], F::N[0]>(ctx, a, nrhs);
+        }
     };
     int form = 0;
     if (NF > 1) {

@@ -335,6 +335,8 @@ struct DslashCall {
     double *red_part = nullptr;
 };
 void dslash64(ddrw_ctx *ctx, const DslashCall &c);
+// out = D(m) in for nrhs fields in the boundary layout (16-byte aligned, in and out apart)
+void apply_D_lex64(ddrw_ctx *ctx, double m, const double2 *in, double2 *out, int nrhs);
 // out (rows of colour `rows`) += beta H_{rows <- other colour} in: the hops between blocks in FP64,
 // one launch per direction over the face sites (hops.cu); other rows untouched
 void hop_between64(ddrw_ctx *ctx, int rows, const double2 *in, double2 *out, int nrhs, double beta);

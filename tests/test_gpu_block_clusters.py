@@ -1,5 +1,5 @@
 """The persistent block solver in its cluster shapes: every block length and storage, an odd number of
-right-hand sides, both launch shapes, against the oracle's block operator.
+right-hand sides, every launch shape (in FP64 also the one with eight lanes per site), against the oracle's block operator.
 
 The bar is the solver's own target: the true residual of every right-hand side over the colour, by
 the oracle's FP64 operator, at most tol_block (the defect correction stops there).
@@ -31,7 +31,7 @@ def test_block_solver_cluster_shapes(dims, l):
         tol = 1e-13 if prec == binding.FP64 else 1e-12
         ctx.set_solver(prec, tol_outer=1e-10, tol_block=tol)
         ctx.set_low_precision(True, low16)
-        for form in (0, 1):
+        for form in (0, 1, 2):
             ctx.block_config(form)
             for colour in (0, 1):
                 x = np.zeros_like(b)
