@@ -160,10 +160,25 @@ GeomDev geom_dev(const ddrw_ctx *ctx)
     return g;
 }
 
+// the inverse in every storage precision, into the entry's arrays
+static void fill_inverse(ddrw_ctx *ctx, MassInv &mi)
+{
+    build_inverse(ctx, mi.m, mi);
+    f32_to_low(ctx, mi.A32, mi.A16, 18L * ctx->V, false);
+    f32_to_low(ctx, mi.A32, mi.Ab16, 18L * ctx->V, true);
+    mi.stale = false;
+}
+
 ddrw_status mass_inverse(ddrw_ctx *ctx, double m, MassInv **out)
 {
     for (auto &mi : ctx->inv)
         if (mi.m == m) {
+            if (mi.stale) {
+                if (ctx->devctl) return set_error(ctx, DDRW_ESTATE, "in-block inverse to be rebuilt during capture");
+                fill_inverse(ctx, mi);
+                DDRW_CUDA_CHECK(cudaGetLastError());
+            }
+            mi.used = true;
             *out = &mi;
             return DDRW_OK;
         }
@@ -180,10 +195,9 @@ ddrw_status mass_inverse(ddrw_ctx *ctx, double m, MassInv **out)
         cudaFree(mi.Ab16);
         return set_cuda_error(ctx, e, "cudaMalloc(in-block inverse)", __FILE__, __LINE__);
     }
-    build_inverse(ctx, m, mi);
-    f32_to_low(ctx, mi.A32, mi.A16, 18L * ctx->V, false);
-    f32_to_low(ctx, mi.A32, mi.Ab16, 18L * ctx->V, true);
+    fill_inverse(ctx, mi);
     DDRW_CUDA_CHECK(cudaGetLastError());
+    mi.used = true;
     ctx->inv.push_back(mi);
     *out = &ctx->inv.back();
     return DDRW_OK;
@@ -667,15 +681,15 @@ static ddrw_status rebuild(ddrw_ctx *ctx)
     // graphs, which hold their addresses, stay valid; a long list of masses is dropped instead
     if (ctx->inv.size() > (size_t)MAXM + 2) free_inverses(ctx);
     for (auto &mi : ctx->inv) {
-        build_inverse(ctx, mi.m, mi);
-        f32_to_low(ctx, mi.A32, mi.A16, 18L * ctx->V, false);
-        f32_to_low(ctx, mi.A32, mi.Ab16, 18L * ctx->V, true);
+        if (mi.used || mi.m == ctx->m1 || mi.m == ctx->m2) fill_inverse(ctx, mi);
+        else mi.stale = true;
     }
     MassInv *mi;
     ddrw_status st = mass_inverse(ctx, ctx->m1, &mi);
     if (st) return st;
     if (ctx->m2 != ctx->m1) st = mass_inverse(ctx, ctx->m2, &mi);
     if (st) return st;
+    for (auto &e : ctx->inv) e.used = false;  // (the context's masses are kept up to date by their values)
     st = sync(ctx);
     ctx->built = st == DDRW_OK;
     return st;
