@@ -87,7 +87,8 @@ __device__ __forceinline__ void hop_shared(const int (&c)[4], int lb, int s, int
     }
     Half<R> h, w;
     project<MU, -DIR>(p, h);
-    if (DIR > 0) link_mul(L, h, w);
+    if constexpr (sizeof(R) == 4) link_mul_packed<(DIR < 0)>(L, h, w);
+    else if (DIR > 0) link_mul(L, h, w);
     else link_dag_mul(L, h, w);
     reconstruct_add<MU, -DIR>(acc, w);
 }

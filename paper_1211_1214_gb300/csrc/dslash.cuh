@@ -223,7 +223,8 @@ constexpr size_t STAGED_SMEM_MAX = (size_t)62 * 128 * 16;
 
 // ROLL selects the hop code form: 0 unrolled, 1 rolled, 2 / 3 batched loads of 4 / 8 hops,
 // 4 / 5 unrolled compiled for at least 3 / 2 CTAs of 256 threads per SM (<= 85 / 128 registers),
-// 6 / 7 as 5 / 4 with the neighbours read from the neighbour table instead of computed,
+// 6 / 7 as 5 / 4 with the neighbours read from the neighbour table instead of computed (6: in 32- and
+// 16-bit storage with the loads of each hop issued before its arithmetic),
 // 11 fully rolled (one body for the eight hops; double-single storage only)
 // RED != 0 adds the inner products of the output to the epilogue (red 1: conj(w) out; red 2:
 // conj(out) x, |out|^2, conj(w) x and conj(w) out), one partial per warp of 32 sites, summed in FP64 by k_bicg_fin; the
@@ -265,11 +266,12 @@ __global__ void __launch_bounds__(256, (ROLL == 4 || ROLL == 7) ? 3 : (ROLL == 5
             static_assert(NR == 1, "the fully rolled form takes one right-hand side per thread");
             hop_fully_rolled<P, BL, HOPSEL>(g, st, (int)s, in, a.U, acc[0]);
         } else if constexpr (ROLL == 6 || ROLL == 7) {
-            hop_tab<P, HOPSEL, 0, NR>(g, n0.x, n0.y, (int)s, in, a.rstride, a.U, acc);
-            hop_tab<P, HOPSEL, 1, NR>(g, n0.z, n0.w, (int)s, in, a.rstride, a.U, acc);
+            constexpr bool FIRST = ROLL == 6 && P::ID < 64;
+            hop_tab<P, HOPSEL, 0, NR, FIRST>(g, n0.x, n0.y, (int)s, in, a.rstride, a.U, acc);
+            hop_tab<P, HOPSEL, 1, NR, FIRST>(g, n0.z, n0.w, (int)s, in, a.rstride, a.U, acc);
             const int4 n1 = g.nbr[g.V + s];  // loaded here: fewer registers live over the first hops
-            hop_tab<P, HOPSEL, 2, NR>(g, n1.x, n1.y, (int)s, in, a.rstride, a.U, acc);
-            hop_tab<P, HOPSEL, 3, NR>(g, n1.z, n1.w, (int)s, in, a.rstride, a.U, acc);
+            hop_tab<P, HOPSEL, 2, NR, FIRST>(g, n1.x, n1.y, (int)s, in, a.rstride, a.U, acc);
+            hop_tab<P, HOPSEL, 3, NR, FIRST>(g, n1.z, n1.w, (int)s, in, a.rstride, a.U, acc);
         } else if constexpr (ROLL == 1) {
             hop_multi_rolled<P, BL, HOPSEL, NR>(g, st, (int)s, in, a.rstride, a.U, acc);
         } else {
