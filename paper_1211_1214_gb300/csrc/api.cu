@@ -1,6 +1,7 @@
 // api.cu -- the C ABI (include/ddrw.h): context, geometry tables, parameters, operator
 // applications.  Solvers and the estimate live in solver.cu and estimate.cu.
 #include <chrono>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 
@@ -292,6 +293,9 @@ ddrw_status residual_stencil(ddrw_ctx *ctx, DslashCall c, bool ds)
     // the stencil reads `in` at the hop neighbours and `x` at the site; both are the same field here
     if (c.x && c.x != c.in) return set_error(ctx, DDRW_EINVAL, "double-single residual needs x == in");
     if (c.hopsel == 2) return set_error(ctx, DDRW_EINVAL, "double-single residual of a hop between blocks");
+    int ex;
+    if (std::fabs(std::frexp(c.alpha, &ex)) != 0.5 || std::fabs(std::frexp(c.beta, &ex)) != 0.5 || c.post)
+        return set_error(ctx, DDRW_EINVAL, "double-single residual with a factor that is no power of two");
     float4 *xs;
     ddrw_status st = workspace(ctx, "ds_split", sizeof(float4) * (size_t)c.rstride * c.nrhs, (void **)&xs);
     if (st) return st;

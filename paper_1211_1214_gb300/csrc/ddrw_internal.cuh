@@ -323,6 +323,18 @@ __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
     return r;
 }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
 template <bool DAG> __device__ __forceinline__ void link_mul_packed(const Link<float> &U, const Half<float> &h, Half<float> &w)
 {
     f32x2 hr[3], hi[3];

@@ -229,8 +229,15 @@ constexpr size_t STAGED_SMEM_MAX = (size_t)62 * 128 * 16;
 // RED != 0 adds the inner products of the output to the epilogue (red 1: conj(w) out; red 2:
 // conj(out) x, |out|^2, conj(w) x and conj(w) out), one partial per warp of 32 sites, summed in FP64 by k_bicg_fin; the
 // launcher only fuses launches whose output sites fill whole CTAs (no thread leaves early)
+// launch bounds by form (CTAs of 256 threads; the double-single rolled form: 128, three per SM)
+template <class P, int ROLL> constexpr int ds_threads() { return std::is_same<P, PrecDD>::value && ROLL == 11 ? 128 : 256; }
+template <class P, int ROLL> constexpr int ds_ctas()
+{
+    return std::is_same<P, PrecDD>::value ? (ROLL == 11 ? 3 : 1) : (ROLL == 4 || ROLL == 7) ? 3 : (ROLL == 5 || ROLL == 6) ? 2 : 1;
+}
+
 template <class P, int BL, int HOPSEL, int NR, int ROLL = 0, int RED = 0>
-__global__ void __launch_bounds__(256, (ROLL == 4 || ROLL == 7) ? 3 : (ROLL == 5 || ROLL == 6) ? 2 : 1)
+__global__ void __launch_bounds__(ds_threads<P, ROLL>(), ds_ctas<P, ROLL>())
     k_dslash(GeomDev g, DsArgs<P> a)
 {
     using R = typename P::R;
@@ -280,8 +287,13 @@ __global__ void __launch_bounds__(256, (ROLL == 4 || ROLL == 7) ? 3 : (ROLL == 5
             hop_dir_multi<P, BL, HOPSEL, 2, NR>(g, st, s, in, a.rstride, a.U, acc);
             hop_dir_multi<P, BL, HOPSEL, 3, NR>(g, st, s, in, a.rstride, a.U, acc);
         }
+        if constexpr (std::is_same<P, PrecDD>::value) {
 #pragma unroll
-        for (int r = 0; r < NR; r++) scale(acc[r], a.beta);
+            for (int k = 0; k < 12; k++) acc[0].v[k / 3][k % 3] = times_pow2(a.beta.hi, acc[0].v[k / 3][k % 3]);
+        } else {
+#pragma unroll
+            for (int r = 0; r < NR; r++) scale(acc[r], a.beta);
+        }
     }
     if constexpr (std::is_same<P, PrecDD>::value) {
         // double-single: one chirality body run twice (the clover multiply in FP32 pairs is large,
@@ -302,11 +314,11 @@ __global__ void __launch_bounds__(256, (ROLL == 4 || ROLL == 7) ? 3 : (ROLL == 5
                 }
                 if (ch == 0) {
 #pragma unroll
-                    for (int k = 0; k < 6; k++) acc[0].v[k / 3][k % 3] = acc[0].v[k / 3][k % 3] + a.alpha * o6[k];
+                    for (int k = 0; k < 6; k++) acc[0].v[k / 3][k % 3] = acc[0].v[k / 3][k % 3] + times_pow2(a.alpha.hi, o6[k]);
                 } else {
 #pragma unroll
                     for (int k = 0; k < 6; k++)
-                        acc[0].v[2 + k / 3][k % 3] = acc[0].v[2 + k / 3][k % 3] + a.alpha * o6[k];
+                        acc[0].v[2 + k / 3][k % 3] = acc[0].v[2 + k / 3][k % 3] + times_pow2(a.alpha.hi, o6[k]);
                 }
             }
         }
@@ -589,6 +601,7 @@ void launch_cfg(ddrw_ctx *ctx, const DslashCall &c, const DsArgs<P> &a, DsConfig
     // has half the code of the unrolled one, which is instruction-fetch bound)
     if (std::is_same<P, PrecDD>::value)
         cfg.nr = 1, cfg.nw = 1, cfg.roll = ((cfg.roll == 1 || cfg.roll == 11) && c.hopsel != 2) ? cfg.roll : 0;
+    if (std::is_same<P, PrecDD>::value && cfg.roll == 11 && cfg.nt > 128) cfg.nt = 128;
     if (!std::is_same<P, PrecDD>::value && c.hopsel == 1 && (cfg.nr != 1 || (cfg.roll != 0 && cfg.roll != 5 && cfg.roll != 6)))
         cfg.nr = 1, cfg.nw = 1, cfg.roll = 0;
     if (c.hopsel == 1 && cfg.roll == 6 && !g.nbr) cfg.roll = 5;

@@ -12,7 +12,7 @@ extern template void launch_bl<PrecDD, 8>(ddrw_ctx *, const DslashCall &);
 
 void dslash_ds(ddrw_ctx *ctx, const DslashCall &c) { launch<PrecDD>(ctx, c); }
 
-// one complex FP64 number (x, y) per element -> (hi(x), lo(x), hi(y), lo(y)).  The elements are
+// one complex FP64 number (x, y) per element -> (hi(x), hi(y), lo(x), lo(y)).  The elements are
 // those of the sites [off, off + len) of parities par0 .. par0 + npar - 1 in the 12 planes of nrhs
 // fields (planes V apart, parities vh apart, fields rs apart).
 // grid: x over the sites, y over (plane, parity), z over the fields -- no per-element division
@@ -25,7 +25,7 @@ __global__ void k_split(long V, long vh, long off, long len, int par0, int npar,
     const long idx = (long)blockIdx.z * rs + (long)k * V + (long)(par0 + p) * vh + off + j;
     double2 v = in[idx];
     float xh = (float)v.x, yh = (float)v.y;
-    out[idx] = make_float4(xh, (float)(v.x - (double)xh), yh, (float)(v.y - (double)yh));
+    out[idx] = make_float4(xh, yh, (float)(v.x - (double)xh), (float)(v.y - (double)yh));
 }
 
 void split64(ddrw_ctx *ctx, const double2 *in, float4 *out, long V, long vh, long off, long len, int par0, int npar,
