@@ -284,30 +284,86 @@ long host_internal_index(const ddrw_ctx *ctx, const std::vector<int> &blk_index,
     return (long)p * ctx->vh + (long)blk_index[B] * vbh + (lb >> 1);
 }
 
-ddrw_status residual_stencil(ddrw_ctx *ctx, DslashCall c, bool ds)
+ddrw_status split_copy(ddrw_ctx *ctx, long rs, int nrhs, float4 **xs)
 {
-    if (!ds) {
-        dslash64(ctx, c);
-        return DDRW_OK;
-    }
+    return workspace(ctx, "ds_split", sizeof(float4) * (size_t)rs * nrhs, (void **)xs);
+}
+
+ddrw_status residual_stencil(ddrw_ctx *ctx, DslashCall c, const float4 *xs)
+{
     // the stencil reads `in` at the hop neighbours and `x` at the site; both are the same field here
     if (c.x && c.x != c.in) return set_error(ctx, DDRW_EINVAL, "double-single residual needs x == in");
     if (c.hopsel == 2) return set_error(ctx, DDRW_EINVAL, "double-single residual of a hop between blocks");
     int ex;
     if (std::fabs(std::frexp(c.alpha, &ex)) != 0.5 || std::fabs(std::frexp(c.beta, &ex)) != 0.5 || c.post)
         return set_error(ctx, DDRW_EINVAL, "double-single residual with a factor that is no power of two");
-    float4 *xs;
-    ddrw_status st = workspace(ctx, "ds_split", sizeof(float4) * (size_t)c.rstride * c.nrhs, (void **)&xs);
-    if (st) return st;
-    // only the sites the stencil reads: its own blocks (hops inside blocks) or every site
-    long vbh = (long)ctx->l * ctx->l * ctx->l * ctx->l / 2;
-    if (c.hopsel == 1)
-        split64(ctx, (const double2 *)c.in, xs, ctx->V, ctx->vh, c.blk0 * vbh, c.nblk * vbh, 0, 2, c.nrhs, c.rstride);
-    else
-        split64(ctx, (const double2 *)c.in, xs, ctx->V, ctx->vh, 0, ctx->vh, 0, 2, c.nrhs, c.rstride);
+    if (!xs) {
+        float4 *buf;
+        ddrw_status st = split_copy(ctx, c.rstride, c.nrhs, &buf);
+        if (st) return st;
+        // only the sites the stencil reads: its own blocks (hops inside blocks) or every site
+        long vbh = (long)ctx->l * ctx->l * ctx->l * ctx->l / 2;
+        if (c.hopsel == 1)
+            split64(ctx, (const double2 *)c.in, buf, ctx->V, ctx->vh, c.blk0 * vbh, c.nblk * vbh, 0, 2, c.nrhs, c.rstride);
+        else
+            split64(ctx, (const double2 *)c.in, buf, ctx->V, ctx->vh, 0, ctx->vh, 0, 2, c.nrhs, c.rstride);
+        xs = buf;
+    }
     c.in = xs;
     c.x = xs;
     dslash_ds(ctx, c);
+    return DDRW_OK;
+}
+
+// out[r] = the sum over the parities of in[p * nrhs + r]
+__global__ void k_add_norms(const double *in, int npar, int nrhs, double *out)
+{
+    for (int r = threadIdx.x; r < nrhs; r += blockDim.x) out[r] = npar == 2 ? in[r] + in[nrhs + r] : in[r];
+}
+
+// out[r] = the sum of n partial sums, in a fixed order (one CTA per right-hand side)
+__global__ void __launch_bounds__(256) k_sum_parts(const double *part, long n, double *out)
+{
+    __shared__ double sm[8][1], tot[1];
+    RunSum<double> v[1];
+    for (long i = threadIdx.x; i < n; i += 256) v[0].add(part[(long)blockIdx.x * n + i]);
+    cta_sum_run<1, 256, double>(v, sm, tot);
+    __syncthreads();
+    if (threadIdx.x == 0) out[blockIdx.x] = tot[0];
+}
+
+ddrw_status residual_norms(ddrw_ctx *ctx, DslashCall c, const double2 *b, double *norms, bool ds, const float4 *xs)
+{
+    const long vbh = (long)ctx->l * ctx->l * ctx->l * ctx->l / 2, per = c.nblk * vbh;
+    ddrw_status st;
+    if (ds) {
+        const long nw = per * c.npar / 32;  // at most V / 32: the Krylov loops' partial sums have room for RED_PARTS V / 64
+        double *part;
+        if ((st = workspace(ctx, "eo_redpart", sizeof(double) * RED_PARTS * (size_t)(ctx->vh / 32) * c.nrhs, (void **)&part)))
+            return st;
+        c.rb = b;
+        c.norm_part = part;
+        if ((st = residual_stencil(ctx, c, xs))) return st;
+        ++ctx->launches;
+        k_sum_parts<<<c.nrhs, 256, 0, ctx->stream>>>(part, nw, norms);
+        return DDRW_OK;
+    }
+    dslash64(ctx, c);
+    double2 *out = (double2 *)c.out;
+    if (c.npar == 2 && per == ctx->vh) {
+        const VecRange all{ctx->V, 0, ctx->V, c.rstride, c.nrhs};
+        Blas<PrecD>::axpby(ctx, all, 1.0, b, 1.0, out);
+        return Blas<PrecD>::norm2(ctx, all, out, norms);
+    }
+    double *two;
+    if ((st = workspace(ctx, "res_norms", sizeof(double) * 2 * c.nrhs, (void **)&two))) return st;
+    for (int p = 0; p < c.npar; p++) {
+        const VecRange vr{ctx->V, (c.par0 + p) * ctx->vh + c.blk0 * vbh, per, c.rstride, c.nrhs};
+        Blas<PrecD>::axpby(ctx, vr, 1.0, b, 1.0, out);
+        if ((st = Blas<PrecD>::norm2(ctx, vr, out, two + p * c.nrhs))) return st;
+    }
+    ++ctx->launches;
+    k_add_norms<<<1, 64, 0, ctx->stream>>>(two, c.npar, c.nrhs, norms);
     return DDRW_OK;
 }
 
@@ -947,7 +1003,7 @@ ddrw_status ddrw_apply_D_ds(ddrw_ctx *ctx, double m, const double *in, double *o
     c.npar = 2;
     c.blk0 = 0;
     c.nblk = ctx->nblk;
-    if ((st = residual_stencil(ctx, c, true))) return st;
+    if ((st = residual_stencil(ctx, c))) return st;
     unpack_spinor64(ctx, fout, (double *)dout, nrhs);
     if ((st = finish_out(ctx, out, dout, ubytes, host_out))) return st;
     return sync(ctx);

@@ -381,23 +381,30 @@ __global__ void __launch_bounds__(NT) k_to_low(long V, long off, long n, long rs
     });
 }
 
-// x64 += scale[r] * e (e in storage precision P)
-template <class P>
+// x64 += scale[r] * e (e in storage precision P), or x64 = scale[r] * e (FIRST); SPLIT: also the split copy of
+// x64 that the double-single residual reads next, which saves its own pass
+template <class P, bool FIRST, bool SPLIT>
 __global__ void __launch_bounds__(NT) k_add_low(long V, long off, long n, long rs64, long rsl,
-                                                const typename P::SElem *e, double2 *x, const double *scale)
+                                                const typename P::SElem *e, double2 *x, float4 *xs, const double *scale)
 {
     using R = typename P::R;
     const double sc = scale ? scale[blockIdx.y] : 1.0;
     const typename P::SElem *eb = e + (long)blockIdx.y * rsl;
     double2 *xb = x + (long)blockIdx.y * rs64;
+    float4 *sb = xs + (SPLIT ? (long)blockIdx.y * rs64 : 0);
     for_chunks<P>(n, [&](long j, int k) {
         cpx<R> c[P::CW];
         P::ld_chunk(eb, V, off + j, k, c);
 #pragma unroll
         for (int q = 0; q < P::CW; q++) {
-            double2 *a = xb + (long)(k * P::CW + q) * V + off + j;
-            double2 av = *a;
-            *a = make_double2(av.x + sc * (double)c[q].re, av.y + sc * (double)c[q].im);
+            const long i = (long)(k * P::CW + q) * V + off + j;
+            double2 v = FIRST ? make_double2(0.0, 0.0) : xb[i];
+            v = make_double2(fma(sc, (double)c[q].re, v.x), fma(sc, (double)c[q].im, v.y));
+            xb[i] = v;
+            if (SPLIT) {
+                const float xh = (float)v.x, yh = (float)v.y;
+                sb[i] = make_float4(xh, yh, (float)(v.x - (double)xh), (float)(v.y - (double)yh));
+            }
         }
     });
 }
@@ -561,11 +568,16 @@ void to_low(ddrw_ctx *ctx, const VecRange &vr, long rsl, const double2 *in, type
 }
 
 template <class P>
-void add_low(ddrw_ctx *ctx, const VecRange &vr, long rsl, const typename P::SElem *e, double2 *x, const double *scale)
+void add_low(ddrw_ctx *ctx, const VecRange &vr, long rsl, const typename P::SElem *e, double2 *x, const double *scale,
+             bool first, float4 *xs)
 {
     ProfScope ps(ctx, PROF_BLAS, 0.0);
     ++ctx->launches;
-    k_add_low<P><<<dim3(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(vr.V, vr.off, vr.n, vr.rs, rsl, e, x, scale);
+    const dim3 g(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs);
+    if (first && xs) k_add_low<P, true, true><<<g, NT, 0, ctx->stream>>>(vr.V, vr.off, vr.n, vr.rs, rsl, e, x, xs, scale);
+    else if (first) k_add_low<P, true, false><<<g, NT, 0, ctx->stream>>>(vr.V, vr.off, vr.n, vr.rs, rsl, e, x, xs, scale);
+    else if (xs) k_add_low<P, false, true><<<g, NT, 0, ctx->stream>>>(vr.V, vr.off, vr.n, vr.rs, rsl, e, x, xs, scale);
+    else k_add_low<P, false, false><<<g, NT, 0, ctx->stream>>>(vr.V, vr.off, vr.n, vr.rs, rsl, e, x, xs, scale);
 }
 
 void f32_to_low(ddrw_ctx *ctx, const float4 *in, uint2 *out, long n, bool bf)
@@ -636,7 +648,7 @@ template void fold_16_into_32<PrecB>(ddrw_ctx *, const VecRange &, long, PrecB::
 
 #define DDRW_LOW_INST(P)                                                                                      \
     template void to_low<P>(ddrw_ctx *, const VecRange &, long, const double2 *, P::SElem *, const double *); \
-    template void add_low<P>(ddrw_ctx *, const VecRange &, long, const P::SElem *, double2 *, const double *);
+    template void add_low<P>(ddrw_ctx *, const VecRange &, long, const P::SElem *, double2 *, const double *, bool, float4 *);
 DDRW_LOW_INST(PrecS)
 DDRW_LOW_INST(PrecH)
 DDRW_LOW_INST(PrecB)

@@ -216,8 +216,10 @@ ddrw_status reduce_ws(ddrw_ctx *ctx, int nrhs, double **part, unsigned **ticket)
 template <class P>
 void to_low(ddrw_ctx *ctx, const VecRange &vr, long rsl, const double2 *in, typename P::SElem *out,
             const double *scale);
+// x += scale e (first: x = scale e); xs, if given, receives the split copy of x (double-single residual)
 template <class P>
-void add_low(ddrw_ctx *ctx, const VecRange &vr, long rsl, const typename P::SElem *e, double2 *x, const double *scale);
+void add_low(ddrw_ctx *ctx, const VecRange &vr, long rsl, const typename P::SElem *e, double2 *x, const double *scale,
+             bool first = false, float4 *xs = nullptr);
 // FP32 field (stride vr.rs) -> 16-bit field (stride rs16) over the range; and x32 += x16, x16 = 0
 template <class P16>
 void f32_to_16(ddrw_ctx *ctx, const VecRange &vr, long rs16, const float4 *in, typename P16::SElem *out);

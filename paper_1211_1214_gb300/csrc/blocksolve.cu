@@ -77,11 +77,12 @@ static ddrw_status colour_norms(ddrw_ctx *ctx, int colour, const double2 *f, int
 
 // One inner cycle of the mixed block solve in storage policy P: the colour's sites of rhs, scaled
 // by scale_d[r], go to P's storage, the persistent kernel solves them to tol_inner, and the
-// solution, scaled back by scale_d[nrhs + r], is added to x (zeroed first on the first cycle).
+// solution, scaled back by scale_d[nrhs + r], is added to x (is x on the first cycle), whose split copy for the
+// residual goes to xs.
 template <class P>
 static ddrw_status low_cycle(ddrw_ctx *ctx, int colour, const MassSet &ms, const double2 *rhs, double2 *x, bool first,
                              int nrhs, void *const *w, const double *scale_d, double tol_inner, int maxiter, int *stat,
-                             const double *tol2_dev = nullptr)
+                             float4 *xs, const double *tol2_dev = nullptr)
 {
     using E = typename P::SElem;
     const long rs64 = 12 * ctx->V, rsl = P::field_elems(ctx->V);
@@ -101,9 +102,8 @@ static ddrw_status low_cycle(ddrw_ctx *ctx, int colour, const MassSet &ms, const
         int hs[2] = {it, 0};
         DDRW_CUDA_CHECK(cudaMemcpyAsync(stat, hs, sizeof(hs), cudaMemcpyHostToDevice, ctx->stream));
         DDRW_SYNC(ctx);  // hs is stack memory
-        if (first) zero_colour64(ctx, x, colour, nrhs);
         for (int p = 0; p < 2; p++)
-            add_low<PrecS>(ctx, colour_range(ctx, colour, p, nrhs, rs64), 6 * ctx->V, x32, x, scale_d + nrhs);
+            add_low<PrecS>(ctx, colour_range(ctx, colour, p, nrhs, rs64), 6 * ctx->V, x32, x, scale_d + nrhs, first, xs);
         return DDRW_OK;
     }
     if ((st = workspace(ctx, "blkl_b", fl, &bl))) return st;
@@ -132,8 +132,8 @@ static ddrw_status low_cycle(ddrw_ctx *ctx, int colour, const MassSet &ms, const
     } else {
         launch_block(ctx, a, nrhs);
     }
-    if (first) zero_colour64(ctx, x, colour, nrhs);
-    for (int p = 0; p < 2; p++) add_low<P>(ctx, colour_range(ctx, colour, p, nrhs, rs64), rsl, (const E *)el, x, scale_d + nrhs);
+    for (int p = 0; p < 2; p++)
+        add_low<P>(ctx, colour_range(ctx, colour, p, nrhs, rs64), rsl, (const E *)el, x, scale_d + nrhs, first, xs);
     return DDRW_OK;
 }
 
@@ -236,6 +236,7 @@ ddrw_status block_solve_dc_prepare(ddrw_ctx *ctx, int nrhs)
     if ((st = workspace(ctx, "dcb_scale", sizeof(double) * 2 * nrhs, &p))) return st;
     if ((st = workspace(ctx, "dcb_ctl", sizeof(double) * 2, &p))) return st;
     if ((st = workspace(ctx, "blk_e64", sizeof(double2) * 12 * ctx->V * nrhs, &p))) return st;
+    if ((st = workspace(ctx, "res_norms", sizeof(double) * 2 * nrhs, &p))) return st;
     return DDRW_OK;
 }
 
@@ -264,7 +265,11 @@ static ddrw_status block_solve_dc(ddrw_ctx *ctx, int colour, const MassSet &ms, 
     for (int k = 0; k < 4; k++)
         if ((st = workspace(ctx, mixed ? names32[k] : names64[k], mixed ? f32 : f64, &w[k]))) return st;
 
+    float4 *xs = nullptr;
+    if (mixed && (st = split_copy(ctx, rs64, nrhs, &xs))) return st;
     if ((st = colour_norms_dev(ctx, colour, b, nrhs, bb2))) return st;
+    // (the residual's norms come summed over the parities: the second half stays zero)
+    DDRW_CUDA_CHECK(cudaMemsetAsync(rr2 + nrhs, 0, sizeof(double) * nrhs, ctx->stream));
     DDRW_CUDA_CHECK(cudaMemcpyAsync(res64, b, f64, cudaMemcpyDeviceToDevice, ctx->stream));
     zero_colour64(ctx, x, colour, nrhs);
     ++ctx->launches;
@@ -275,11 +280,11 @@ static ddrw_status block_solve_dc(ddrw_ctx *ctx, int colour, const MassSet &ms, 
         k_zero_ints<<<1, 32, 0, ctx->stream>>>(stat, 2);
         if (mixed) {  // the solution is added to x (zeroed above)
             if (prec == DDRW_MIXED_FP32)
-                s2 = low_cycle<PrecS>(ctx, colour, ms, res64, x, false, nrhs, w, scale, 1.0, maxiter, stat, tol2);
+                s2 = low_cycle<PrecS>(ctx, colour, ms, res64, x, false, nrhs, w, scale, 1.0, maxiter, stat, xs, tol2);
             else if (prec == DDRW_MIXED_FP16)
-                s2 = low_cycle<PrecH>(ctx, colour, ms, res64, x, false, nrhs, w, scale, 1.0, maxiter, stat, tol2);
+                s2 = low_cycle<PrecH>(ctx, colour, ms, res64, x, false, nrhs, w, scale, 1.0, maxiter, stat, xs, tol2);
             else
-                s2 = low_cycle<PrecB>(ctx, colour, ms, res64, x, false, nrhs, w, scale, 1.0, maxiter, stat, tol2);
+                s2 = low_cycle<PrecB>(ctx, colour, ms, res64, x, false, nrhs, w, scale, 1.0, maxiter, stat, xs, tol2);
             if (s2) return s2;
         } else {
             BlkArgs<PrecD> a;
@@ -298,9 +303,7 @@ static ddrw_status block_solve_dc(ddrw_ctx *ctx, int colour, const MassSet &ms, 
                 Blas<PrecD>::axpby(ctx, colour_range(ctx, colour, p, nrhs, rs64), 1.0, e64, 1.0, x);
         }
         DslashCall c = residual_call(ctx, ms, colour, x, res64, nrhs);
-        if ((s2 = residual_stencil(ctx, c, mixed))) return s2;
-        for (int p = 0; p < 2; p++) Blas<PrecD>::axpby(ctx, colour_range(ctx, colour, p, nrhs, rs64), 1.0, b, 1.0, res64);
-        if ((s2 = colour_norms_dev(ctx, colour, res64, nrhs, rr2))) return s2;
+        if ((s2 = residual_norms(ctx, c, b, rr2, mixed, xs))) return s2;
         ++ctx->launches;
         k_blk_ctl<<<1, 1, 0, ctx->stream>>>(1, nrhs, bb2, rr2, tol, floor, mixed, stat, scale, tol2, cyc, ctx->dc, slot, h);
         return DDRW_OK;
@@ -339,9 +342,12 @@ ddrw_status block_solve64(ddrw_ctx *ctx, int colour, const MassSet &ms, const do
     const char *names32[4] = {"blk32_r", "blk32_rh", "blk32_p", "blk32_v"};
     for (int k = 0; k < 4; k++)
         if ((st = workspace(ctx, mixed ? names32[k] : names64[k], mixed ? f32 : f64, &w[k]))) return st;
-    double *scale_d = nullptr;
+    double *scale_d = nullptr, *rr_d;
+    float4 *xs = nullptr;
+    if ((st = workspace(ctx, "blk_rr", sizeof(double) * nrhs, (void **)&rr_d))) return st;
     if (mixed) {
         if ((st = workspace(ctx, "blk_scale", sizeof(double) * 2 * nrhs, (void **)&scale_d))) return st;
+        if ((st = split_copy(ctx, rs64, nrhs, &xs))) return st;
     } else {
         if ((st = workspace(ctx, "blk_e64", f64, (void **)&e64))) return st;
     }
@@ -369,11 +375,11 @@ ddrw_status block_solve64(ddrw_ctx *ctx, int colour, const MassSet &ms, const do
             DDRW_CUDA_CHECK(cudaMemcpyAsync(scale_d + nrhs, unscale.data(), sizeof(double) * nrhs, cudaMemcpyHostToDevice,
                                             ctx->stream));
             if (prec == DDRW_MIXED_FP32)
-                st = low_cycle<PrecS>(ctx, colour, ms, rhs, x, first, nrhs, w, scale_d, tol_inner, maxiter, stat);
+                st = low_cycle<PrecS>(ctx, colour, ms, rhs, x, first, nrhs, w, scale_d, tol_inner, maxiter, stat, xs);
             else if (prec == DDRW_MIXED_FP16)
-                st = low_cycle<PrecH>(ctx, colour, ms, rhs, x, first, nrhs, w, scale_d, tol_inner, maxiter, stat);
+                st = low_cycle<PrecH>(ctx, colour, ms, rhs, x, first, nrhs, w, scale_d, tol_inner, maxiter, stat, xs);
             else
-                st = low_cycle<PrecB>(ctx, colour, ms, rhs, x, first, nrhs, w, scale_d, tol_inner, maxiter, stat);
+                st = low_cycle<PrecB>(ctx, colour, ms, rhs, x, first, nrhs, w, scale_d, tol_inner, maxiter, stat, xs);
             if (st) return st;
         } else {
             BlkArgs<PrecD> a;
@@ -393,12 +399,13 @@ ddrw_status block_solve64(ddrw_ctx *ctx, int colour, const MassSet &ms, const do
         }
         int hstat[2];
         DDRW_CUDA_CHECK(cudaMemcpyAsync(hstat, stat, sizeof(hstat), cudaMemcpyDeviceToHost, ctx->stream));
-        // true residual res = b - D_cc x in FP64
+        // true residual res = b - D_cc x in FP64 (or double-single), and its norms
         DslashCall c = residual_call(ctx, ms, colour, x, res64, nrhs);
-        if ((st = residual_stencil(ctx, c, mixed))) return st;
+        if ((st = residual_norms(ctx, c, b, rr_d, mixed, xs))) return st;
         if (stats) stats->fp64_dslash_half += 1;
-        for (int p = 0; p < 2; p++) Blas<PrecD>::axpby(ctx, colour_range(ctx, colour, p, nrhs, rs64), 1.0, b, 1.0, res64);
-        if ((st = colour_norms(ctx, colour, res64, nrhs, rr))) return st;
+        rr.resize(nrhs);
+        DDRW_CUDA_CHECK(cudaMemcpyAsync(rr.data(), rr_d, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, ctx->stream));
+        DDRW_SYNC(ctx);
         if (stats) {
             stats->block_iters_max = std::max(stats->block_iters_max, hstat[0]);
             stats->block_iters_total += hstat[0];

@@ -336,6 +336,10 @@ struct DslashCall {
     int red = 0;
     const void *w = nullptr;
     double *red_part = nullptr;
+    // double-single storage: out = rb + (the stencil's result), rb an FP64 field like out, and |out|^2 per
+    // warp of 32 sites into norm_part[rhs * (n / 32) + warp]
+    const double2 *rb = nullptr;
+    double *norm_part = nullptr;
 };
 void dslash64(ddrw_ctx *ctx, const DslashCall &c);
 // out = D(m) in for nrhs fields in the boundary layout (16-byte aligned, in and out apart)
@@ -352,9 +356,14 @@ void dslash_ds(ddrw_ctx *ctx, const DslashCall &c);
 // j < len) of nrhs fields rs elements apart; the same offsets in out
 void split64(ddrw_ctx *ctx, const double2 *in, float4 *out, long V, long vh, long off, long len, int par0, int npar,
              int nrhs, long rs);
-// out = alpha D x + ... as DslashCall c on FP64 fields, in FP64 (ds = false) or in double-single
-// arithmetic through a split copy of the input (ds = true)
-ddrw_status residual_stencil(ddrw_ctx *ctx, DslashCall c, bool ds);
+// out = alpha D x + ... as DslashCall c on FP64 fields in double-single arithmetic through a split copy of the
+// input; xs is that copy if the caller has it already (split_copy), else it is made here
+ddrw_status residual_stencil(ddrw_ctx *ctx, DslashCall c, const float4 *xs = nullptr);
+// out = b + (the stencil of call c) and norms[r] = |out|^2 over the call's sites (device): in FP64, or (ds) in
+// double-single arithmetic with the sum and the norm in the stencil's epilogue
+ddrw_status residual_norms(ddrw_ctx *ctx, DslashCall c, const double2 *b, double *norms, bool ds, const float4 *xs = nullptr);
+// the context's buffer for split copies of nrhs fields rs elements apart
+ddrw_status split_copy(ddrw_ctx *ctx, long rs, int nrhs, float4 **xs);
 
 // x = D_cc(ms)^-1 b on the sites of colour c (persistent block solver + FP64 defect correction)
 // device buffers of the device-controlled block solve (to allocate before a capture)

@@ -550,11 +550,11 @@ ddrw_status colour_bicgstab_reliable(ddrw_ctx *ctx, int pid, const MassSet &ms, 
 }
 
 // One inner solve of the defect correction in storage policy P: e = D^-1 rhs (rhs scaled by
-// scale_d[r] into P's storage, the solution scaled back by scale_d[nrhs + r] and added to x, which
-// is zeroed first on the first cycle).
+// scale_d[r] into P's storage, the solution scaled back by scale_d[nrhs + r] and added to x, or stored
+// there on the first cycle; the split copy of x for the residual goes to xs).
 template <class P>
 static ddrw_status inner_solve(ddrw_ctx *ctx, const MassSet &ms, const double2 *rhs, double2 *x, bool first, int nrhs,
-                               const double *scale_d, const std::vector<double> &th, int maxiter, int *iters)
+                               const double *scale_d, const std::vector<double> &th, int maxiter, int *iters, float4 *xs)
 {
     using E = typename P::SElem;
     const long V = ctx->V, rsl = P::field_elems(V);
@@ -575,8 +575,7 @@ static ddrw_status inner_solve(ddrw_ctx *ctx, const MassSet &ms, const double2 *
         if ((st = workspace(ctx, "full_e32", f32, (void **)&x32))) return st;
         to_low<PrecS>(ctx, all, 6 * V, rhs, b32, scale_d);
         if ((st = eo_bicgstab_reliable<P>(ctx, ms, b32, x32, nrhs, th, maxiter, iters))) return st;
-        if (first) DDRW_CUDA_CHECK(cudaMemsetAsync(x, 0, sizeof(double2) * 12 * V * nrhs, ctx->stream));
-        add_low<PrecS>(ctx, all, 6 * V, x32, x, scale_d + nrhs);
+        add_low<PrecS>(ctx, all, 6 * V, x32, x, scale_d + nrhs, first, xs);
         return DDRW_OK;
     }
     to_low<P>(ctx, all, rsl, rhs, (E *)bl, scale_d);
@@ -586,8 +585,7 @@ static ddrw_status inner_solve(ddrw_ctx *ctx, const MassSet &ms, const double2 *
     } else if ((st = eo_bicgstab<P>(ctx, ms, (const E *)bl, (E *)el, nrhs, th, maxiter, iters))) {
         return st;
     }
-    if (first) DDRW_CUDA_CHECK(cudaMemsetAsync(x, 0, sizeof(double2) * 12 * V * nrhs, ctx->stream));
-    add_low<P>(ctx, all, rsl, (const E *)el, x, scale_d + nrhs);
+    add_low<P>(ctx, all, rsl, (const E *)el, x, scale_d + nrhs, first, xs);
     return DDRW_OK;
 }
 
@@ -767,7 +765,7 @@ __global__ void k_full_ctl(int mode, int nrhs, const double *bb, const double *r
 
 template <class P>
 static ddrw_status inner_solve_dc(ddrw_ctx *ctx, const MassSet &ms, const double2 *rhs, double2 *x, int nrhs,
-                                  const double *scale, const double *th, int maxiter)
+                                  const double *scale, const double *th, int maxiter, float4 *xs)
 {
     using E = typename P::SElem;
     const long V = ctx->V, rsl = P::field_elems(V);
@@ -782,7 +780,7 @@ static ddrw_status inner_solve_dc(ddrw_ctx *ctx, const MassSet &ms, const double
     VecRange all{V, 0, V, 12 * V, nrhs};
     to_low<P>(ctx, all, rsl, rhs, (E *)bl, scale);
     if ((st = eo_bicgstab_dc<P>(ctx, ms, (const E *)bl, (E *)el, nrhs, th, maxiter))) return st;
-    add_low<P>(ctx, all, rsl, (const E *)el, x, scale + nrhs);
+    add_low<P>(ctx, all, rsl, (const E *)el, x, scale + nrhs, false, xs);
     return DDRW_OK;
 }
 
@@ -816,6 +814,8 @@ static ddrw_status full_solve_dc(ddrw_ctx *ctx, const MassSet &ms, const double2
     if ((st = workspace(ctx, "dcf_scale", sizeof(double) * 3 * nrhs, (void **)&scale))) return st;
     if ((st = workspace(ctx, "dcf_ctl", sizeof(int), (void **)&cyc))) return st;
     double *bb = norms, *rr = norms + nrhs, *th = scale + 2 * nrhs;
+    float4 *xs = nullptr;
+    if (mixed && (st = split_copy(ctx, rs64, nrhs, &xs))) return st;
     const VecRange all{V, 0, V, rs64, nrhs};
     if ((st = Blas<PrecD>::norm2(ctx, all, b, bb))) return st;
     DDRW_CUDA_CHECK(cudaMemcpyAsync(res, b, f64, cudaMemcpyDeviceToDevice, ctx->stream));
@@ -825,18 +825,16 @@ static ddrw_status full_solve_dc(ddrw_ctx *ctx, const MassSet &ms, const double2
     return capture_while(ctx, (const void *)k_full_ctl, [&](cudaGraphConditionalHandle h, int slot) -> ddrw_status {
         ddrw_status s2;
         if (mixed) {
-            if (prec == DDRW_MIXED_FP32) s2 = inner_solve_dc<PrecS>(ctx, ms, res, x, nrhs, scale, th, maxiter);
-            else if (prec == DDRW_MIXED_FP16) s2 = inner_solve_dc<PrecH>(ctx, ms, res, x, nrhs, scale, th, maxiter);
-            else s2 = inner_solve_dc<PrecB>(ctx, ms, res, x, nrhs, scale, th, maxiter);
+            if (prec == DDRW_MIXED_FP32) s2 = inner_solve_dc<PrecS>(ctx, ms, res, x, nrhs, scale, th, maxiter, xs);
+            else if (prec == DDRW_MIXED_FP16) s2 = inner_solve_dc<PrecH>(ctx, ms, res, x, nrhs, scale, th, maxiter, xs);
+            else s2 = inner_solve_dc<PrecB>(ctx, ms, res, x, nrhs, scale, th, maxiter, xs);
             if (s2) return s2;
         } else {
             if ((s2 = eo_bicgstab_dc<PrecD>(ctx, ms, res, e64, nrhs, th, maxiter))) return s2;
             Blas<PrecD>::axpby(ctx, all, 1.0, e64, 1.0, x);
         }
         DslashCall c = outer_residual_call(ctx, ms, x, res, nrhs);
-        if ((s2 = residual_stencil(ctx, c, mixed))) return s2;
-        Blas<PrecD>::axpby(ctx, all, 1.0, b, 1.0, res);
-        if ((s2 = Blas<PrecD>::norm2(ctx, all, res, rr))) return s2;
+        if ((s2 = residual_norms(ctx, c, b, rr, mixed, xs))) return s2;
         ++ctx->launches;
         k_full_ctl<<<1, 1, 0, ctx->stream>>>(1, nrhs, bb, rr, tol, floor, mixed, maxiter, scale, th, cyc, ctx->dc, slot, h);
         return DDRW_OK;
@@ -861,8 +859,12 @@ ddrw_status full_solve64(ddrw_ctx *ctx, const MassSet &ms, const double2 *b, dou
     double2 *res, *e64 = nullptr;
     double *scale_d = nullptr;
     if ((st = workspace(ctx, "full_res", f64, (void **)&res))) return st;
+    double *rr_d;
+    float4 *xs = nullptr;
+    if ((st = workspace(ctx, "full_rr", sizeof(double) * nrhs, (void **)&rr_d))) return st;
     if (mixed) {
         if ((st = workspace(ctx, "full_scale", sizeof(double) * 2 * nrhs, (void **)&scale_d))) return st;
+        if ((st = split_copy(ctx, rs64, nrhs, &xs))) return st;
     } else if ((st = workspace(ctx, "full_e64", f64, (void **)&e64))) {
         return st;
     }
@@ -889,9 +891,9 @@ ddrw_status full_solve64(ddrw_ctx *ctx, const MassSet &ms, const double2 *b, dou
                 double ti = std::max(floor, std::min(need, 0.5));
                 th[r] = nr[r] > 0 ? ti * ti : 0.0;
             }
-            if (prec == DDRW_MIXED_FP32) st = inner_solve<PrecS>(ctx, ms, rhs, x, first, nrhs, scale_d, th, maxiter, &iters);
-            else if (prec == DDRW_MIXED_FP16) st = inner_solve<PrecH>(ctx, ms, rhs, x, first, nrhs, scale_d, th, maxiter, &iters);
-            else st = inner_solve<PrecB>(ctx, ms, rhs, x, first, nrhs, scale_d, th, maxiter, &iters);
+            if (prec == DDRW_MIXED_FP32) st = inner_solve<PrecS>(ctx, ms, rhs, x, first, nrhs, scale_d, th, maxiter, &iters, xs);
+            else if (prec == DDRW_MIXED_FP16) st = inner_solve<PrecH>(ctx, ms, rhs, x, first, nrhs, scale_d, th, maxiter, &iters, xs);
+            else st = inner_solve<PrecB>(ctx, ms, rhs, x, first, nrhs, scale_d, th, maxiter, &iters, xs);
             if (st) return st;
         } else {
             double2 *target = first ? x : e64;
@@ -900,12 +902,13 @@ ddrw_status full_solve64(ddrw_ctx *ctx, const MassSet &ms, const double2 *b, dou
             if ((st = eo_bicgstab<PrecD>(ctx, ms, rhs, target, nrhs, th, maxiter, &iters))) return st;
             if (!first) Blas<PrecD>::axpby(ctx, VecRange{V, 0, V, rs64, nrhs}, 1.0, e64, 1.0, x);
         }
-        // res = b - D x in FP64
+        // res = b - D x in FP64 (or double-single), and its norms
         DslashCall c = outer_residual_call(ctx, ms, x, res, nrhs);
-        if ((st = residual_stencil(ctx, c, mixed))) return st;
+        if ((st = residual_norms(ctx, c, b, rr_d, mixed, xs))) return st;
         if (stats) stats->fp64_dslash_full += 1;
-        Blas<PrecD>::axpby(ctx, VecRange{V, 0, V, rs64, nrhs}, 1.0, b, 1.0, res);
-        if ((st = full_norms(ctx, res, nrhs, rr))) return st;
+        rr.resize(nrhs);
+        DDRW_CUDA_CHECK(cudaMemcpyAsync(rr.data(), rr_d, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, ctx->stream));
+        DDRW_SYNC(ctx);
         double worst = 0;
         for (int r = 0; r < nrhs; r++)
             if (!std::isfinite(rr[r])) worst = NAN;
