@@ -367,6 +367,7 @@ __global__ void __launch_bounds__(NT) k_to_low(long V, long off, long n, long rs
                                                typename P::SElem *out, const double *scale)
 {
     using R = typename P::R;
+    static_assert(sizeof(R) == 4, "");
     const double sc = scale ? scale[blockIdx.y] : 1.0;
     const double2 *ib = in + (long)blockIdx.y * rs64;
     typename P::SElem *ob = out + (long)blockIdx.y * rsl;
@@ -375,7 +376,7 @@ __global__ void __launch_bounds__(NT) k_to_low(long V, long off, long n, long rs
 #pragma unroll
         for (int q = 0; q < P::CW; q++) {
             double2 a = ib[(long)(k * P::CW + q) * V + off + j];
-            c[q] = {R(a.x * sc), R(a.y * sc)};
+            c[q] = {to_f32(a.x * sc), to_f32(a.y * sc)};
         }
         P::st_chunk(ob, V, off + j, k, c);
     });
@@ -399,11 +400,11 @@ __global__ void __launch_bounds__(NT) k_add_low(long V, long off, long n, long r
         for (int q = 0; q < P::CW; q++) {
             const long i = (long)(k * P::CW + q) * V + off + j;
             double2 v = FIRST ? make_double2(0.0, 0.0) : xb[i];
-            v = make_double2(fma(sc, (double)c[q].re, v.x), fma(sc, (double)c[q].im, v.y));
+            v = make_double2(fma(sc, to_f64(c[q].re), v.x), fma(sc, to_f64(c[q].im), v.y));
             xb[i] = v;
             if (SPLIT) {
-                const float xh = (float)v.x, yh = (float)v.y;
-                sb[i] = make_float4(xh, yh, (float)(v.x - (double)xh), (float)(v.y - (double)yh));
+                const float xh = to_f32(v.x), yh = to_f32(v.y);
+                sb[i] = make_float4(xh, yh, to_f32(v.x - to_f64(xh)), to_f32(v.y - to_f64(yh)));
             }
         }
     });

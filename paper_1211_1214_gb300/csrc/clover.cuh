@@ -163,7 +163,7 @@ static __global__ void __launch_bounds__(128) k_clover_assemble(long V, const do
 #pragma unroll
         for (int k = 0; k < 9; k++)
             C32[((long)ch * 9 + k) * V + s] =
-                make_float4((float)r[4 * k], (float)r[4 * k + 1], (float)r[4 * k + 2], (float)r[4 * k + 3]);
+                make_float4(to_f32(r[4 * k]), to_f32(r[4 * k + 1]), to_f32(r[4 * k + 2]), to_f32(r[4 * k + 3]));
     }
 }
 

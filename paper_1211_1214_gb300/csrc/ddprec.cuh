@@ -212,16 +212,6 @@ struct PrecDD {
 #pragma unroll
         for (int k = 0; k < 12; k++) p.v[k / 3][k % 3] = unpack(f[k * stride + s]);
     }
-    // the output field is FP64 (16-byte double2 elements at the same offsets)
-    __device__ static __forceinline__ void store_spinor(SElem *__restrict__ f, int stride, int s, const Spinor<R> &p)
-    {
-        double2 *o = reinterpret_cast<double2 *>(f);
-#pragma unroll
-        for (int k = 0; k < 12; k++) {
-            const cpx<dd> &c = p.v[k / 3][k % 3];
-            o[k * stride + s] = make_double2((double)c.re.hi + (double)c.re.lo, (double)c.im.hi + (double)c.im.lo);
-        }
-    }
     __device__ static __forceinline__ void load_chiral(const SElem *__restrict__ f, int stride, int s, int ch, cpx<R> *v)
     {
 #pragma unroll

@@ -295,6 +295,29 @@ __device__ __forceinline__ void link_dag_mul(const Link<R> &U, const Half<R> &h,
         }
 }
 
+// FP32 <-> FP64 conversions in integer arithmetic, for the kernels that convert whole fields: the conversion
+// instructions run in the FP64 pipe at 2 per clock and SM, the integer ones (4 and 9 of them) at 64.  Same bits as
+// the casts: ordinary numbers and zeros here, the rest (subnormals, overflow, infinities, NaN) by the cast.
+// 16^4, 16 right-hand sides, one block solve's fields: x += scale e with its split copy 98 -> 55 us, FP64 to FP32 35 -> 25 us.
+__device__ __forceinline__ double to_f64(float f)
+{
+    const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u || m == 0u)
+        return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + (m ? 0x38000000u : 0u))), (int)(b << 29));
+    return (double)f;
+}
+// round to nearest, ties to even: half an ulp less one unit, plus the last bit kept, carries out of the dropped 29 bits
+__device__ __forceinline__ float to_f32(double d)
+{
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d), m = hi & 0x7fffffffu;
+    if (m - 0x38100000u < 0x0fe00000u) {  // 2^-126 <= |d| < 2^128 (what rounds up to 2^128 becomes infinity)
+        const unsigned q = __funnelshift_l(lo, m - 0x38000000u, 3);
+        return __uint_as_float((hi & 0x80000000u) | (q + (((lo & 0x1fffffffu) + 0x0fffffffu + (q & 1u)) >> 29)));
+    }
+    if ((m | lo) == 0u) return __uint_as_float(hi);
+    return (float)d;
+}
+
 // ---- packed FP32 (two FP32 operations per instruction, Blackwell's f32x2 forms): U h or U^dag h with the two
 // spins of a half spinor packed, which meet the same link element; the products and sums of
 // link_mul in the same order.  The FMA units take as long as for two scalar instructions (measured), but a

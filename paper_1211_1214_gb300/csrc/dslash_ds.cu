@@ -24,8 +24,8 @@ __global__ void k_split(long V, long vh, long off, long len, int par0, int npar,
     const int k = blockIdx.y / npar, p = blockIdx.y - k * npar;
     const long idx = (long)blockIdx.z * rs + (long)k * V + (long)(par0 + p) * vh + off + j;
     double2 v = in[idx];
-    float xh = (float)v.x, yh = (float)v.y;
-    out[idx] = make_float4(xh, yh, (float)(v.x - (double)xh), (float)(v.y - (double)yh));
+    const float xh = to_f32(v.x), yh = to_f32(v.y);
+    out[idx] = make_float4(xh, yh, to_f32(v.x - to_f64(xh)), to_f32(v.y - to_f64(yh)));
 }
 
 void split64(ddrw_ctx *ctx, const double2 *in, float4 *out, long V, long vh, long off, long len, int par0, int npar,
