@@ -156,10 +156,10 @@ ddrw_status ddrw_set_low_precision(ddrw_ctx *ctx, int reliable_updates, int bloc
 
 /* With enable != 0 the FP32 even-odd BiCGStab of the full-lattice solves computes the inner
  * products of alpha = rho / (rh, v) and omega = (t, s) / (t, t) in the epilogue of the stencil launch
- * that writes v and t (one partial per warp of 32 sites, summed in FP64 in a fixed order by a small
- * kernel) instead of re-reading v, t and s in separate reductions; 0 (the default) uses the
- * separate reduction kernels -- on one GB300 the fused launch is 40 % slower than the plain one,
- * which outweighs the reductions it saves.  Results differ only by the rounding of the sums. */
+ * that writes v and t (one partial per warp of 32 sites, summed in a fixed order by a small kernel)
+ * instead of re-reading v, t and s in separate reductions; with 0 it uses the separate reduction
+ * kernels.  A context on which this was never called chooses by size (the fused form on small
+ * lattices with few right-hand sides).  Results differ only by the rounding of the sums. */
 ddrw_status ddrw_fuse_reductions(ddrw_ctx *ctx, int enable);
 
 /* How the block solves D_cc(m)^-1 of the mixed precisions run (Eq. 1; the four solves of r and the

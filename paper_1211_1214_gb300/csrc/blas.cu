@@ -242,29 +242,33 @@ __global__ void __launch_bounds__(NT, 2) k_bicg_xrp(VecArgs<P> va, typename P::S
     }
 }
 
-// alpha (MODE 1) or omega and beta (MODE 2) from the per-warp partial sums a fused stencil epilogue
-// wrote: part[(r * nwt + j) * RED_PARTS + k], summed in FP64 in a fixed order (one CTA per
-// right-hand side)
+// alpha (MODE 1) or omega and beta (MODE 2) from the per-warp partial sums (float pairs) a fused stencil
+// epilogue wrote: part[(r * nwt + j) * RED_PARTS + k], in a fixed order (one CTA per right-hand side)
 template <int MODE>
-__global__ void __launch_bounds__(NT) k_bicg_fin(const double *part, long nwt, KScal *sc)
+__global__ void __launch_bounds__(NT) k_bicg_fin(const float2 *part, long nwt, KScal *sc)
 {
     constexpr int K = MODE == 1 ? 2 : RED_PARTS;
-    __shared__ double sm[NT / 32][K], tot[K];
+    __shared__ float2 sm[NT / 32][K], tot[K];
     const int r = blockIdx.x;
     if (!sc[r].active) return;
-    RunSum<double> v[K];
+    RunSum<float> v[K];
+#pragma unroll 2
     for (long j = threadIdx.x; j < nwt; j += NT) {
-        const double *pp = part + ((long)r * nwt + j) * RED_PARTS;
+        const float2 *pp = part + ((long)r * nwt + j) * RED_PARTS;
 #pragma unroll
-        for (int k = 0; k < K; k++) v[k].add(pp[k]);
+        for (int k = 0; k < K; k++) v[k].join(pp[k]);
     }
-    cta_sum_run<K, NT, double>(v, sm, tot);
+    cta_sum_run<K, NT, float>(v, sm, tot);
     if (threadIdx.x >= 32) return;
     __syncwarp();
     if (threadIdx.x != 0) return;
     double val[K];
 #pragma unroll
-    for (int k = 0; k < K; k++) val[k] = tot[k];
+    for (int k = 0; k < K; k++) {
+        RunSum<float> q;
+        q.join(tot[k]);
+        val[k] = q.value();
+    }
     KScal &s = sc[r];
     if constexpr (MODE == 1) {  // alpha = rho / (rh, v)
         const double den = val[0] * val[0] + val[1] * val[1];
@@ -284,8 +288,8 @@ void bicg_fin(ddrw_ctx *ctx, int mode, int nrhs, const double *part, long nwt, K
 {
     ProfScope ps(ctx, PROF_BLAS, 0.0);
     ++ctx->launches;
-    if (mode == 1) k_bicg_fin<1><<<nrhs, NT, 0, ctx->stream>>>(part, nwt, sc);
-    else k_bicg_fin<2><<<nrhs, NT, 0, ctx->stream>>>(part, nwt, sc);
+    if (mode == 1) k_bicg_fin<1><<<nrhs, NT, 0, ctx->stream>>>((const float2 *)part, nwt, sc);
+    else k_bicg_fin<2><<<nrhs, NT, 0, ctx->stream>>>((const float2 *)part, nwt, sc);
 }
 
 // ----------------------------------------------------------------------------- generic kernels

@@ -133,9 +133,8 @@ struct ddrw_ctx {
     // side), 1 the Krylov-loop BiCGStab on the colour's blocks as one block-diagonal system
     int block_method = 0;
     // the BiCGStab inner products of alpha and omega fused into the epilogue of the stencil launch
-    // that writes v and t (FP32 storage, full lattice); off (the default, measured faster on
-    // GB300): separate reduction kernels
-    bool fuse_dots = false;
+    // that writes v and t (FP32 storage, full lattice): 1 always, 0 never, -1 by size (solver.cu)
+    int fuse_dots = -1;
     // 16-bit storage precisions: the full-lattice inner solves keep their Krylov vectors in 16-bit
     // storage with reliable updates into FP32 (true), or restart at each defect-correction cycle;
     // the block solves run on 16-bit storage (true) or in FP32

@@ -20,6 +20,7 @@
 
 #include <type_traits>
 
+#include "blas.cuh"
 #include "ctx.h"
 #include "ddprec.cuh"
 #include "lowprec.cuh"
@@ -229,7 +230,7 @@ constexpr size_t STAGED_SMEM_MAX = (size_t)62 * 128 * 16;
 // 16-bit storage with the loads of each hop issued before its arithmetic),
 // 11 fully rolled (one body for the eight hops; double-single storage only)
 // RED != 0 adds the inner products of the output to the epilogue (red 1: conj(w) out; red 2:
-// conj(out) x, |out|^2, conj(w) x and conj(w) out), one partial per warp of 32 sites, summed in FP64 by k_bicg_fin; the
+// conj(out) x, |out|^2, conj(w) x and conj(w) out), one partial (float pair) per warp of 32 sites, summed by k_bicg_fin; the
 // launcher only fuses launches whose output sites fill whole CTAs (no thread leaves early)
 // launch bounds by form (CTAs of 256 threads; the double-single rolled form: 128, three per SM)
 template <class P, int ROLL> constexpr int ds_threads() { return std::is_same<P, PrecDD>::value && ROLL == 11 ? 128 : 256; }
@@ -365,38 +366,44 @@ __global__ void __launch_bounds__(ds_threads<P, ROLL>(), ds_ctas<P, ROLL>())
     if constexpr (RED != 0) {
         static_assert(NR == 1, "fused inner products take one right-hand side per thread");
         constexpr int K = RED == 1 ? 2 : RED_PARTS;
-        Spinor<R> h, q;
-        P::load_spinor(a.w + roff, g.V, s, h);
-        if (RED == 2) P::load_spinor(a.x + roff, g.V, s, q);
-        R d[K] = {};
+        using WS = WarpSums<K, R>;
+        RunSum<R> d[K];
 #pragma unroll
-        for (int sp = 0; sp < 4; sp++)
+        for (int k = 0; k < P::NCHUNK; k++) {
+            cpx<R> hv[P::CW], qv[P::CW], os = {R(0), R(0)}, hs = {R(0), R(0)}, ho = {R(0), R(0)};
+            R oo = 0;
+            P::ld_chunk(a.w + roff, g.V, s, k, hv);
+            if (RED == 2) P::ld_chunk(a.x + roff, g.V, s, k, qv);
 #pragma unroll
-            for (int c = 0; c < 3; c++) {
-                const cpx<R> o = acc[0].v[sp][c], hv = h.v[sp][c];
-                const cpx<R> ho = cmulc(hv, o);
-                if constexpr (RED == 1) {
-                    d[0] += ho.re;
-                    d[1] += ho.im;
-                } else {
-                    const cpx<R> os = cmulc(o, q.v[sp][c]), hs = cmulc(hv, q.v[sp][c]);
-                    d[0] += os.re;
-                    d[1] += os.im;
-                    d[2] += o.re * o.re + o.im * o.im;
-                    d[3] += hs.re;
-                    d[4] += hs.im;
-                    d[5] += ho.re;
-                    d[6] += ho.im;
+            for (int q = 0; q < P::CW; q++) {
+                const int e = k * P::CW + q;
+                const cpx<R> o = acc[0].v[e / 3][e % 3];
+                cmacc(ho, hv[q], o);
+                if constexpr (RED == 2) {
+                    cmacc(os, o, qv[q]);
+                    oo = fmad(o.re, o.re, fmad(o.im, o.im, oo));
+                    cmacc(hs, hv[q], qv[q]);
                 }
             }
-        double *pp = a.part + ((long)r0 * a.nwt + tile * (blockDim.x >> 5) + (threadIdx.x >> 5)) * RED_PARTS;
-#pragma unroll
-        for (int k = 0; k < K; k++) {
-            double e = d[k];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-            if ((threadIdx.x & 31) == 0) pp[k] = e;
+            if constexpr (RED == 1) {
+                d[0].add(ho.re);
+                d[1].add(ho.im);
+            } else {
+                d[0].add(os.re);
+                d[1].add(os.im);
+                d[2].add(oo);
+                d[3].add(hs.re);
+                d[4].add(hs.im);
+                d[5].add(ho.re);
+                d[6].add(ho.im);
+            }
         }
+        using Raw = typename RunSum<R>::Raw;
+        Raw *pp = reinterpret_cast<Raw *>(a.part) +
+                  ((long)r0 * a.nwt + tile * (blockDim.x >> 5) + (threadIdx.x >> 5)) * RED_PARTS;
+        const RunSum<R> t = WS::total(d);
+        const int lane = threadIdx.x & 31, k = lane >> WS::SHIFT;
+        if ((lane & ((1 << WS::SHIFT) - 1)) == 0 && k < K) pp[k] = t.raw();
     }
     if constexpr (std::is_same<P, PrecDD>::value) {
         // the residual b - D x and its norm here instead of in an axpby and a norm pass over FP64 fields
@@ -635,17 +642,20 @@ void launch_cfg(ddrw_ctx *ctx, const DslashCall &c, const DsArgs<P> &a, DsConfig
     if (c.hopsel == 1 && cfg.roll == 6 && !g.nbr) cfg.roll = 5;
     if constexpr (std::is_same<P, PrecS>::value) {
         if (c.red != 0) {
-            // the fused epilogue: one right-hand side per thread, unrolled or register-capped form,
+            // the fused epilogue: one right-hand side per thread, the unrolled, register-capped or table form,
             // whole CTAs (the caller checks that 256 divides the output sites)
-            if (cfg.nr != 1 || (cfg.roll != 0 && cfg.roll != 5) || n % cfg.nt) cfg = DsConfig{1, 64, 1, 5};
+            if (cfg.nr != 1 || (cfg.roll != 0 && cfg.roll != 5 && cfg.roll != 6) || n % cfg.nt) cfg = DsConfig{1, 64, 1, 5};
+            if (cfg.roll == 6 && !g.nbr) cfg.roll = 5;
             const unsigned gr = (unsigned)((n / cfg.nt) * (c.nrhs / cfg.nw));
             const dim3 bk((unsigned)cfg.nt, (unsigned)cfg.nw);
             ++ctx->launches;
             if (c.red == 1) {
-                if (cfg.roll == 5) k_dslash<P, BL, 0, 1, 5, 1><<<gr, bk, 0, ctx->stream>>>(g, a);
+                if (cfg.roll == 6) k_dslash<P, BL, 0, 1, 6, 1><<<gr, bk, 0, ctx->stream>>>(g, a);
+                else if (cfg.roll == 5) k_dslash<P, BL, 0, 1, 5, 1><<<gr, bk, 0, ctx->stream>>>(g, a);
                 else k_dslash<P, BL, 0, 1, 0, 1><<<gr, bk, 0, ctx->stream>>>(g, a);
             } else {
-                if (cfg.roll == 5) k_dslash<P, BL, 0, 1, 5, 2><<<gr, bk, 0, ctx->stream>>>(g, a);
+                if (cfg.roll == 6) k_dslash<P, BL, 0, 1, 6, 2><<<gr, bk, 0, ctx->stream>>>(g, a);
+                else if (cfg.roll == 5) k_dslash<P, BL, 0, 1, 5, 2><<<gr, bk, 0, ctx->stream>>>(g, a);
                 else k_dslash<P, BL, 0, 1, 0, 2><<<gr, bk, 0, ctx->stream>>>(g, a);
             }
             return;

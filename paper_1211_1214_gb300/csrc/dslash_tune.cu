@@ -62,7 +62,8 @@ DsConfig tuned_config(ddrw_ctx *ctx, const DslashCall &c, int prec, int bl,
         if (p.roll != 8 && (c.nrhs % (p.nr * p.nw) || rpm % (p.nr * p.nw))) p.nr = 1, p.nw = 1;
         return p;
     }
-    std::array<int, 8> key = {prec, bl, c.npar, c.nrhs, c.diag, c.post, rpm, (c.beta != 0.0) + 2 * c.hopsel};
+    // (a launch with a fused epilogue is another kernel: diag + 4 red)
+    std::array<int, 8> key = {prec, bl, c.npar, c.nrhs, c.diag + 4 * c.red, c.post, rpm, (c.beta != 0.0) + 2 * c.hopsel};
     auto it = ctx->tune.find(key);
     if (it != ctx->tune.end()) return DsConfig{it->second.nr, it->second.nt, it->second.nw, it->second.roll};
     if (ctx->autotune) {
@@ -196,7 +197,7 @@ ddrw_status ddrw_autotune_report(ddrw_ctx *ctx, char *buf, long len)
         char line[200];
         snprintf(line, sizeof line,
                  "fp%d l=%d npar=%d nrhs=%d diag=%d post=%d rpm=%d hop=%d sel=%d -> nr=%d nt=%d nw=%d roll=%d ms=%.4f\n",
-                 k[0], k[1], k[2], k[3], k[4], k[5], k[6], k[7] & 1, k[7] >> 1, kv.second.nr, kv.second.nt, kv.second.nw,
+                 k[0], k[1], k[2], k[3], k[4] & 3, k[5], k[6], k[7] & 1, k[7] >> 1, kv.second.nr, kv.second.nt, kv.second.nw,
                  kv.second.roll, kv.second.ms);
         s += line;
     }

@@ -171,6 +171,17 @@ void apply_mhat(ddrw_ctx *ctx, const MassSet &ms, int nrhs, long rs, const typen
     stencil<P>(ctx, d);
 }
 
+// Where the inner products of alpha and omega go into the epilogue of the stencil that writes v and t (FP32
+// storage), if the caller has not said: small launches, whose reduction kernels are mostly their fixed 5 to 8 us.
+// Whole FP32 solves, separate / fused: 24x12^3 with 5 right-hand sides 5097 / 4813 us, 16^4 with 2 3426 / 3217,
+// with 4 5407 / 5310, with 8 9122 / 9150, 8^4 with 16 2121 / 1969; on 32x16^3 one CTA has 2048 partial sums to
+// add: with 2 6136 / 6185, with 4 10782 / 10974.  (With FP64 sums in the epilogue the fused form lost everywhere.)
+static bool fuse_reductions(const ddrw_ctx *ctx, int nrhs)
+{
+    if (ctx->vh % 256) return false;  // whole CTAs
+    return ctx->fuse_dots < 0 ? ctx->vh <= 1L << 15 && ctx->vh * nrhs <= 1L << 17 : ctx->fuse_dots > 0;
+}
+
 // One BiCGStab iteration on the even-odd operator for nrhs right-hand sides (scalars on the device)
 template <class P>
 static ddrw_status bicg_iteration(ddrw_ctx *ctx, const MassSet &ms, int nrhs, long rs, const VecRange &ev,
@@ -179,7 +190,7 @@ static ddrw_status bicg_iteration(ddrw_ctx *ctx, const MassSet &ms, int nrhs, lo
                                   typename P::SElem *tmp, KScal *sc, int colour = -1)
 {
     ddrw_status s2;
-    if (P::ID == 32 && colour < 0 && ctx->fuse_dots && ctx->vh % 256 == 0) {
+    if (P::ID == 32 && colour < 0 && fuse_reductions(ctx, nrhs)) {
         // the inner products of alpha and omega in the epilogue of the stencil that writes v and t
         const long nwt = ctx->vh / 32;
         double *part;
