@@ -163,8 +163,8 @@ ddrw_status ddrw_set_low_precision(ddrw_ctx *ctx, int reliable_updates, int bloc
 ddrw_status ddrw_fuse_reductions(ddrw_ctx *ctx, int enable);
 
 /* How the block solves D_cc(m)^-1 of the mixed precisions run (Eq. 1; the four solves of r and the
- * block solves of the Schur operator): method 0, the persistent kernel -- one CTA per (block,
- * right-hand side) running the whole in-block even-odd BiCGStab with CTA-wide reductions; method 1,
+ * block solves of the Schur operator): method 0, the persistent kernel -- one cluster of CTAs per
+ * (block, right-hand side) running the whole in-block even-odd BiCGStab with cluster-wide reductions; method 1,
  * all blocks of the colour as one block-diagonal system in the graph-captured even-odd BiCGStab
  * of the outer solver (tuned stencil launches restricted to the hops inside the blocks, scalars
  * per right-hand side over the colour).  Both feed the same FP64 defect correction to tol_block;
@@ -294,7 +294,7 @@ ddrw_status ddrw_force(ddrw_ctx *ctx, int nhit, uint64_t seed, uint64_t hit_offs
  * this is an integration aid.  Some callers may not call cudaMalloc -- code running while a
  * framework's memory pool is frozen, or a host application that owns every device allocation and
  * forbids libraries their own -- and ddrw_solve_block grows its workspace with cudaMalloc.  This
- * call allocates nothing: its scratch (about 40 MB: ten FP64 fields of up to 20736 sites plus
+ * call allocates nothing: its scratch (about 32 MB: eight FP64 fields of up to 20736 sites plus
  * reduction slots) is one fixed array in device memory that every GPU using the library holds
  * until the process exits.
  *   - One right-hand side, FP64 (whatever ddrw_set_solver chose), tolerance tol_block, same
@@ -373,7 +373,8 @@ ddrw_status ddrw_test_stall_staging(ddrw_ctx *ctx, int enable);
  * log prod_k det D_k^2(m2) / det D_k^2(m1) for the m1, m2 of ddrw_set_params (two flavours).
  * Method: det D_k = det A_oo det S_k with S_k = A_ee - D_eo A_oo^-1 D_oe the block's even-odd
  * Schur complement (dimension 6 l^4), assembled by the FP64 block stencil and factorised by a
- * batched LU with partial pivoting in FP64 (one CTA per block).  The paper calls the exact block
+ * batched LU with partial pivoting in FP64 (one CTA per block; for l = 2 one kernel does both in
+ * shared memory).  The paper calls the exact block
  * determinants feasible for l^4 <= 6^4; l > 6 returns DDRW_EINVAL, and blocks are processed in
  * batches that fit 60 % of the free device memory (DDRW_ENOMEM if one matrix does not fit).
  * Cost: (6 l^4)^3 / 3 complex FP64 multiply-adds per block and mass, one SM per block: 16^4

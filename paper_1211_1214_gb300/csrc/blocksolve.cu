@@ -3,8 +3,9 @@
 //
 // One cluster of CTAs owns one (block, right-hand side) pair and runs the whole Krylov solve inside the
 // kernel: in-block even-odd preconditioning S = A_ee - 1/4 H_eo A_oo^-1 H_oe (hops inside the block
-// only), BiCGStab on S with cluster-wide reductions (warp shuffles and distributed shared memory), then x_o = A_oo^-1 (b_o + 1/2 H_oe x_e).  The block's sites of one parity are contiguous in the
-// block-major layout, so every pass is a coalesced sweep over the block.
+// only), BiCGStab on S with cluster-wide reductions (warp shuffles and distributed shared memory), then
+// x_o = A_oo^-1 (b_o + 1/2 H_oe x_e).  The block's sites of one parity are contiguous in the block-major
+// layout, so every pass is a coalesced sweep over the block.
 //
 // The host driver wraps the kernel in FP64 defect correction: r = b - D_cc x in FP64, the kernel
 // (FP64 or FP32) solves D_cc e = r to a relative tolerance per block, x += e, until

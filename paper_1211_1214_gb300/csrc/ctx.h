@@ -129,7 +129,7 @@ struct ddrw_ctx {
     int outer_method = 0;
     int sap_ncy = 4, sap_nmr = 4, sap_nkv = 8;
     int sap_last_iters = 0;
-    // block solves of the mixed precisions: 0 the persistent kernel (one CTA per block and right-hand
+    // block solves of the mixed precisions: 0 the persistent kernel (one cluster of CTAs per block and right-hand
     // side), 1 the Krylov-loop BiCGStab on the colour's blocks as one block-diagonal system
     int block_method = 0;
     // the BiCGStab inner products of alpha and omega fused into the epilogue of the stencil launch

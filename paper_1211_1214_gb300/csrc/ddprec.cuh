@@ -12,9 +12,9 @@
 // (dd2_acc below).
 //
 // Storage: a "split" field holds one complex number per 16-byte element (re.hi, im.hi, re.lo,
-// im.lo: the register pairs of the packed arithmetic), the same bytes as an FP64 field; links (9 complex per direction) and the clover term
-// (72 reals per site) are split once per configuration, the stencil input once per residual, and
-// the result is written back as FP64 (hi + lo).
+// im.lo: the register pairs of the packed arithmetic), the same bytes as an FP64 field; links (9 complex per
+// direction) and the clover term (72 reals per site) are split once per configuration, the stencil input
+// once per residual, and the result is written back as FP64 (hi + lo).
 #pragma once
 
 #include "ddrw_internal.cuh"

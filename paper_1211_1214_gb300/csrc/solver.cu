@@ -179,7 +179,9 @@ void apply_mhat(ddrw_ctx *ctx, const MassSet &ms, int nrhs, long rs, const typen
 static bool fuse_reductions(const ddrw_ctx *ctx, int nrhs)
 {
     if (ctx->vh % 256) return false;  // whole CTAs
-    return ctx->fuse_dots < 0 ? ctx->vh <= 1L << 15 && ctx->vh * nrhs <= 1L << 17 : ctx->fuse_dots > 0;
+    if (ctx->fuse_dots < 0)  // (a pinned launch form keeps its launches)
+        return ctx->pinned_nr == 0 && ctx->vh <= 1L << 15 && ctx->vh * nrhs <= 1L << 17;
+    return ctx->fuse_dots > 0;
 }
 
 // One BiCGStab iteration on the even-odd operator for nrhs right-hand sides (scalars on the device)
