@@ -20,6 +20,7 @@
 namespace ddrw {
 
 template <class P, int BL> void launch_block_kernel(ddrw_ctx *ctx, const BlkArgs<P> &a, int nrhs);
+ddrw_status block_plain32(ddrw_ctx *ctx, const BlkArgs<PrecS> &args, int nrhs);  // blockplain.cu
 
 // ----------------------------------------------------------------------------- host side
 
@@ -83,7 +84,7 @@ static ddrw_status colour_norms(ddrw_ctx *ctx, int colour, const double2 *f, int
 template <class P>
 static ddrw_status low_cycle(ddrw_ctx *ctx, int colour, const MassSet &ms, const double2 *rhs, double2 *x, bool first,
                              int nrhs, void *const *w, const double *scale_d, double tol_inner, int maxiter, int *stat,
-                             float4 *xs, const double *tol2_dev = nullptr)
+                             float4 *xs, const double *tol2_dev = nullptr, bool plain = false)
 {
     using E = typename P::SElem;
     const long rs64 = 12 * ctx->V, rsl = P::field_elems(ctx->V);
@@ -131,7 +132,10 @@ static ddrw_status low_cycle(ddrw_ctx *ctx, int colour, const MassSet &ms, const
         DDRW_CUDA_CHECK(cudaMemcpyAsync(stat, hs, sizeof(hs), cudaMemcpyHostToDevice, ctx->stream));
         DDRW_SYNC(ctx);  // hs is stack memory
     } else {
-        launch_block(ctx, a, nrhs);
+        if constexpr (P::ID == 32) {
+            if (plain && (st = block_plain32(ctx, a, nrhs))) return st;
+        }
+        if (P::ID != 32 || !plain) launch_block(ctx, a, nrhs);
     }
     for (int p = 0; p < 2; p++)
         add_low<P>(ctx, colour_range(ctx, colour, p, nrhs, rs64), rsl, (const E *)el, x, scale_d + nrhs, first, xs);
@@ -314,7 +318,7 @@ static ddrw_status block_solve_dc(ddrw_ctx *ctx, int colour, const MassSet &ms, 
 // x = D_cc(ms)^-1 b on the sites of colour c (FP64 fields, full-field layout, nrhs rhs).
 // Sites of the other colour in x are left untouched.
 ddrw_status block_solve64(ddrw_ctx *ctx, int colour, const MassSet &ms, const double2 *b, double2 *x, int nrhs,
-                          double tol, int maxiter, ddrw_prec prec, SolveStats *stats)
+                          double tol, int maxiter, ddrw_prec prec, SolveStats *stats, bool plain)
 {
     // under the 16-bit precisions the block solves may run in FP32 instead (ddrw_set_low_precision)
     if ((prec == DDRW_MIXED_FP16 || prec == DDRW_MIXED_BF16) && !ctx->block16) prec = DDRW_MIXED_FP32;
@@ -376,7 +380,7 @@ ddrw_status block_solve64(ddrw_ctx *ctx, int colour, const MassSet &ms, const do
             DDRW_CUDA_CHECK(cudaMemcpyAsync(scale_d + nrhs, unscale.data(), sizeof(double) * nrhs, cudaMemcpyHostToDevice,
                                             ctx->stream));
             if (prec == DDRW_MIXED_FP32)
-                st = low_cycle<PrecS>(ctx, colour, ms, rhs, x, first, nrhs, w, scale_d, tol_inner, maxiter, stat, xs);
+                st = low_cycle<PrecS>(ctx, colour, ms, rhs, x, first, nrhs, w, scale_d, tol_inner, maxiter, stat, xs, nullptr, plain);
             else if (prec == DDRW_MIXED_FP16)
                 st = low_cycle<PrecH>(ctx, colour, ms, rhs, x, first, nrhs, w, scale_d, tol_inner, maxiter, stat, xs);
             else

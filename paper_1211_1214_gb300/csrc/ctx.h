@@ -367,8 +367,9 @@ ddrw_status split_copy(ddrw_ctx *ctx, long rs, int nrhs, float4 **xs);
 // x = D_cc(ms)^-1 b on the sites of colour c (persistent block solver + FP64 defect correction)
 // device buffers of the device-controlled block solve (to allocate before a capture)
 ddrw_status block_solve_dc_prepare(ddrw_ctx *ctx, int nrhs);
+// (plain: the FP32 inner solves by the one-CTA kernel of blockplain.cu)
 ddrw_status block_solve64(ddrw_ctx *ctx, int colour, const MassSet &ms, const double2 *b, double2 *x, int nrhs,
-                          double tol, int maxiter, ddrw_prec prec, SolveStats *stats);
+                          double tol, int maxiter, ddrw_prec prec, SolveStats *stats, bool plain = false);
 // x = D(ms)^-1 b on the full lattice (even-odd BiCGStab + FP64 defect correction)
 // device buffers of the device-controlled outer solve (to allocate before a capture)
 ddrw_status full_solve_dc_prepare(ddrw_ctx *ctx, int nrhs);

@@ -134,3 +134,18 @@ def test_residuals_with_a_zero_right_hand_side(dims, l, prec):
             assert np.linalg.norm(y[r] - b[r]) <= (1e-10 + 1e-14) * np.linalg.norm(b[r])
         assert np.max(np.abs(x[1])) == 0.0
     ctx.close()
+
+
+@pytest.mark.parametrize("dims,l,n", [((4, 4, 4, 8), 2, 3), ((8, 8, 8, 8), 4, 1), ((12, 12, 12, 12), 6, 2), ((16, 16, 16, 16), 8, 1)])
+def test_force_block_solves_of_every_length(dims, l, n):
+    """The force with FP32 inner solves against FP64 ones: block residuals of 1e-12, magnified by 1 / (m1 - m2) = 20 and
+    a condition number of order ten."""
+    ctx = context(dims, l)
+    dU = []
+    for prec, tol in ((binding.MIXED_FP32, 1e-12), (binding.FP64, 1e-13)):
+        ctx.set_solver(prec, tol_outer=1e-11, tol_block=tol)
+        u = torch.empty((int(np.prod(dims)), 4, 8), dtype=torch.float64, device="cuda")
+        ctx.force(n, seed=5, dU=u)
+        dU.append(u.clone())
+    assert rel(dU[0], dU[1]) <= 1e-9
+    ctx.close()
