@@ -167,19 +167,21 @@ static void fill_inverse(ddrw_ctx *ctx, MassInv &mi)
     build_inverse(ctx, mi.m, mi);
     f32_to_low(ctx, mi.A32, mi.A16, 18L * ctx->V, false);
     f32_to_low(ctx, mi.A32, mi.Ab16, 18L * ctx->V, true);
-    mi.stale = false;
+}
+
+static void free_inverse(MassInv &mi)
+{
+    cudaFree(mi.A64);
+    cudaFree(mi.A32);
+    cudaFree(mi.A16);
+    cudaFree(mi.Ab16);
 }
 
 ddrw_status mass_inverse(ddrw_ctx *ctx, double m, MassInv **out)
 {
     for (auto &mi : ctx->inv)
         if (mi.m == m) {
-            if (mi.stale) {
-                if (ctx->devctl) return set_error(ctx, DDRW_ESTATE, "in-block inverse to be rebuilt during capture");
-                fill_inverse(ctx, mi);
-                DDRW_CUDA_CHECK(cudaGetLastError());
-            }
-            mi.used = true;
+            mi.asked = true;
             *out = &mi;
             return DDRW_OK;
         }
@@ -190,15 +192,12 @@ ddrw_status mass_inverse(ddrw_ctx *ctx, double m, MassInv **out)
     if (e == cudaSuccess) e = cudaMalloc(&mi.A16, sizeof(uint2) * 18 * (size_t)ctx->V);
     if (e == cudaSuccess) e = cudaMalloc(&mi.Ab16, sizeof(uint2) * 18 * (size_t)ctx->V);
     if (e != cudaSuccess) {
-        cudaFree(mi.A64);
-        cudaFree(mi.A32);
-        cudaFree(mi.A16);
-        cudaFree(mi.Ab16);
+        free_inverse(mi);
         return set_cuda_error(ctx, e, "cudaMalloc(in-block inverse)", __FILE__, __LINE__);
     }
     fill_inverse(ctx, mi);
     DDRW_CUDA_CHECK(cudaGetLastError());
-    mi.used = true;
+    mi.asked = true;
     ctx->inv.push_back(mi);
     *out = &ctx->inv.back();
     return DDRW_OK;
@@ -207,12 +206,7 @@ ddrw_status mass_inverse(ddrw_ctx *ctx, double m, MassInv **out)
 static void free_inverses(ddrw_ctx *ctx)
 {
     clear_graphs(ctx);
-    for (auto &mi : ctx->inv) {
-        cudaFree(mi.A64);
-        cudaFree(mi.A32);
-        cudaFree(mi.A16);
-        cudaFree(mi.Ab16);
-    }
+    for (auto &mi : ctx->inv) free_inverse(mi);
     ctx->inv.clear();
 }
 
@@ -738,19 +732,30 @@ static ddrw_status rebuild(ddrw_ctx *ctx)
     split64(ctx, ctx->U64, ctx->Udd, ctx->V, 0, 0, ctx->V, 0, 1, 3, 12L * ctx->V);
     split64(ctx, ctx->C64, ctx->Cdd, ctx->V, 0, 0, ctx->V, 0, 1, 3, 12L * ctx->V);
     // in-block inverses of the masses already in use: recomputed in place, so that the captured
-    // graphs, which hold their addresses, stay valid; a long list of masses is dropped instead
+    // graphs, which hold their addresses, stay valid; a long list of masses is dropped instead, and so is a
+    // mass that no call asked for and that is no longer the context's (the 0 of a field loaded before the
+    // parameters: 32x16^3 load + first operator application 2.9 -> 2.5 ms)
     if (ctx->inv.size() > (size_t)MAXM + 2) free_inverses(ctx);
-    for (auto &mi : ctx->inv) {
-        if (mi.used || mi.m == ctx->m1 || mi.m == ctx->m2) fill_inverse(ctx, mi);
-        else mi.stale = true;
+    const double own[2] = {ctx->m1, ctx->m2};
+    for (size_t k = 0; k < ctx->inv.size();) {
+        MassInv &mi = ctx->inv[k];
+        if (mi.asked || mi.m == own[0] || mi.m == own[1]) {
+            fill_inverse(ctx, mi);
+            k++;
+        } else {
+            free_inverse(mi);
+            ctx->inv.erase(ctx->inv.begin() + k);
+        }
     }
-    MassInv *mi;
-    ddrw_status st = mass_inverse(ctx, ctx->m1, &mi);
-    if (st) return st;
-    if (ctx->m2 != ctx->m1) st = mass_inverse(ctx, ctx->m2, &mi);
-    if (st) return st;
-    for (auto &e : ctx->inv) e.used = false;  // (the context's masses are kept up to date by their values)
-    st = sync(ctx);
+    for (double m : own) {
+        bool have = false;
+        for (auto &e : ctx->inv) have = have || e.m == m;
+        MassInv *mi;
+        ddrw_status st = have ? DDRW_OK : mass_inverse(ctx, m, &mi);
+        if (st) return st;
+        if (!have) mi->asked = false;
+    }
+    ddrw_status st = sync(ctx);
     ctx->built = st == DDRW_OK;
     return st;
 }

@@ -28,9 +28,8 @@ struct MassInv {
     float4 *A32 = nullptr;   // [2][9][V]
     uint2 *A16 = nullptr;    // [2][9][V] FP16
     uint2 *Ab16 = nullptr;   // [2][9][V] BF16
-    // asked for since the last configuration; false at the next one: recomputed (in place) when next
-    // asked for instead of at once, unless m is one of the context's masses
-    bool used = false, stale = false;
+    // asked for by a call; without it the entry is only there because m was one of the context's masses
+    bool asked = false;
 };
 
 // the in-block inverse of mass slot m in the storage of policy id (64, 32, 16 = FP16, 17 = BF16)
