@@ -138,7 +138,9 @@ ddrw_status ddrw_set_max_rhs(ddrw_ctx *ctx, int max_rhs);
  * threads for 4^4 blocks, three of 224 for 6^4, four of 512 for 8^4), form 1 or 2 the smallest (four of
  * 32, six of 128, eight of 256: more CTAs where a small lattice has few blocks; 2^4 blocks have one
  * shape), form 2 in FP64 with 4^4 blocks eight threads per site (four CTAs of 256).  -1 (the
- * default): the first launch of each shape times them on its real arguments and keeps the fastest.  Same results in every form to the solver's tolerance.  DDRW_EINVAL outside -1..2. */
+ * default): a fixed rule in the storage precision and the numbers of blocks and right-hand sides, the same in
+ * every context.  The forms agree to the solver's tolerance, not bit for bit.  DDRW_EINVAL outside
+ * -1..2. */
 ddrw_status ddrw_block_config(ddrw_ctx *ctx, int form);
 
 /* The 16-bit storage precisions (DDRW_MIXED_FP16, DDRW_MIXED_BF16).  reliable_updates != 0 (the
@@ -331,8 +333,7 @@ ddrw_status ddrw_use_graphs(ddrw_ctx *ctx, int enable, long *graph_launches);
  * (unrolled, rolled, batched loads, register caps, neighbour table) with CUDA events and keeps the fastest.  Tuned choices are
  * also kept for the process, by device and lattice geometry, and reused by later contexts of the
  * same geometry.  enable = 0 uses a fixed choice; either call clears the tuned tables of the context
- * and of the process.  The report lists the tuned shapes, one per line, and the launch shapes the
- * persistent block solver chose (ddrw_block_config). */
+ * and of the process.  The report lists the tuned shapes, one per line. */
 ddrw_status ddrw_autotune(ddrw_ctx *ctx, int enable);
 ddrw_status ddrw_autotune_report(ddrw_ctx *ctx, char *buf, long len);
 

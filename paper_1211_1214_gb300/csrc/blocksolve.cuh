@@ -456,7 +456,7 @@ __global__ void __launch_bounds__(NT, sizeof(typename P::R) == 4 ? 512 / NT : 1)
 // 8 of a warp's 32 lanes.  Here lane u does hop u, then its share of spin u & 3; the Krylov vectors stay in
 // registers for the whole solve (lane (al, q) owns colours 0, 1 of spin al for q = 0, colour 2 for q = 1).
 // ms per launch of a colour, one thread per site / split: 8^4 in 4^4 blocks, 4 right-hand sides 3.47 / 1.42,
-// 16 right-hand sides 3.64 / 5.58, 16^4, 4 right-hand sides 13.1 / 20.5 (the tuner chooses).
+// 16 right-hand sides 3.64 / 5.58, 16^4, 4 right-hand sides 13.1 / 20.5 (block_form chooses).
 template <int BL, int C> struct SplitShape {
     static constexpr int HL = BlockShape<BL>::VBH / C, NT = 8 * HL;
     static constexpr size_t SMEM = (size_t)HL * (2 * 12 + 48) * sizeof(double2);  // G, T, the half spinors
@@ -728,27 +728,45 @@ __global__ void __launch_bounds__(SplitShape<BL, C>::NT) k_block_split(GeomDev g
 // Launch shapes: C CTAs of NT threads per block and right-hand side.  Form 0 is the wider CTA, form 1 the
 // smaller one (more CTAs for few blocks and right-hand sides, more distributed-memory hops).
 // Measured on FP32 storage, ms per launch of a colour, form 0 / form 1 / the kernel with its vectors in
-// global memory: 24x12^3 in 6^4 blocks, 5 right-hand sides 0.43 / 0.45 / 1.07; 16^4 in 4^4 blocks, 16
-// right-hand sides 0.97 / 1.80 / 1.54; 32x16^3 in 8^4 blocks, 18 right-hand sides 4.4 / 5.1 / 7.0;
-// 48x24^3 in 6^4 blocks, 6 right-hand sides 6.3 / 7.2 / 9.1; 64x32^3 in 8^4 blocks, 4 right-hand sides
-// 15.5 / 17.9 / 25.2.  What bounds it now is L2: 1.9 MB of links, clover terms and own-site vectors per
-// CTA and iteration in 38 us (8^4 blocks), 7.6 of the chip's 9.7 TB/s.  Two or four right-hand sides in
-// a CTA, to share the links through L1, lost (22.8 ms on 64x32^3): their barriers couple them.
+// global memory: 24x12^3 in 6^4 blocks, 5 right-hand sides 0.38 / 0.40 / 1.07; 16^4 in 4^4 blocks, 16
+// right-hand sides 0.85 / 1.57 / 1.54; 32x16^3 in 8^4 blocks, 24 right-hand sides 5.5 / 6.2; 48x24^3 in 6^4
+// blocks, 6 right-hand sides 5.8 / 6.3 / 9.1.  What bounds it now is L2: 1.9 MB of links, clover terms
+// and own-site vectors per CTA and iteration (8^4 blocks).  Two or four right-hand sides in
+// a CTA, to share the links through L1, lost (22.8 ms on 64x32^3, 4 right-hand sides, against 15.5): their
+// barriers couple them.
 template <int BL> struct BlkForms;
 template <> struct BlkForms<2> { static constexpr int C[2] = {1, 1}, N[2] = {32, 32}; };
 template <> struct BlkForms<4> { static constexpr int C[2] = {1, 4}, N[2] = {128, 32}; };
 template <> struct BlkForms<6> { static constexpr int C[2] = {3, 6}, N[2] = {224, 128}; };
 template <> struct BlkForms<8> { static constexpr int C[2] = {4, 8}, N[2] = {512, 256}; };
 
+// The form of a launch of n clusters (blocks of a colour times right-hand sides): a rule on sizes, so that every
+// context, captured or not, adds in the same order and no launch is spent on timing.  One GB300, ms
+// per launch with near-unit links.
+//   * 4^4 blocks, 32- and 16-bit storage: form 0 at every size (8 clusters 0.149 / 0.191, 2048 0.85 / 1.57).
+//   * 6^4 and 8^4, 32- and 16-bit: form 1 while its CTAs have SMs to themselves (6^4: 8 clusters 0.315 / 0.291, 16 0.300 /
+//     0.284, 24 0.314 / 0.316; 8^4: 8 0.518 / 0.456, 16 0.537 / 0.524, 24 0.553 / 0.587), then form 0 (at most
+//     3 % behind in FP32, 7 % in 16-bit storage, where its last wave is short).
+//   * FP64, where a CTA has an SM to itself and a launch takes whole waves of clusters.  6^4: form 0 runs 45
+//     clusters per wave of 7.9 ms, form 1 22 of 4.5 (16 clusters 8.2 / 5.0, 40 8.2 / 9.2, 64 15.9 / 13.4, 80 16.2 /
+//     18.6); 8^4: 34 of 22.5 ms and 15 of 11.4 (8 clusters 23.0 / 11.9, 32 23.1 / 34.3, 40 44.7 / 34.7).
+//     4^4: eight lanes per site (form 2) take waves of 36 clusters of 1.3 ms, form 0 of 152 of 3.3 (64
+//     clusters 3.29 / 2.61, 80 3.46 / 3.79); form 1, four CTAs of a warp, fills the SMs that form 0's second wave
+//     leaves idle (160 clusters 6.0 / 5.0, 192 6.0 to 6.2 / 5.4 to 5.7, 256 6.2 / 7.3 to 7.9).
+inline int block_form(int id, int bl, long n)
+{
+    if (bl == 2) return 0;
+    if (id != 64) return bl != 4 && n <= 16;
+    if (bl == 4) return n <= 72 ? 2 : n > 152 && n <= 200 ? 1 : 0;
+    const long per0 = bl == 6 ? 45 : 34, per1 = bl == 6 ? 22 : 15;
+    const double t0 = bl == 6 ? 7.9 : 22.5, t1 = bl == 6 ? 4.5 : 11.4;
+    return t1 * (double)((n + per1 - 1) / per1) < t0 * (double)((n + per0 - 1) / per0);
+}
+
 template <class P>
 void launch_clusters(ddrw_ctx *ctx, void (*kernel)(GeomDev, BlkArgs<P>), int C, int NT, size_t smem, const BlkArgs<P> &a,
-                     int nrhs, bool load)
+                     int nrhs)
 {
-    if (load) {  // have the kernel on the device without running it
-        cudaFuncAttributes fa;
-        cudaFuncGetAttributes(&fa, (const void *)kernel);
-        return;
-    }
     BlkArgs<P> b = a;
     b.nrhs = nrhs;
     if (smem > 40 * 1024)  // (static shared memory counts towards the default limit of 48 KB)
@@ -770,71 +788,30 @@ void launch_clusters(ddrw_ctx *ctx, void (*kernel)(GeomDev, BlkArgs<P>), int C, 
 }
 
 template <class P, int BL, int C, int NT>
-void launch_block_shape(ddrw_ctx *ctx, const BlkArgs<P> &a, int nrhs, bool load)
+void launch_block_shape(ddrw_ctx *ctx, const BlkArgs<P> &a, int nrhs)
 {
-    launch_clusters<P>(ctx, k_block_solve<P, BL, C, NT>, C, NT, BlkShape<P, BL, C>::SMEM, a, nrhs, load);
+    launch_clusters<P>(ctx, k_block_solve<P, BL, C, NT>, C, NT, BlkShape<P, BL, C>::SMEM, a, nrhs);
 }
 
-// The first launch of each (storage, block length, right-hand sides) shape times the forms on the real
-// arguments -- the kernel reads b and overwrites all of x, so a repeat gives the same result --
-// and keeps the fastest.  The kernels are loaded before the first event: a load that fell between the
-// events (a kernel's first launch in the process) once made the form that takes 1572 us win over 846.
 template <class P, int BL>
 void launch_block_kernel(ddrw_ctx *ctx, const BlkArgs<P> &a, int nrhs)
 {
     using F = BlkForms<BL>;
-    // FP64 solves of 4^4 blocks have the split kernel as a third form, those of 2^4 blocks as the only one
-    constexpr bool SPLIT = P::ID == 64 && BL == 4;
-    constexpr int NF = BL == 2 ? 1 : SPLIT ? 3 : 2;
-    const int kind = P::ID == 64 ? PROF_BLOCK64 : P::ID == 32 ? PROF_BLOCK32 : PROF_BLOCK16;
-    auto run = [&](int form, bool load = false) {
-        if constexpr (P::ID == 64 && BL == 2) {
-            launch_clusters<P>(ctx, k_block_split<2, 1>, 1, SplitShape<2, 1>::NT, SplitShape<2, 1>::SMEM, a, nrhs, load);
-        } else {
-            if constexpr (SPLIT) {
-                if (form == 2) {
-                    launch_clusters<P>(ctx, k_block_split<4, 4>, 4, SplitShape<4, 4>::NT, SplitShape<4, 4>::SMEM, a, nrhs, load);
-                    return;
-                }
+    // pinned (ddrw_block_config), else by size
+    const int form = ctx->blk_form >= 0 ? ctx->blk_form : block_form(P::ID, BL, (long)ctx->nblk_c * nrhs);
+    ProfScope ps(ctx, P::ID == 64 ? PROF_BLOCK64 : P::ID == 32 ? PROF_BLOCK32 : PROF_BLOCK16, 0.0);
+    if constexpr (P::ID == 64 && BL == 2) {
+        launch_clusters<P>(ctx, k_block_split<2, 1>, 1, SplitShape<2, 1>::NT, SplitShape<2, 1>::SMEM, a, nrhs);
+    } else {
+        if constexpr (P::ID == 64 && BL == 4) {
+            if (form == 2) {
+                launch_clusters<P>(ctx, k_block_split<4, 4>, 4, SplitShape<4, 4>::NT, SplitShape<4, 4>::SMEM, a, nrhs);
+                return;
             }
-            if (NF > 1 && form) launch_block_shape<P, BL, F::C[1], F::N[1]>(ctx, a, nrhs, load);
-            else launch_block_shape<P, BL, F::C[0], F::N[0]>(ctx, a, nrhs, load);
         }
-    };
-    int form = 0;
-    if (NF > 1) {
-        const std::array<int, 3> key = {P::ID, BL, nrhs};
-        auto it = ctx->blk_tune.find(key);
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        cudaStreamIsCapturing(ctx->stream, &cs);
-        if (ctx->blk_form >= 0) {
-            form = ctx->blk_form;  // pinned (ddrw_block_config)
-        } else if (it != ctx->blk_tune.end()) {
-            form = it->second;
-        } else if (ctx->autotune && cs == cudaStreamCaptureStatusNone && a.b != a.x) {
-            cudaEvent_t e[NF + 1];
-            for (auto &ev : e) cudaEventCreate(&ev);
-            for (int f = 0; f < NF; f++) run(f, true);
-            cudaEventRecord(e[0], ctx->stream);
-            for (int f = 0; f < NF; f++) {
-                run(f);
-                cudaEventRecord(e[f + 1], ctx->stream);
-            }
-            cudaEventSynchronize(e[NF]);
-            float best = 0;
-            for (int f = 0; f < NF; f++) {
-                float ms = 0;
-                cudaEventElapsedTime(&ms, e[f], e[f + 1]);
-                if (f == 0 || ms < best) best = ms, form = f;
-            }
-            for (auto &ev : e) cudaEventDestroy(ev);
-            if (cudaGetLastError() != cudaSuccess) form = 0;
-            ctx->blk_tune[key] = form;
-            cudaMemsetAsync(a.stat, 0, 2 * sizeof(int), ctx->stream);  // the timing runs counted too
-        }
+        if (BL > 2 && form) launch_block_shape<P, BL, F::C[1], F::N[1]>(ctx, a, nrhs);
+        else launch_block_shape<P, BL, F::C[0], F::N[0]>(ctx, a, nrhs);
     }
-    ProfScope ps(ctx, kind, 0.0);
-    run(form);
 }
 
 }  // namespace ddrw

@@ -151,7 +151,6 @@ ddrw_status ddrw_autotune(ddrw_ctx *ctx, int enable)
     if (!ctx) return DDRW_EINVAL;
     ctx->autotune = enable != 0;
     ctx->tune.clear();
-    ctx->blk_tune.clear();
     {
         std::lock_guard<std::mutex> lock(g_tune_mutex);
         g_tune.clear();
@@ -199,12 +198,6 @@ ddrw_status ddrw_autotune_report(ddrw_ctx *ctx, char *buf, long len)
                  "fp%d l=%d npar=%d nrhs=%d diag=%d post=%d rpm=%d hop=%d sel=%d -> nr=%d nt=%d nw=%d roll=%d ms=%.4f\n",
                  k[0], k[1], k[2], k[3], k[4] & 3, k[5], k[6], k[7] & 1, k[7] >> 1, kv.second.nr, kv.second.nt, kv.second.nw,
                  kv.second.roll, kv.second.ms);
-        s += line;
-    }
-    for (auto &kv : ctx->blk_tune) {  // persistent block solver: key (storage, l, nrhs)
-        char line[120];
-        snprintf(line, sizeof line, "block fp%d l=%d nrhs=%d -> form=%d\n", kv.first[0], kv.first[1], kv.first[2],
-                 kv.second);
         s += line;
     }
     if ((long)s.size() + 1 > len) return set_error(ctx, DDRW_EINVAL, "report buffer too small");

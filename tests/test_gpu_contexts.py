@@ -42,3 +42,25 @@ def test_inverses_of_a_used_mass_are_made_by_load_gauge(m):
     ctx.apply_D(m, x, y)
     assert np.linalg.norm(y - b) <= 1.01e-11 * np.linalg.norm(b)
     ctx.close()
+
+
+@pytest.mark.parametrize("dims,l,nrhs", [((8, 8, 8, 8), 4, 4), ((12, 12, 12, 12), 6, 1), ((16, 16, 16, 16), 8, 1)])
+@pytest.mark.parametrize("prec", [binding.FP64, binding.MIXED_FP32])
+def test_block_solves_have_the_same_bits_in_every_context(dims, l, nrhs, prec):
+    """Two contexts, one of them with the autotuner off, give the same bits: the block solver's launch shape follows
+    from the sizes (these have few blocks, where the shapes differ most)."""
+    b = torch.from_numpy(synth.spinor_field(dims, seed=21, nrhs=nrhs)).cuda()
+    xs = []
+    for tune in (True, False, True):
+        ctx = context(dims, l)
+        if not tune:
+            ctx.autotune(False)
+        ctx.set_solver(prec, tol_outer=1e-10, tol_block=1e-12)
+        for colour in (0, 1):
+            x = torch.zeros_like(b)
+            torch.cuda.synchronize()
+            ctx.solve_block(colour, 0.07, b, x, nrhs=nrhs)
+            xs.append(x)
+        ctx.close()
+    for k in (2, 3, 4, 5):
+        assert torch.equal(xs[k], xs[k % 2])
