@@ -128,10 +128,14 @@ __global__ void __launch_bounds__(NT) k_bicg_s(VecArgs<P> va, typename P::SElem 
     });
 }
 
-// omega = (t, s) / (t, t) and, from the same pass over t, s and rh, the next direction's scalars:
-// rho' = (rh, s - omega t) = (rh, s) - omega (rh, t), beta = (rho' alpha) / (rho omega).  With beta
-// known here, the updates of x, r and p need one kernel (k_bicg_xrp) instead of two that
-// read and write r twice: 16 passes over a vector and 4 vector kernels per iteration, not 18 and 5.
+// omega = (t, s) / (t, t) and, from the same pass over t, s and rh, the next direction's beta = (rho' alpha) /
+// (rho omega) with rho' = (rh, s - omega t) = (rh, s) - omega (rh, t).  With beta known here, the updates of
+// x, r and p need one kernel (k_bicg_xrp) instead of two that read and write r twice: 17 passes over a
+// vector and 4 vector kernels per iteration, not 18 and 5.  The difference is rounded relative to |s|, which
+// exceeds |r| where BiCGStab stagnates, so the rho that the next alpha divides by is the
+// product (rh, r) itself, from the kernel that forms r (one pass, 0.4 to 1.4 % of the cases).  With the difference as rho
+// too, FP64 solves of thousands of steps took 1.6 times as many (8^4, m = -0.11, eight fields, geometric
+// mean: (rh, r) in both 4813, in rho 4716, in neither 9540); below 700 steps there is nothing to see.
 // val: (t, s) re, im, (t, t), (rh, s) re, im, (rh, t) re, im
 __device__ __forceinline__ void omega_beta(KScal &s, const double *val)
 {
@@ -148,10 +152,10 @@ __device__ __forceinline__ void omega_beta(KScal &s, const double *val)
     const double2 den = make_double2(s.rho.x * om.x - s.rho.y * om.y, s.rho.x * om.y + s.rho.y * om.x);
     const double d2 = den.x * den.x + den.y * den.y;
     s.omega = om;
-    // a zero denominator ends the recurrence after this iteration's x and r (k_bicg_xrp)
     s.beta = d2 > 0.0 ? make_double2((num.x * den.x + num.y * den.y) / d2, (num.y * den.x - num.x * den.y) / d2)
                       : make_double2(0.0, 0.0);
-    s.rho = d2 > 0.0 ? rn : make_double2(0.0, 0.0);
+    // a zero denominator ends the recurrence after this iteration's x and r (k_bicg_xrp)
+    if (!(d2 > 0.0)) s.rho = make_double2(0.0, 0.0);
 }
 
 template <class P>
@@ -188,12 +192,12 @@ __global__ void __launch_bounds__(NT) k_bicg_omega(VecArgs<P> va, const typename
     if (grid_sum_run<7, NT, R>(sums, val, part, ticket)) omega_beta(sc[blockIdx.y], val);
 }
 
-// x += alpha p + omega s;  r = s - omega t;  p = r + beta (p - omega v);  rr = (r, r)
+// x += alpha p + omega s;  r = s - omega t;  p = r + beta (p - omega v);  rr = (r, r), rho = (rh, r)
 template <class P>
 __global__ void __launch_bounds__(NT, 2) k_bicg_xrp(VecArgs<P> va, typename P::SElem *x, typename P::SElem *p,
                                                     typename P::SElem *r, const typename P::SElem *t,
-                                                    const typename P::SElem *v, KScal *sc, double *part,
-                                                    unsigned *ticket)
+                                                    const typename P::SElem *v, const typename P::SElem *rh, KScal *sc,
+                                                    double *part, unsigned *ticket)
 {
     using R = typename P::R;
     const KScal &s0 = sc[blockIdx.y];
@@ -201,21 +205,23 @@ __global__ void __launch_bounds__(NT, 2) k_bicg_xrp(VecArgs<P> va, typename P::S
     const cpx<R> al = {R(s0.alpha.x), R(s0.alpha.y)}, om = {R(s0.omega.x), R(s0.omega.y)};
     const cpx<R> be = {R(s0.beta.x), R(s0.beta.y)};
     const long rb = (long)blockIdx.y * va.rs;
-    RunSum<R> rr[1];
+    RunSum<R> rr[3];
     for_chunks<P>(va.n, [&](long j, int k) {
-        cpx<R> xv[P::CW], pv[P::CW], sv[P::CW], tv[P::CW], vv[P::CW];
+        cpx<R> xv[P::CW], pv[P::CW], sv[P::CW], tv[P::CW], vv[P::CW], hv[P::CW], z = {R(0), R(0)};
         R b = 0;
         P::ld_chunk(x + rb, va.V, va.off + j, k, xv);
         P::ld_chunk(p + rb, va.V, va.off + j, k, pv);
         P::ld_chunk(r + rb, va.V, va.off + j, k, sv);
         P::ld_chunk(t + rb, va.V, va.off + j, k, tv);
         P::ld_chunk(v + rb, va.V, va.off + j, k, vv);
+        P::ld_chunk(rh + rb, va.V, va.off + j, k, hv);
 #pragma unroll
         for (int q = 0; q < P::CW; q++) {
             cmac(xv[q], al, pv[q]);
             cmac(xv[q], om, sv[q]);
             cmsub(sv[q], om, tv[q]);
             b = fmad(sv[q].re, sv[q].re, fmad(sv[q].im, sv[q].im, b));
+            cmacc(z, hv[q], sv[q]);
             cmsub(pv[q], om, vv[q]);
             tv[q] = sv[q];
             cmac(tv[q], be, pv[q]);
@@ -224,12 +230,15 @@ __global__ void __launch_bounds__(NT, 2) k_bicg_xrp(VecArgs<P> va, typename P::S
         P::st_chunk(r + rb, va.V, va.off + j, k, sv);
         P::st_chunk(p + rb, va.V, va.off + j, k, tv);
         rr[0].add(b);
+        rr[1].add(z.re);
+        rr[2].add(z.im);
     });
-    double val[1];
-    if (grid_sum_run<1, NT, R>(rr, val, part, ticket)) {
+    double val[3];
+    if (grid_sum_run<3, NT, R>(rr, val, part, ticket)) {
         KScal &s = sc[blockIdx.y];
         s.rr = val[0];
         s.iters += 1;
+        if (s.rho.x * s.rho.x + s.rho.y * s.rho.y != 0.0) s.rho = make_double2(val[1], val[2]);
         if (!(val[0] == val[0])) {
             s.breakdown = 3;
             s.active = 0;
@@ -513,7 +522,8 @@ ddrw_status Blas<P>::bicg_omega(ddrw_ctx *ctx, const VecRange &vr, const E *t, c
 }
 
 template <class P>
-ddrw_status Blas<P>::bicg_xrp(ddrw_ctx *ctx, const VecRange &vr, E *x, E *p, E *r, const E *t, const E *v, KScal *sc)
+ddrw_status Blas<P>::bicg_xrp(ddrw_ctx *ctx, const VecRange &vr, E *x, E *p, E *r, const E *t, const E *v, const E *rh,
+                              KScal *sc)
 {
     double *part;
     unsigned *tk;
@@ -522,7 +532,8 @@ ddrw_status Blas<P>::bicg_xrp(ddrw_ctx *ctx, const VecRange &vr, E *x, E *p, E *
     VecArgs<P> va{vr.V, vr.off, vr.n, vr.rs};
     ProfScope ps(ctx, PROF_BLAS, 0.0);
     ++ctx->launches;
-    k_bicg_xrp<P><<<dim3(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(va, x, p, r, t, v, sc, part, tk);
+    k_bicg_xrp<P><<<dim3(grid_for(vr.n, P::NCHUNK, vr.nrhs), vr.nrhs), NT, 0, ctx->stream>>>(va, x, p, r, t, v, rh, sc, part,
+                                                                                         tk);
     return DDRW_OK;
 }
 

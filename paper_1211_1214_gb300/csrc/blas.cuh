@@ -29,7 +29,8 @@ template <class P> struct Blas {
     static ddrw_status bicg_alpha(ddrw_ctx *ctx, const VecRange &vr, const E *rh, const E *v, KScal *sc);
     static void bicg_s(ddrw_ctx *ctx, const VecRange &vr, E *r, const E *v, const KScal *sc);
     static ddrw_status bicg_omega(ddrw_ctx *ctx, const VecRange &vr, const E *t, const E *r, const E *rh, KScal *sc);
-    static ddrw_status bicg_xrp(ddrw_ctx *ctx, const VecRange &vr, E *x, E *p, E *r, const E *t, const E *v, KScal *sc);
+    static ddrw_status bicg_xrp(ddrw_ctx *ctx, const VecRange &vr, E *x, E *p, E *r, const E *t, const E *v, const E *rh,
+                                KScal *sc);
     static ddrw_status norm2(ddrw_ctx *ctx, const VecRange &vr, const E *f, double *out);
     static ddrw_status norm_dot(ddrw_ctx *ctx, const VecRange &vr, const E *d, const E *e, double *out);
     static void axpby(ddrw_ctx *ctx, const VecRange &vr, double a, const E *x, double b, E *y);

@@ -264,20 +264,30 @@ __global__ void __launch_bounds__(NT, sizeof(typename P::R) == 4 ? 512 / NT : 1)
             axpy(acc, R(1), own);
         }
         if (stage == V_OF_P) {
-            RunSum<R> d[2];
+            // (rh, v) and rho = (rh, r): the difference that beta is formed with is rounded relative to |s|
+            RunSum<R> d[4];
+            Spinor<R> s;
             if (act) {
                 Spinor<R> w;
                 P::load_spinor_rw(a.rh + ro, V, se, w);
-                cpx<R> z = {R(0), R(0)};
+                P::load_spinor_rw(a.r + ro, V, se, s);
+                cpx<R> z = {R(0), R(0)}, y = {R(0), R(0)};
 #pragma unroll
-                for (int k = 0; k < 12; k++) cmacc(z, w.v[k / 3][k % 3], acc.v[k / 3][k % 3]);
+                for (int k = 0; k < 12; k++) {
+                    cmacc(z, w.v[k / 3][k % 3], acc.v[k / 3][k % 3]);
+                    cmacc(y, w.v[k / 3][k % 3], s.v[k / 3][k % 3]);
+                }
                 d[0].add(z.re);
                 d[1].add(z.im);
+                d[2].add(y.re);
+                d[3].add(y.im);
                 P::store_spinor(a.v + ro, V, se, acc);
             }
-            double o[2];
-            cluster_totals<2, NT, C, R>(d, o, red, buf, q);
+            double o[4];
+            cluster_totals<4, NT, C, R>(d, o, red, buf, q);
             if (threadIdx.x == 0) {  // alpha = rho / (rh, v); a zero or NaN is a breakdown: x as it is
+                rho_x = o[2];
+                rho_y = o[3];
                 const double den = o[0] * o[0] + o[1] * o[1];
                 live = !(den == 0.0 || !(den == den));
                 const double iv = 1.0 / den;
@@ -293,8 +303,6 @@ __global__ void __launch_bounds__(NT, sizeof(typename P::R) == 4 ? 512 / NT : 1)
             } else {
                 if (act) {  // s = r - alpha v
                     const cpx<R> al = {scal[0], scal[1]};
-                    Spinor<R> s;
-                    P::load_spinor_rw(a.r + ro, V, se, s);
 #pragma unroll
                     for (int k = 0; k < 12; k++) cmsub(s.v[k / 3][k % 3], al, acc.v[k / 3][k % 3]);
                     P::store_spinor(G, HL, hl, s);
@@ -369,7 +377,8 @@ __global__ void __launch_bounds__(NT, sizeof(typename P::R) == 4 ? 512 / NT : 1)
             double o[7];
             cluster_totals<7, NT, C, R>(d, o, red, buf, q);
             if (threadIdx.x == 0) {
-                // omega = (t, s) / (t, t), rho' = (rh, s) - omega (rh, t), beta = rho' alpha / (rho omega)
+                // omega = (t, s) / (t, t), rho' = (rh, s) - omega (rh, t), beta = rho' alpha / (rho omega); a zero
+                // denominator (rho = 0) ends the recurrence after this iteration
                 const double tt = o[2];
                 const bool go = !(tt == 0.0 || !(tt == tt));
                 live = go;
@@ -383,7 +392,7 @@ __global__ void __launch_bounds__(NT, sizeof(typename P::R) == 4 ? 512 / NT : 1)
                 scal[3] = R(oy);
                 scal[4] = R((nx * dx + ny * dy) * jv);
                 scal[5] = R((ny * dx - nx * dy) * jv);
-                rho_x = d2 > 0.0 ? rx : 0.0;  // a zero denominator ends the recurrence after this iteration
+                rho_x = d2 > 0.0 ? rx : 0.0;
                 rho_y = d2 > 0.0 ? ry : 0.0;
             }
             __syncthreads();
@@ -584,18 +593,23 @@ __global__ void __launch_bounds__(SplitShape<BL, C>::NT) k_block_split(GeomDev g
         split_join(o);
         own2(o, e);
         if (stage == V_OF_P) {
-            RunSum<double> d[2];
-            cpx<double> z = {0.0, 0.0};
+            RunSum<double> d[4];  // (rh, v) and rho = (rh, r)
+            cpx<double> z = {0.0, 0.0}, y = {0.0, 0.0};
 #pragma unroll
             for (int k = 0; k < 2; k++) {
                 v[k] = e[k];
                 cmacc(z, rh[k], v[k]);
+                cmacc(y, rh[k], r[k]);
             }
             d[0].s = z.re;
             d[1].s = z.im;
-            double t[2];
-            cluster_totals<2, NT, C, double>(d, t, red, buf, q);
+            d[2].s = y.re;
+            d[3].s = y.im;
+            double t[4];
+            cluster_totals<4, NT, C, double>(d, t, red, buf, q);
             if (threadIdx.x == 0) {  // alpha = rho / (rh, v); a zero or NaN is a breakdown: x as it is
+                rho_x = t[2];
+                rho_y = t[3];
                 const double den = t[0] * t[0] + t[1] * t[1];
                 live = !(den == 0.0 || !(den == den));
                 const double iv = 1.0 / den;

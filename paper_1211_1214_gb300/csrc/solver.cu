@@ -209,7 +209,7 @@ static ddrw_status bicg_iteration(ddrw_ctx *ctx, const MassSet &ms, int nrhs, lo
         apply_mhat<P>(ctx, ms, nrhs, rs, r, tmp, t, colour);
         if ((s2 = Blas<P>::bicg_omega(ctx, ev, t, r, rh, sc))) return s2;
     }
-    return Blas<P>::bicg_xrp(ctx, ev, x, p, r, t, v, sc);
+    return Blas<P>::bicg_xrp(ctx, ev, x, p, r, t, v, rh, sc);
 }
 
 // Inner even-odd BiCGStab in policy P: solve D x = b (full fields) until the even-odd residual of

@@ -64,3 +64,20 @@ def test_block_solves_have_the_same_bits_in_every_context(dims, l, nrhs, prec):
         ctx.close()
     for k in (2, 3, 4, 5):
         assert torch.equal(xs[k], xs[k % 2])
+
+
+def test_hard_fp64_solves_keep_their_step_counts():
+    """Solves of thousands of BiCGStab steps (a mass beyond the critical one), where ||s|| exceeds ||r|| by orders of
+    magnitude and an inner product known only relative to ||s|| costs steps.  Steps of sixteen solves: 122e3 with
+    rho and beta from (rh, r), 85e3 with rho alone from it, 174e3 with both from (rh, s) - omega (rh, t); the bar is
+    halfway between the last two."""
+    dims, steps = (8, 8, 8, 8), 0
+    for seed in range(1, 17):
+        ctx = binding.Context(dims, (4,) * 4)
+        ctx.load_gauge(synth.gauge_field(dims, 0.25, seed=seed))
+        ctx.set_params(1.5, -0.105, -0.11)
+        ctx.set_solver(binding.FP64, tol_outer=1e-11, tol_block=1e-12, maxiter=4000)
+        b = synth.spinor_field(dims, seed=70 + seed)
+        steps += ctx.solve_D(-0.11, b, np.zeros_like(b))["iters_outer"]
+        ctx.close()
+    assert steps <= 130e3
