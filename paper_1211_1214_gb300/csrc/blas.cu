@@ -49,17 +49,17 @@ __global__ void __launch_bounds__(NT) k_bicg_init(VecArgs<P> va, typename P::SEl
     RunSum<R> acc;
     for_chunks<P>(va.n, [&](long j, int k) {
         cpx<R> c[P::CW], z[P::CW];
-        R a = 0;
+        SiteNorm<R> a;
         P::ld_chunk(r + rb, va.V, va.off + j, k, c);
 #pragma unroll
         for (int q = 0; q < P::CW; q++) {
-            a += c[q].re * c[q].re + c[q].im * c[q].im;
+            a.add(q, c[q]);
             z[q] = {R(0), R(0)};
         }
         P::st_chunk(rh + rb, va.V, va.off + j, k, c);
         P::st_chunk(p + rb, va.V, va.off + j, k, c);
         P::st_chunk(x + rb, va.V, va.off + j, k, z);
-        acc.add(a);
+        acc.add(a.total());
     });
     RunSum<R> sums[1] = {acc};
     double v[1];
@@ -83,15 +83,14 @@ __global__ void __launch_bounds__(NT) k_bicg_alpha(VecArgs<P> va, const typename
     const long rb = (long)blockIdx.y * va.rs;
     RunSum<R> are, aim;
     for_chunks<P>(va.n, [&](long j, int k) {
-        cpx<R> c[P::CW], d[P::CW], a = {R(0), R(0)};
+        cpx<R> c[P::CW], d[P::CW];
+        SiteDot<R> a;
         P::ld_chunk(rh + rb, va.V, va.off + j, k, c);
         P::ld_chunk(v + rb, va.V, va.off + j, k, d);
 #pragma unroll
-        for (int q = 0; q < P::CW; q++) {
-            cmacc(a, c[q], d[q]);
-        }
-        are.add(a.re);
-        aim.add(a.im);
+        for (int q = 0; q < P::CW; q++) a.add(q, c[q], d[q]);
+        are.add(a.total().re);
+        aim.add(a.total().im);
     });
     RunSum<R> sums[2] = {are, aim};
     double val[2];
@@ -168,25 +167,26 @@ __global__ void __launch_bounds__(NT) k_bicg_omega(VecArgs<P> va, const typename
     const long rb = (long)blockIdx.y * va.rs;
     RunSum<R> sums[7];
     for_chunks<P>(va.n, [&](long j, int k) {
-        cpx<R> c[P::CW], d[P::CW], h[P::CW], ts = {R(0), R(0)}, hs = {R(0), R(0)}, ht = {R(0), R(0)};
-        R b = 0;
+        cpx<R> c[P::CW], d[P::CW], h[P::CW];
+        SiteDot<R> ts, hs, ht;
+        SiteNorm<R> b;
         P::ld_chunk(t + rb, va.V, va.off + j, k, c);
         P::ld_chunk(r + rb, va.V, va.off + j, k, d);
         P::ld_chunk(rh + rb, va.V, va.off + j, k, h);
 #pragma unroll
         for (int q = 0; q < P::CW; q++) {
-            cmacc(ts, c[q], d[q]);
-            b = fmad(c[q].re, c[q].re, fmad(c[q].im, c[q].im, b));
-            cmacc(hs, h[q], d[q]);
-            cmacc(ht, h[q], c[q]);
+            ts.add(q, c[q], d[q]);
+            b.add(q, c[q]);
+            hs.add(q, h[q], d[q]);
+            ht.add(q, h[q], c[q]);
         }
-        sums[0].add(ts.re);
-        sums[1].add(ts.im);
-        sums[2].add(b);
-        sums[3].add(hs.re);
-        sums[4].add(hs.im);
-        sums[5].add(ht.re);
-        sums[6].add(ht.im);
+        sums[0].add(ts.total().re);
+        sums[1].add(ts.total().im);
+        sums[2].add(b.total());
+        sums[3].add(hs.total().re);
+        sums[4].add(hs.total().im);
+        sums[5].add(ht.total().re);
+        sums[6].add(ht.total().im);
     });
     double val[7];
     if (grid_sum_run<7, NT, R>(sums, val, part, ticket)) omega_beta(sc[blockIdx.y], val);
@@ -207,8 +207,9 @@ __global__ void __launch_bounds__(NT, 2) k_bicg_xrp(VecArgs<P> va, typename P::S
     const long rb = (long)blockIdx.y * va.rs;
     RunSum<R> rr[3];
     for_chunks<P>(va.n, [&](long j, int k) {
-        cpx<R> xv[P::CW], pv[P::CW], sv[P::CW], tv[P::CW], vv[P::CW], hv[P::CW], z = {R(0), R(0)};
-        R b = 0;
+        cpx<R> xv[P::CW], pv[P::CW], sv[P::CW], tv[P::CW], vv[P::CW], hv[P::CW];
+        SiteNorm<R> b;
+        SiteDot<R> z;
         P::ld_chunk(x + rb, va.V, va.off + j, k, xv);
         P::ld_chunk(p + rb, va.V, va.off + j, k, pv);
         P::ld_chunk(r + rb, va.V, va.off + j, k, sv);
@@ -220,8 +221,8 @@ __global__ void __launch_bounds__(NT, 2) k_bicg_xrp(VecArgs<P> va, typename P::S
             cmac(xv[q], al, pv[q]);
             cmac(xv[q], om, sv[q]);
             cmsub(sv[q], om, tv[q]);
-            b = fmad(sv[q].re, sv[q].re, fmad(sv[q].im, sv[q].im, b));
-            cmacc(z, hv[q], sv[q]);
+            b.add(q, sv[q]);
+            z.add(q, hv[q], sv[q]);
             cmsub(pv[q], om, vv[q]);
             tv[q] = sv[q];
             cmac(tv[q], be, pv[q]);
@@ -229,9 +230,9 @@ __global__ void __launch_bounds__(NT, 2) k_bicg_xrp(VecArgs<P> va, typename P::S
         P::st_chunk(x + rb, va.V, va.off + j, k, xv);
         P::st_chunk(r + rb, va.V, va.off + j, k, sv);
         P::st_chunk(p + rb, va.V, va.off + j, k, tv);
-        rr[0].add(b);
-        rr[1].add(z.re);
-        rr[2].add(z.im);
+        rr[0].add(b.total());
+        rr[1].add(z.total().re);
+        rr[2].add(z.total().im);
     });
     double val[3];
     if (grid_sum_run<3, NT, R>(rr, val, part, ticket)) {
@@ -313,11 +314,11 @@ __global__ void __launch_bounds__(NT) k_norm2(VecArgs<P> va, const typename P::S
     RunSum<R> acc;
     for_chunks<P>(va.n, [&](long j, int k) {
         cpx<R> c[P::CW];
-        R a = 0;
+        SiteNorm<R> a;
         P::ld_chunk(f + rb, va.V, va.off + j, k, c);
 #pragma unroll
-        for (int q = 0; q < P::CW; q++) a = fmad(c[q].re, c[q].re, fmad(c[q].im, c[q].im, a));
-        acc.add(a);
+        for (int q = 0; q < P::CW; q++) a.add(q, c[q]);
+        acc.add(a.total());
     });
     RunSum<R> sums[1] = {acc};
     double v[1];
@@ -335,18 +336,19 @@ __global__ void __launch_bounds__(NT) k_norm_dot(VecArgs<P> va, const typename P
     const long rb = (long)blockIdx.y * va.rs;
     RunSum<R> nn, dr, di;
     for_chunks<P>(va.n, [&](long j, int k) {
-        cpx<R> c[P::CW], f[P::CW], a = {R(0), R(0)};
-        R b = 0;
+        cpx<R> c[P::CW], f[P::CW];
+        SiteDot<R> a;
+        SiteNorm<R> b;
         P::ld_chunk(d + rb, va.V, va.off + j, k, c);
         P::ld_chunk(e + rb, va.V, va.off + j, k, f);
 #pragma unroll
         for (int q = 0; q < P::CW; q++) {
-            b = fmad(c[q].re, c[q].re, fmad(c[q].im, c[q].im, b));
-            cmacc(a, c[q], f[q]);
+            b.add(q, c[q]);
+            a.add(q, c[q], f[q]);
         }
-        nn.add(b);
-        dr.add(a.re);
-        di.add(a.im);
+        nn.add(b.total());
+        dr.add(a.total().re);
+        di.add(a.total().im);
     });
     RunSum<R> sums[3] = {nn, dr, di};
     double v[3];

@@ -83,6 +83,28 @@ template <> struct RunSum<float> {
     }
 };
 
+// Sums of products over the components k = 0, 1, ... of a site (unrolled loops), in chains of four: a chain of
+// all twelve, 24 terms deep, rounds 1.25 times as much as adding up |z|^2 or conj(a) b component by component,
+// chains of four 0.8 times (rms error against 64 bits, 128 to 131072 sites), for one more addition per chain.
+template <typename R> struct SiteNorm {
+    R s = R(0), c = R(0);
+    __device__ __forceinline__ void add(int k, cpx<R> z)  // += |z|^2
+    {
+        if (k > 0 && k % 4 == 0) s += c, c = R(0);
+        c = fmad(z.re, z.re, fmad(z.im, z.im, c));
+    }
+    __device__ __forceinline__ R total() const { return s + c; }
+};
+template <typename R> struct SiteDot {
+    cpx<R> s = {R(0), R(0)}, c = {R(0), R(0)};
+    __device__ __forceinline__ void add(int k, cpx<R> a, cpx<R> b)  // += conj(a) b
+    {
+        if (k > 0 && k % 4 == 0) s = s + c, c = {R(0), R(0)};
+        cmacc(c, a, b);
+    }
+    __device__ __forceinline__ cpx<R> total() const { return s + c; }
+};
+
 // Warp totals of K running sums at once: while several sums are left, each exchange step also halves the
 // sums a lane keeps, so K = 7 takes 9 additions per lane instead of 35 (FP64 additions are what these
 // reductions wait for).  Afterwards lane l holds the total of sum l >> SHIFT.

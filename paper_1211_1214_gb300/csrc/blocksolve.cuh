@@ -271,16 +271,16 @@ __global__ void __launch_bounds__(NT, sizeof(typename P::R) == 4 ? 512 / NT : 1)
                 Spinor<R> w;
                 P::load_spinor_rw(a.rh + ro, V, se, w);
                 P::load_spinor_rw(a.r + ro, V, se, s);
-                cpx<R> z = {R(0), R(0)}, y = {R(0), R(0)};
+                SiteDot<R> z, y;
 #pragma unroll
                 for (int k = 0; k < 12; k++) {
-                    cmacc(z, w.v[k / 3][k % 3], acc.v[k / 3][k % 3]);
-                    cmacc(y, w.v[k / 3][k % 3], s.v[k / 3][k % 3]);
+                    z.add(k, w.v[k / 3][k % 3], acc.v[k / 3][k % 3]);
+                    y.add(k, w.v[k / 3][k % 3], s.v[k / 3][k % 3]);
                 }
-                d[0].add(z.re);
-                d[1].add(z.im);
-                d[2].add(y.re);
-                d[3].add(y.im);
+                d[0].add(z.total().re);
+                d[1].add(z.total().im);
+                d[2].add(y.total().re);
+                d[3].add(y.total().im);
                 P::store_spinor(a.v + ro, V, se, acc);
             }
             double o[4];
@@ -316,29 +316,19 @@ __global__ void __launch_bounds__(NT, sizeof(typename P::R) == 4 ? 512 / NT : 1)
         RunSum<R> rr[2];  // ||r||^2 and, at the start, ||b||^2
         if (stage == START) {
             if (act) {
-                R n = 0, nb = 0;
+                SiteNorm<R> n, be2, bo2;
                 Spinor<R> o;
 #pragma unroll
-                for (int k = 0; k < 12; k++) {
-                    const cpx<R> z = acc.v[k / 3][k % 3];
-                    n = fmad(z.re, z.re, fmad(z.im, z.im, n));
-                }
+                for (int k = 0; k < 12; k++) n.add(k, acc.v[k / 3][k % 3]);
                 P::load_spinor(a.b + ro, V, se, o);
 #pragma unroll
-                for (int k = 0; k < 12; k++) {
-                    const cpx<R> z = o.v[k / 3][k % 3];
-                    nb = fmad(z.re, z.re, fmad(z.im, z.im, nb));
-                }
-                rr[1].add(nb);
-                nb = 0;
+                for (int k = 0; k < 12; k++) be2.add(k, o.v[k / 3][k % 3]);
                 P::load_spinor(a.b + ro, V, so, o);
 #pragma unroll
-                for (int k = 0; k < 12; k++) {
-                    const cpx<R> z = o.v[k / 3][k % 3];
-                    nb = fmad(z.re, z.re, fmad(z.im, z.im, nb));
-                }
-                rr[0].add(n);
-                rr[1].add(nb);
+                for (int k = 0; k < 12; k++) bo2.add(k, o.v[k / 3][k % 3]);
+                rr[0].add(n.total());
+                rr[1].add(be2.total());
+                rr[1].add(bo2.total());
                 P::store_spinor(a.r + ro, V, se, acc);
                 P::store_spinor(a.rh + ro, V, se, acc);
                 P::store_spinor(a.p + ro, V, se, acc);
@@ -351,28 +341,28 @@ __global__ void __launch_bounds__(NT, sizeof(typename P::R) == 4 ? 512 / NT : 1)
             if (act) {
                 Spinor<R> w;
                 P::load_spinor_rw(G, HL, hl, w);
-                cpx<R> ts = {R(0), R(0)}, hs = {R(0), R(0)}, ht = {R(0), R(0)};
-                R tt = 0;
+                SiteDot<R> ts, hs, ht;
+                SiteNorm<R> tt;
 #pragma unroll
                 for (int k = 0; k < 12; k++) {
                     const cpx<R> z = acc.v[k / 3][k % 3];
-                    cmacc(ts, z, w.v[k / 3][k % 3]);
-                    tt = fmad(z.re, z.re, fmad(z.im, z.im, tt));
+                    ts.add(k, z, w.v[k / 3][k % 3]);
+                    tt.add(k, z);
                 }
                 Spinor<R> hh;
                 P::load_spinor_rw(a.rh + ro, V, se, hh);
 #pragma unroll
                 for (int k = 0; k < 12; k++) {
-                    cmacc(hs, hh.v[k / 3][k % 3], w.v[k / 3][k % 3]);
-                    cmacc(ht, hh.v[k / 3][k % 3], acc.v[k / 3][k % 3]);
+                    hs.add(k, hh.v[k / 3][k % 3], w.v[k / 3][k % 3]);
+                    ht.add(k, hh.v[k / 3][k % 3], acc.v[k / 3][k % 3]);
                 }
-                d[0].add(ts.re);
-                d[1].add(ts.im);
-                d[2].add(tt);
-                d[3].add(hs.re);
-                d[4].add(hs.im);
-                d[5].add(ht.re);
-                d[6].add(ht.im);
+                d[0].add(ts.total().re);
+                d[1].add(ts.total().im);
+                d[2].add(tt.total());
+                d[3].add(hs.total().re);
+                d[4].add(hs.total().im);
+                d[5].add(ht.total().re);
+                d[6].add(ht.total().im);
             }
             double o[7];
             cluster_totals<7, NT, C, R>(d, o, red, buf, q);
@@ -408,14 +398,14 @@ __global__ void __launch_bounds__(NT, sizeof(typename P::R) == 4 ? 512 / NT : 1)
                 P::load_spinor_rw(G, HL, hl, s);
                 P::load_spinor_rw(a.p + ro, V, se, pv);
                 P::load_spinor_rw(a.x + ro, V, se, y);
-                R n = 0;
+                SiteNorm<R> n;
 #pragma unroll
                 for (int k = 0; k < 12; k++) {
                     cpx<R> &sk = s.v[k / 3][k % 3], &xk = y.v[k / 3][k % 3];
                     cmac(xk, al, pv.v[k / 3][k % 3]);
                     cmac(xk, om, sk);
                     cmsub(sk, om, acc.v[k / 3][k % 3]);
-                    n = fmad(sk.re, sk.re, fmad(sk.im, sk.im, n));
+                    n.add(k, sk);
                 }
                 P::store_spinor(a.x + ro, V, se, y);
                 P::store_spinor(a.r + ro, V, se, s);
@@ -428,7 +418,7 @@ __global__ void __launch_bounds__(NT, sizeof(typename P::R) == 4 ? 512 / NT : 1)
                 }
                 P::store_spinor(a.p + ro, V, se, s);
                 P::store_spinor(G, HL, hl, s);
-                rr[0].add(n);
+                rr[0].add(n.total());
             }
             it++;
         }
