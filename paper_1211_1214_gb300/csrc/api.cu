@@ -839,6 +839,7 @@ ddrw_status ddrw_block_config(ddrw_ctx *ctx, int form)
 {
     if (!ctx) return DDRW_EINVAL;
     if (form < -1 || form > 2) return set_error(ctx, DDRW_EINVAL, "block-solver launch shape must be -1, 0, 1 or 2");
+    if (ctx->blk_form != form) clear_graphs(ctx);  // captured launches keep the shape they were captured with
     ctx->blk_form = form;
     return DDRW_OK;
 }

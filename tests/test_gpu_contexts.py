@@ -81,3 +81,20 @@ def test_hard_fp64_solves_keep_their_step_counts():
         steps += ctx.solve_D(-0.11, b, np.zeros_like(b))["iters_outer"]
         ctx.close()
     assert steps <= 130e3
+
+
+def test_block_config_reaches_captured_estimates():
+    """A launch shape pinned after an estimate was captured whole is used by the next estimate: the bits of a context
+    on which it was pinned before.  (The shapes add in different orders, so their bits differ.)"""
+    e = {}
+    for forms in ((0, 2), (2,)):
+        ctx = context()
+        ctx.set_solver(binding.FP64, tol_outer=1e-11, tol_block=1e-12)
+        ctx.use_graphs(1)
+        for form in forms:
+            ctx.block_config(form)
+            for _ in range(3):  # eager, captured, replayed
+                e[forms, form] = np.asarray(ctx.estimate(4, seed=5)[0])
+        ctx.close()
+    assert np.array_equal(e[(0, 2), 2], e[(2,), 2])
+    assert not np.array_equal(e[(0, 2), 0], e[(0, 2), 2])
