@@ -156,12 +156,12 @@ ddrw_status ddrw_block_config(ddrw_ctx *ctx, int form);
  * mode 1) use the plain form. */
 ddrw_status ddrw_set_low_precision(ddrw_ctx *ctx, int reliable_updates, int block_solves_16bit);
 
-/* With enable != 0 the FP32 even-odd BiCGStab of the full-lattice solves computes the inner
+/* With enable > 0 the FP32 even-odd BiCGStab of the full-lattice solves computes the inner
  * products of alpha = rho / (rh, v) and omega = (t, s) / (t, t) in the epilogue of the stencil launch
  * that writes v and t (one partial per warp of 32 sites, summed in a fixed order by a small kernel)
  * instead of re-reading v, t and s in separate reductions; with 0 it uses the separate reduction
- * kernels.  A context on which this was never called chooses by size (the fused form on small
- * lattices with few right-hand sides).  Results differ only by the rounding of the sums. */
+ * kernels; a negative value (the state of a new context) chooses by size, the fused form on small
+ * lattices with few right-hand sides.  Results differ only by the rounding of the sums. */
 ddrw_status ddrw_fuse_reductions(ddrw_ctx *ctx, int enable);
 
 /* How the block solves D_cc(m)^-1 of the mixed precisions run (Eq. 1; the four solves of r and the

@@ -342,8 +342,10 @@ class Context:
         self._check(self.L.ddrw_block_config(self._h, int(form)), "ddrw_block_config")
 
     def fuse_reductions(self, enable=True):
-        """Inner products of the BiCGStab recurrence in the stencil epilogue (True) or separate kernels."""
-        self._check(self.L.ddrw_fuse_reductions(self._h, int(bool(enable))), "ddrw_fuse_reductions")
+        """Inner products of the BiCGStab recurrence in the stencil epilogue (True), in separate kernels (False) or
+        by size as in a new context (-1)."""
+        self._check(self.L.ddrw_fuse_reductions(self._h, -1 if enable == -1 else int(bool(enable))),
+                    "ddrw_fuse_reductions")
 
     def set_block_solver(self, method):
         """Block solves of the mixed precisions: 0 persistent kernel, 1 Krylov-loop BiCGStab."""

@@ -856,7 +856,7 @@ ddrw_status ddrw_set_low_precision(ddrw_ctx *ctx, int reliable_updates, int bloc
 ddrw_status ddrw_fuse_reductions(ddrw_ctx *ctx, int enable)
 {
     if (!ctx) return DDRW_EINVAL;
-    ctx->fuse_dots = enable != 0 ? 1 : 0;
+    ctx->fuse_dots = enable < 0 ? -1 : enable != 0 ? 1 : 0;
     clear_graphs(ctx);  // captured iterations keep the kernels they were captured with
     return DDRW_OK;
 }

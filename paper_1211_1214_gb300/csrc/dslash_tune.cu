@@ -195,8 +195,8 @@ ddrw_status ddrw_autotune_report(ddrw_ctx *ctx, char *buf, long len)
         const auto &k = kv.first;
         char line[200];
         snprintf(line, sizeof line,
-                 "fp%d l=%d npar=%d nrhs=%d diag=%d post=%d rpm=%d hop=%d sel=%d -> nr=%d nt=%d nw=%d roll=%d ms=%.4f\n",
-                 k[0], k[1], k[2], k[3], k[4] & 3, k[5], k[6], k[7] & 1, k[7] >> 1, kv.second.nr, kv.second.nt, kv.second.nw,
+                 "fp%d l=%d npar=%d nrhs=%d diag=%d red=%d post=%d rpm=%d hop=%d sel=%d -> nr=%d nt=%d nw=%d roll=%d ms=%.4f\n",
+                 k[0], k[1], k[2], k[3], k[4] & 3, k[4] >> 2, k[5], k[6], k[7] & 1, k[7] >> 1, kv.second.nr, kv.second.nt, kv.second.nw,
                  kv.second.roll, kv.second.ms);
         s += line;
     }

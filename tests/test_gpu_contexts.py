@@ -98,3 +98,22 @@ def test_block_config_reaches_captured_estimates():
         ctx.close()
     assert np.array_equal(e[(0, 2), 2], e[(2,), 2])
     assert not np.array_equal(e[(0, 2), 0], e[(0, 2), 2])
+
+
+@pytest.mark.parametrize("nrhs,fused", [(1, True), (8, False)])  # 2^15 x 8 sites are beyond the rule's 2^17
+def test_fuse_reductions_returns_to_the_size_rule(nrhs, fused):
+    """After an explicit setting, -1 chooses by size again (the report lists the stencil shapes that ran)."""
+    ctx = context((16, 16, 16, 16))
+    ctx.set_solver(binding.MIXED_FP32, tol_outer=1e-10, tol_block=1e-12)
+    b = torch.from_numpy(synth.spinor_field((16, 16, 16, 16), seed=5, nrhs=nrhs)).cuda()
+    x = torch.zeros_like(b)
+    torch.cuda.synchronize()
+    ran = []
+    for switch in (None, False, True, -1):
+        ctx.autotune(True)  # an empty list of shapes
+        if switch is not None:
+            ctx.fuse_reductions(switch)
+        ctx.solve_D(0.12, b, x, nrhs=nrhs)
+        ran.append("red=2" in ctx.autotune_report())
+    assert ran == [fused, False, True, fused]
+    ctx.close()
