@@ -116,7 +116,7 @@ struct ForceArgs {
     long rs;
     const double2 *U64;
     double2 *omega;  // [6 planes][9][V]
-    double *plaq;    // [6 planes][4 links of the loop][8][V]
+    double *plaq[6]; // per plane [4 links of the loop][8][V]
     double csw;
     double *out;     // [V lexicographic][4][8]
 };
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(128) k_plaq(GeomDev g, ForceArgs a)
     const double f = 0.5 * a.csw / 8.0 * (j < 2 ? -1.0 : 1.0);
     if (s0 < g.V)
 #pragma unroll
-        for (int k = 0; k < 8; k++) a.plaq[(((long)pl * 4 + j) * 8 + k) * g.V + s] = f * tr[k];
+        for (int k = 0; k < 8; k++) a.plaq[pl][((long)j * 8 + k) * g.V + s] = f * tr[k];
 }
 
 // h = (1 + sg g_mu) psi restricted to its two independent spin components, psi_u + sg e_mu psi_d
@@ -360,8 +360,8 @@ __global__ void __launch_bounds__(64) k_force(GeomDev g, ForceArgs a)
             const int pl = al == 0 ? be - 1 : al == 1 ? be + 1 : 5;
             // link 0 of the loop at x and 2 of the one at x - nu (mu = al), 3 at x and 1 at x - nu (mu = be)
             const long sn = shifted(x, g, nu, -1, mu, 0, internal_index<BL>);
-            const double *p0 = a.plaq + ((long)pl * 4 + (mu == al ? 0 : 3)) * 8 * g.V + s;
-            const double *p1 = a.plaq + ((long)pl * 4 + (mu == al ? 2 : 1)) * 8 * g.V + sn;
+            const double *p0 = a.plaq[pl] + (mu == al ? 0L : 3L) * 8 * g.V + s;
+            const double *p1 = a.plaq[pl] + (mu == al ? 2L : 1L) * 8 * g.V + sn;
 #pragma unroll
             for (int k = 0; k < 8; k++) de[k] += p0[(long)k * g.V] + p1[(long)k * g.V];
         }
@@ -527,16 +527,21 @@ extern "C" ddrw_status ddrw_force(ddrw_ctx *ctx, int nhit, uint64_t seed, uint64
     }
     if (dU) {
         double2 *omega;
-        double *plaq;
         if ((st = workspace(ctx, "frc_omega", sizeof(double2) * 54 * V, (void **)&omega))) return st;
-        if ((st = workspace(ctx, "frc_plaq", sizeof(double) * 192 * V, (void **)&plaq))) return st;
+        // the plaquettes' traces, 256 bytes per site and plane, take the place of fields that are done with: four of
+        // the chain's and two of the block solves', each at least 384 bytes per site
+        double *plaq[6] = {(double *)V2, (double *)T1, (double *)T2, (double *)Zf};
+        const size_t pb = sizeof(double) * 32 * V;
+        if ((st = workspace(ctx, "blk_res64", pb, (void **)&plaq[4]))) return st;
+        if ((st = workspace(ctx, ctx->prec == DDRW_FP64 ? "blk_e64" : "ds_split", pb, (void **)&plaq[5]))) return st;
         double *out;
         void *dout;
         bool host;
         size_t ob = sizeof(double) * 32 * V;
         if ((st = stage_out(ctx, dU, ob, "stage_force", &dout, &host))) return st;
         out = (double *)dout;
-        ForceArgs fa{ZT, Q, WT, A, cd, R2, rs, ctx->U64, omega, plaq, ctx->csw, out};
+        ForceArgs fa{ZT, Q, WT, A, cd, R2, rs, ctx->U64, omega, {}, ctx->csw, out};
+        std::copy(plaq, plaq + 6, fa.plaq);
         if (ctx->csw != 0.0) {
             ++ctx->launches;
             k_omega<<<(unsigned)((V + 63) / 64), 64, 0, ctx->stream>>>(V, fa);

@@ -117,3 +117,18 @@ def test_fuse_reductions_returns_to_the_size_rule(nrhs, fused):
         ran.append("red=2" in ctx.autotune_report())
     assert ran == [fused, False, True, fused]
     ctx.close()
+
+
+@pytest.mark.parametrize("prec", [binding.FP64, binding.MIXED_FP32])
+def test_force_scratch(prec):
+    """The link force takes no more device memory beyond the mass derivative's than its six 3x3 matrices per site
+    (864 bytes), the allocator's rounding and the code of its kernels (16 MB for both)."""
+    dims = (16, 16, 16, 16)
+    ctx = context(dims, 8)
+    ctx.set_solver(prec, tol_outer=1e-8, tol_block=1e-8)
+    dU = torch.empty((ctx.V, 4, 8), dtype=torch.float64, device="cuda")
+    ctx.force(1, seed=5)
+    free = torch.cuda.mem_get_info()[0]
+    ctx.force(1, seed=5, dU=dU)
+    assert free - torch.cuda.mem_get_info()[0] <= 864 * ctx.V + (16 << 20)
+    ctx.close()
