@@ -352,7 +352,8 @@ ddrw_status ddrw_autotune_report(ddrw_ctx *ctx, char *buf, long len);
  * precisions run form 5) or 11 (fully rolled: one body for the eight hops, the direction and
  * the signs chosen at run time; used by the double-single residual stencil, which is limited by
  * instruction fetch, and as form 0 elsewhere); roll 2-4 and 7-11 need nr = 1, roll 5 and 6
- * nr <= 2.  The double-single stencil runs forms 0, 1 and 11, with nr = nw = 1.
+ * nr <= 2.  The double-single stencil runs forms 0, 1 and 11, with nr = nw = 1 (11 with nt = 128 for a
+ * larger nt).
  * A launch whose right-hand sides per mass slot are not a multiple of nr * nw runs with nr = nw = 1.
  * nr = 0 returns to autotuning.  DDRW_EINVAL for values outside these ranges.  A change drops the
  * captured CUDA graphs (they are captured again with the new form on next use). */

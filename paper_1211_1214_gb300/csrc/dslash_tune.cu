@@ -114,7 +114,7 @@ DsConfig tuned_config(ddrw_ctx *ctx, const DslashCall &c, int prec, int bl,
             const int nw = nwl[iw];
             if (prec == 128 && nw != 1) continue;
             if (roll == 8 ? (nt > 128 || nw > rpm) : (c.nrhs / nr) % nw != 0) continue;
-            if (nt * nw > 256) continue;
+            if (nt * nw > 256 || (roll == 11 && nt > 128)) continue;  // (form 11 has CTAs of at most 128 threads)
             DsConfig cfg{nr, nt, nw, roll};
             run(ctx, c, cfg);  // warm
             cudaEventRecord(e0, ctx->stream);

@@ -132,3 +132,20 @@ def test_force_scratch(prec):
     ctx.force(1, seed=5, dU=dU)
     assert free - torch.cuda.mem_get_info()[0] <= 864 * ctx.V + (16 << 20)
     ctx.close()
+
+
+def test_report_names_the_launches_that_ran():
+    """The fully rolled residual stencil (form 11) has CTAs of at most 128 threads, and no larger one is reported."""
+    dims = (8, 8, 8, 8)
+    ctx = context(dims)
+    ctx.set_solver(binding.MIXED_FP32, tol_outer=1e-10, tol_block=1e-12)
+    for _ in range(4):
+        ctx.autotune(True)
+        for nrhs in range(1, 9):
+            b = synth.spinor_field(dims, seed=5, nrhs=nrhs)
+            x = np.zeros_like(b)
+            ctx.solve_block(0, 0.12, b, x, nrhs=nrhs)
+            ctx.solve_D(0.12, b, x, nrhs=nrhs)
+        lines = [line for line in ctx.autotune_report().splitlines() if "roll=11" in line]
+        assert lines and not any("nt=256" in line for line in lines)
+    ctx.close()
