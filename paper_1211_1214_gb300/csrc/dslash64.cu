@@ -13,6 +13,10 @@ namespace {
 // split: 256 updates 43 / 9, 4096 42 / 19, 8192 43 / 31, 16384 46 / 50, 131072 286 / 330.
 constexpr long SPLIT_MOST = 12000;
 
+// the block lengths with launches that small: 8^4 blocks come in launches of at least 16384 updates (a colour and
+// parity of the smallest lattice, 16^4), D on the whole lattice with 6^4 blocks in 20736 (12^4)
+template <bool LEX> constexpr int split_longest() { return LEX ? 4 : 6; }
+
 // ---- one thread per site, boundary layout (in / out: [rhs][lexicographic site][12] complex): FP64 issue
 // bounds the stencil (0.95 of it), so the strided 16-byte accesses of 192-byte spinors cost nothing, and
 // the two layout passes over the fields are gone.
@@ -193,8 +197,8 @@ template <bool LEX> void run_split(ddrw_ctx *ctx, const SplitArgs &a)
     switch (ctx->l) {
     case 2: k_dslash_split<2, LEX><<<grid, 32, 0, ctx->stream>>>(g, a); break;
     case 4: k_dslash_split<4, LEX><<<grid, 32, 0, ctx->stream>>>(g, a); break;
-    case 6: k_dslash_split<6, LEX><<<grid, 32, 0, ctx->stream>>>(g, a); break;
-    default: k_dslash_split<8, LEX><<<grid, 32, 0, ctx->stream>>>(g, a); break;
+    default:
+        if constexpr (!LEX) k_dslash_split<6, LEX><<<grid, 32, 0, ctx->stream>>>(g, a);
     }
 }
 
@@ -234,7 +238,7 @@ void dslash64(ddrw_ctx *ctx, const DslashCall &c)
     const long n = (long)c.npar * c.nblk * ctx->l * ctx->l * ctx->l * ctx->l / 2;
     if (n == 0 || c.nrhs == 0) return;
     // (a pinned launch form, ddrw_stencil_config, selects among the forms of k_dslash)
-    if (n * c.nrhs <= SPLIT_MOST && ctx->pinned_nr == 0) {
+    if (n * c.nrhs <= SPLIT_MOST && ctx->l <= split_longest<false>() && ctx->pinned_nr == 0) {
         ProfScope ps(ctx, PROF_DSLASH64 + (c.hopsel != 0 ? 2 : 0), compulsory_bytes<PrecD>(c, n), (double)n * c.nrhs);
         run_split<false>(ctx, split_args(ctx, c));
         return;
@@ -259,7 +263,7 @@ void apply_D_lex64(ddrw_ctx *ctx, double m, const double2 *in, double2 *out, int
     c.blk0 = 0;
     c.nblk = ctx->nblk;
     ProfScope ps(ctx, PROF_DSLASH64, compulsory_bytes<PrecD>(c, ctx->V), (double)ctx->V * nrhs);
-    if (ctx->V * nrhs <= SPLIT_MOST) {
+    if (ctx->V * nrhs <= SPLIT_MOST && ctx->l <= split_longest<true>()) {
         run_split<true>(ctx, split_args(ctx, c));
         return;
     }
