@@ -149,3 +149,46 @@ def test_force_block_solves_of_every_length(dims, l, n):
         dU.append(u.clone())
     assert rel(dU[0], dU[1]) <= 1e-9
     ctx.close()
+
+
+@pytest.mark.parametrize("antiperiodic", [False, True])
+def test_apply_D_one_thread_per_site_on_2x2x2x2_blocks(antiperiodic):
+    """12288 site updates: beyond the split kernel's range with the smallest blocks."""
+    test_apply_D_layouts_and_block_hops((8, 8, 8, 8), 2, 3, antiperiodic)
+
+
+# half lattices that are multiples of 256 sites: the size rule fuses all of these
+@pytest.mark.parametrize("dims,l,nrhs", [((8, 8, 8, 8), 2, 3), ((24, 12, 12, 12), 6, 5), ((16, 16, 16, 16), 8, 1)])
+def test_fused_inner_products_of_every_block_length(dims, l, nrhs):
+    """The fused stencils ran (the report of tuned shapes lists them), and the solves reach their tolerance as the
+    operator sees it."""
+    ctx = context(dims, l)
+    b = synth.spinor_field(dims, seed=13, nrhs=nrhs)
+    ctx.set_solver(binding.MIXED_FP32, tol_outer=1e-10, tol_block=1e-12)
+    for fuse in (-1, False, True):
+        ctx.autotune(True)
+        ctx.fuse_reductions(fuse)
+        x, y = np.zeros_like(b), np.zeros_like(b)
+        ctx.solve_D(0.12, b, x, nrhs=nrhs)
+        ctx.apply_D(0.12, x, y, nrhs=nrhs)
+        for r in range(nrhs):
+            assert np.linalg.norm(y[r] - b[r]) <= (1e-10 + 1e-14) * np.linalg.norm(b[r])
+        report = ctx.autotune_report()
+        assert ("red=1" in report and "red=2" in report) == (fuse is not False)
+    ctx.close()
+
+
+@pytest.mark.parametrize("l", [2, 4])
+def test_determinants_of_a_nan_link_and_of_singular_blocks(l):
+    """Shared memory (l = 2) and dense (l = 4) determinants answer both with DDRW_ENUMERIC."""
+    dims = (8, 8, 8, 8)
+    U = synth.gauge_field(dims, 0.3, seed=3)
+    U[100, 2, 1, 1] = np.nan
+    for links, csw, m in ((U, 1.4, 0.1), (synth.gauge_field(dims, 0.3, seed=3), 0.0, -4.0)):  # A = 4 + m = 0
+        ctx = binding.Context(dims, (l,) * 4)
+        ctx.load_gauge(links)
+        ctx.set_params(csw, 0.12, 0.07)
+        with pytest.raises(binding.DDRWError) as e:
+            ctx.block_logdet(m)
+        assert e.value.status == 5
+        ctx.close()
