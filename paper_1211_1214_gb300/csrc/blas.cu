@@ -1,10 +1,11 @@
 // blas.cu -- vector kernels and reductions of the Krylov solvers (K7).
 //
 // A vector is a site range [off, off + n) of a field (all planes), for nrhs right-hand sides along
-// gridDim.y.  Reductions: each thread accumulates in the storage precision's arithmetic type,
-// warps and CTAs sum in FP64 (warp shuffles, shared memory), and the last CTA of a right-hand side
-// to finish (atomic ticket after a fence) sums the per-CTA partials in a fixed order, so the
-// result does not depend on scheduling.  The solver scalars stay on the device; the last CTA
+// gridDim.y.  Reductions: products are formed and summed over a storage chunk (at most a site) in the
+// storage precision's arithmetic type; threads, warps, CTAs and the grid sum these in FP64 for FP64
+// fields and in float pairs (RunSum, blas.cuh) for FP32 arithmetic, the last CTA of a right-hand side to
+// finish (atomic ticket after a fence) in a fixed order, so the result does not depend on
+// scheduling.  The solver scalars stay on the device; the last CTA
 // also performs the scalar update of the Krylov recurrence.
 #include <algorithm>
 

@@ -40,7 +40,8 @@ template <class P> struct Blas {
 // (deterministic grid-wide sums shared by the vector kernels of blas.cu and sap.cu)
 
 // A running sum: FP64 for FP64 fields; for FP32 arithmetic an unevaluated pair hi + lo (Knuth's
-// two-sum, about 48 significant bits against the 24 of the terms).  GB300 adds FP64 at 1/64 of its FP32
+// two-sum, about 48 significant bits against the 24 of the terms, in the range of a float: sums of FP32
+// products, whose vectors are scaled to unit right-hand sides).  GB300 adds FP64 at 1/64 of its FP32
 // rate: with FP64 shuffle steps in every warp and FP64 sums over the warps, the reductions took longer
 // than the fields' passes (bicg_omega on 12 x 65536 FP16 sites 43 us, against 14 us for the
 // three passes of bicg_s, which does not reduce).
@@ -227,7 +228,7 @@ template <int K, int NT> __device__ bool grid_sum(double (&v)[K], double *part, 
 }
 
 // alpha (mode 1) or omega (mode 2) of the BiCGStab recurrence from the per-warp partial sums of a
-// fused stencil epilogue (DslashCall::red), nwt partials of RED_PARTS doubles per right-hand side
+// fused stencil epilogue (DslashCall::red), nwt times RED_PARTS 8-byte partial sums per right-hand side
 void bicg_fin(ddrw_ctx *ctx, int mode, int nrhs, const double *part, long nwt, KScal *sc);
 
 // partial-sum and ticket buffers of grid_sum for nrhs right-hand sides (at most 608 CTAs per

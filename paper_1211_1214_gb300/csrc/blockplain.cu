@@ -2,14 +2,15 @@
 //
 // The force of one noise vector is the difference of two nearly equal terms (target masses m1 and m2), which
 // magnifies what the block solves leave behind a hundredfold: at a block tolerance of 1e-11 a force is known to
-// 1e-9, and another order of the sums gives another, equally good one 1.3e-9 away.  Its block solves
-// therefore keep this kernel's order of operations (inner products in FP64 over a fixed number of
-// threads): forces then repeat to 4e-10 with 4^4 blocks and to about 1e-9 with 6^4 and 8^4 ones whatever
-// the outer solver's launch forms.  It costs a tenth of the force (16^4, 4^4 blocks, 4 noise vectors 39.7 ms,
-// with the cluster kernel of blocksolve.cuh 35.9).
+// 1e-9, and another order of the sums gives another, equally good one 1.3e-9 away (either is 1.1e-9 from
+// the exact one).  The FP32 block solves of the force keep this kernel's order of operations, so that its results
+// stay within that distance of those of earlier versions; it makes them no more exact.  FP64 block solves,
+// 16-bit ones (ddrw_set_low_precision) and block method 1 (ddrw_set_block_solver) take the
+// solvers they take elsewhere, whose order follows from the sizes.  It costs a tenth of the force (16^4, 4^4
+// blocks, 4 noise vectors: 39.7 ms, with the cluster kernel of blocksolve.cuh 35.9).
 //
 // One CTA of NT threads owns one (block, right-hand side) pair and runs the whole even-odd BiCGStab with the
-// vectors in global memory; it waits on L2 (27 % of the issue slots for 8^4 blocks).
+// vectors in global memory; it waits on L2.
 #include "blocksolve.cuh"
 
 namespace ddrw {

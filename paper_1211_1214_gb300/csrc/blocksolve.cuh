@@ -734,10 +734,11 @@ __global__ void __launch_bounds__(SplitShape<BL, C>::NT) k_block_split(GeomDev g
 // Measured on FP32 storage, ms per launch of a colour, form 0 / form 1 / the kernel with its vectors in
 // global memory: 24x12^3 in 6^4 blocks, 5 right-hand sides 0.38 / 0.40 / 1.07; 16^4 in 4^4 blocks, 16
 // right-hand sides 0.85 / 1.57 / 1.54; 32x16^3 in 8^4 blocks, 24 right-hand sides 5.5 / 6.2; 48x24^3 in 6^4
-// blocks, 6 right-hand sides 5.8 / 6.3 / 9.1.  What bounds it now is L2: 1.9 MB of links, clover terms
-// and own-site vectors per CTA and iteration (8^4 blocks).  Two or four right-hand sides in
-// a CTA, to share the links through L1, lost (22.8 ms on 64x32^3, 4 right-hand sides, against 15.5): their
-// barriers couple them.
+// blocks, 6 right-hand sides 5.8 / 6.3 / 9.1; 64x32^3 in 8^4 blocks, 4 right-hand sides 14.9 / 25.2 (form 0 / global).
+// What bounds it now is waiting at 16 warps per SM (8^4 blocks, 16 right-hand sides: of 10.4 cycles between
+// a warp's instructions 2.4 at cluster barriers and 2.2 for loads; issue 0.33, L1 0.45, L2 0.24 of their
+// rates).  Two or four right-hand sides in a CTA, to share the links through L1, lost (22.8 ms on
+// 64x32^3, 4 right-hand sides): their barriers couple them.
 template <int BL> struct BlkForms;
 template <> struct BlkForms<2> { static constexpr int C[2] = {1, 1}, N[2] = {32, 32}; };
 template <> struct BlkForms<4> { static constexpr int C[2] = {1, 4}, N[2] = {128, 32}; };

@@ -1,7 +1,7 @@
 // ddprec.cuh -- double-single ("double-float") arithmetic for the defect-correction residuals of
 // the mixed path.
 //
-// GB300 runs FP64 at about 1/58 of its FP32 rate, so the FP64 stencil of the residual
+// GB300 runs FP64 at 1/64 of its FP32 rate, so the FP64 stencil of the residual
 // r = b - D x costs several FP32 stencils.  Here each real number is an unevaluated sum hi + lo of
 // two FP32 numbers (|lo| <= ulp(hi)/2), about 44 significant bits, and the arithmetic uses the
 // error-free transformations of Knuth's two-sum and the FMA-based two-product (Dekker's

@@ -29,7 +29,8 @@
 
 namespace ddrw {
 
-// doubles per warp of a fused stencil epilogue: (t, s), (t, t), (rh, s), (rh, t), or (rh, v) in the first two
+// 8-byte partial sums (float pairs) per warp of a fused stencil epilogue: (t, s), (t, t), (rh, s), (rh, t), or (rh, v)
+// in the first two
 constexpr int RED_PARTS = 7;
 
 constexpr int MAXM = 8;  // mass slots per launch (right-hand sides grouped by mass)

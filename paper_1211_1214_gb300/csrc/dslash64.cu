@@ -18,7 +18,7 @@ constexpr long SPLIT_MOST = 12000;
 template <bool LEX> constexpr int split_longest() { return LEX ? 4 : 6; }
 
 // ---- one thread per site, boundary layout (in / out: [rhs][lexicographic site][12] complex): FP64 issue
-// bounds the stencil (0.95 of it), so the strided 16-byte accesses of 192-byte spinors cost nothing, and
+// bounds the stencil (0.92 of it), so the strided 16-byte accesses of 192-byte spinors cost nothing, and
 // the two layout passes over the fields are gone.
 
 // internal-order neighbour geometry with lexicographic spinor access

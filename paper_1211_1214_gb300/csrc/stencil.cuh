@@ -151,8 +151,7 @@ __device__ __forceinline__ void hop_dir_multi(const GeomDev &g, const Site<BL> &
 // entries of the forward / backward hop (index, block-crossing bit, time-boundary sign bit).  FIRST: the
 // loads of a hop (link and NR spinors, raw) are all issued before any of its arithmetic, which the
 // compiler otherwise starts as soon as the link is there, waiting for memory once per right-hand side.
-// The kernel is bound by that latency at 16 warps per SM (long scoreboard 2.7 of 6.7 cycles per
-// instruction): 64x32^3, 4 right-hand sides, FP16 362 -> 349 us, FP32 457 -> 448 us per launch.
+// The kernel is bound by that latency at 16 warps per SM: 64x32^3, 4 right-hand sides, FP16 362 -> 349 us, FP32 457 -> 448 us per launch.
 // Loading a whole hop ahead, or one spin at a time under fewer registers, gave nothing more.
 template <class P, int HOPSEL, int MU, int NR, bool FIRST = false>
 __device__ __forceinline__ void hop_tab(const GeomDev &g, int nf, int nb, int s, const typename P::SElem *in,
