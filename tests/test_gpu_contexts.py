@@ -149,3 +149,27 @@ def test_report_names_the_launches_that_ran():
         lines = [line for line in ctx.autotune_report().splitlines() if "roll=11" in line]
         assert lines and not any("nt=256" in line for line in lines)
     ctx.close()
+
+
+def test_masses_of_changing_parameters():
+    """Solves after changes of the parameters, before and after loads, with masses that were used, that were only the
+    context's, and 0 (the mass before the parameters): every residual, by the operator."""
+    dims = (8, 8, 8, 8)
+    ctx, b = context(dims), synth.spinor_field(dims, seed=9)
+    ctx.set_solver(binding.MIXED_FP32, tol_outer=1e-11, tol_block=1e-12)
+
+    def check(*masses):
+        for m in masses:
+            x, y = np.zeros_like(b), np.zeros_like(b)
+            ctx.solve_D(m, b, x)
+            ctx.apply_D(m, x, y)
+            assert np.linalg.norm(y - b) <= 1.01e-11 * np.linalg.norm(b), m
+
+    for step, (m1, m2) in enumerate([(0.12, 0.07), (0.2, 0.2), (0.07, 0.3), (0.4, 0.0), (0.2, 0.12)]):
+        ctx.set_params(1.4, m1, m2)
+        if step % 2:
+            ctx.load_gauge(synth.gauge_field(dims, 0.3, seed=20 + step))
+        if step != 1:  # 0.2 is only the context's at first
+            check(m1, m2, 0.25)
+    check(0.0, 0.2, 0.07, 0.3, 0.12, 0.25)
+    ctx.close()
